@@ -124,8 +124,8 @@ clb_status clb_init_fields(clb_handle *h, const double *rho, const double *ux, c
 clb_status clb_init_fields_device(clb_handle *h, const double *rho, const double *ux,
                                   const double *uy, const double *T);
 
-/* Advance n >= 0 time steps (one fused collide-and-stream kernel per step, replayed from a CUDA
- * graph in chunks). Asynchronous. */
+/* Advance n >= 0 time steps (one fused collide-and-stream kernel per step, or per two steps on FP32
+ * lattices too large for the L2 cache, replayed from a CUDA graph in chunks). Asynchronous. */
 clb_status clb_step(clb_handle *h, long n);
 
 /* rho, u (force-corrected, Eq. 13) and T (Eq. 23) at the current time, into host arrays (any may
@@ -197,7 +197,9 @@ clb_status clb_load(clb_handle *h, const void *buf, size_t bytes);
  * clb_autotune times candidate shapes on the live lattice (the populations are restored
  * afterwards; it allocates one buffer-sized scratch with cudaMallocAsync) and keeps the fastest;
  * results are cached per (storage, nx, ny) for later clb_create calls. The shape never changes
- * the results (the per-node arithmetic does not depend on it). */
+ * the results (the per-node arithmetic does not depend on it). Lattices whose default takes two
+ * steps per launch step one at a time, with the given shape, after clb_set_launch or
+ * clb_set_pipeline; clb_autotune weighs both. */
 clb_status clb_set_launch(clb_handle *h, int block_x, int block_y, int nodes_per_thread);
 clb_status clb_get_launch(clb_handle *h, int *block_x, int *block_y, int *nodes_per_thread);
 clb_status clb_autotune(clb_handle *h, int *block_x, int *block_y, int *nodes_per_thread);

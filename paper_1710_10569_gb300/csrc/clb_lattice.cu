@@ -1,5 +1,5 @@
 // clb_lattice.cu -- C ABI of one lattice (include/clb.h): creation, initialisation, the stepping
-// loop (CUDA-graph chunks of the fused step kernel), field extraction, FP64 diagnostics,
+// loop (CUDA-graph chunks of the fused step kernel, or of the kernel that takes two steps), field extraction, FP64 diagnostics,
 // checkpoints and the launch-shape autotuner.
 #include <cuda_runtime.h>
 
@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "clb_diag.cuh"
+#include "clb_march.cuh"
 
 using namespace clb;
 
@@ -158,6 +159,7 @@ struct clb_handle {
     long steps = 0;
     int bx = 128, by = 1, npt = 1;
     int pipe_stages = 0, pipe_rows = 8;  // 0 stages: direct kernel
+    int march = 0;  // > 0: pairs of steps run in k_step_two, in segments of this many rows
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     LatParams<double> Pd{};
     LatParams<float> Pf{};
@@ -277,9 +279,66 @@ cudaError_t enqueue_step_npt(const clb_handle* h, const void* a, void* b, cudaSt
 
 struct Launch {
     int bx, by, npt, stages, rows;
+    int march;  // rows per segment of the two-step kernel, 0: one step per launch
 };
 
-Launch current_launch(const clb_handle* h) { return {h->bx, h->by, h->npt, h->pipe_stages, h->pipe_rows}; }
+Launch current_launch(const clb_handle* h)
+{
+    return {h->bx, h->by, h->npt, h->pipe_stages, h->pipe_rows, h->march};
+}
+
+// Strips and segments of the two-step kernel with segments of `rows` rows.
+MarchGeom march_geom(int nx, int ny, int rows)
+{
+    MarchGeom G;
+    G.strips = (nx + kMarchOut - 1) / kMarchOut;
+    G.width = ((nx + G.strips - 1) / G.strips + 1) & ~1;
+    G.strips = (nx + G.width - 1) / G.width;
+    G.rows = rows;
+    G.segs = (ny + rows - 1) / rows;
+    return G;
+}
+
+// Rows per segment of the two-step kernel, 0 where one step per launch is the faster form.
+// Longer segments repeat fewer rows of the first step, shorter ones fill the last round of resident
+// warps. With w warps per SM a warp takes 0.5 + 0.068 w us per row (fitted to 1 to 20 warps per SM),
+// and a segment of R rows costs it R + 1 of these per step; the R of the least time over the rounds
+// of resident warps is taken (2048 x 1024: 12, one round of 3,010 warps, 24.2 us per step against
+// 26.1 at 6 and 27.6 at 20). One step per launch is kept where its own time, the bytes at the copy
+// bandwidth, is less (few rows, or rows that fill their windows badly), and below kMarchNodes: the two
+// buffers of such lattices sit in the 129 MB L2, from where one step per launch runs without the
+// repeated columns and rows (1024 x 512: 6.9 us against 7.9).
+constexpr long long kMarchNodes = 1000000;
+int march_rows_rule(int nx, int ny, const clb_params& p, int sms)
+{
+    const bool wet = p.wall[0] == CLB_WALL_WET || p.wall[2] == CLB_WALL_WET;
+    if (p.storage != CLB_F32 || wet || (long long)nx * ny < kMarchNodes) return 0;
+    const int resident = sms * kMarchResident;
+    int best = 0;
+    double least = 1.0 + 112.0 * nx * ny / 6.7e6;
+    for (int rows = 4; rows <= 64; ++rows) {
+        const int warps = march_geom(nx, ny, rows).warps(), rest = warps % resident;
+        const double t = (rows + 1) * ((warps / resident) * (0.5 + 0.068 * kMarchResident) +
+                                       (rest ? 0.5 + 0.068 * rest / sms : 0.0));
+        if (t < least) {
+            least = t;
+            best = rows;
+        }
+    }
+    return best;
+}
+
+// Enqueue two steps from buffer `from` into the other buffer on stream s.
+clb_status launch_two(const clb_handle* h, int from, cudaStream_t s, const Launch& L)
+{
+    const MarchGeom G = march_geom(h->nx, h->ny, L.march);
+    const float* a = (const float*)h->buf[from];
+    float* b = (float*)h->buf[from ^ 1];
+    if (h->p.s_3 == 1.0 && h->p.s_4 == 1.0 && h->p.lambda2 == 1.0) k_step_two<true><<<G.warps(), 32, 0, s>>>(a, b, h->Pf, G);
+    else k_step_two<false><<<G.warps(), 32, 0, s>>>(a, b, h->Pf, G);
+    CLB_CUDA(cudaGetLastError());
+    return CLB_OK;
+}
 
 // Enqueue one step from buffer `from` into the other buffer on stream s.
 clb_status launch_step(clb_handle* h, int from, cudaStream_t s, const Launch& L)
@@ -307,7 +366,10 @@ clb_status build_graph(clb_handle* h, int start)
 {
     CLB_CUDA(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
     clb_status st = CLB_OK;
-    for (int k = 0; k < kGraphChunk && st == CLB_OK; ++k) st = launch_step(h, start ^ (k & 1), h->cap, current_launch(h));
+    const Launch L = current_launch(h);
+    const int per = L.march > 0 ? 2 : 1;  // steps per launch; kGraphChunk / per launches are an even number
+    for (int k = 0; k < kGraphChunk / per && st == CLB_OK; ++k)
+        st = per == 2 ? launch_two(h, start ^ (k & 1), h->cap, L) : launch_step(h, start ^ (k & 1), h->cap, L);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(h->cap, &g);
     if (st != CLB_OK) {
@@ -387,7 +449,7 @@ clb_status take_snapshot(clb_handle* h)
 }
 
 std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int>, std::array<int, 5>> g_tune_cache;
+std::map<std::tuple<int, int, int>, std::array<int, 6>> g_tune_cache;
 
 }  // namespace
 
@@ -450,6 +512,7 @@ extern "C" clb_status clb_create(int nx, int ny, const clb_params* p, void* stre
         h->Pd = make_lat_params<double>(nx, ny, *p);
         h->Pf = make_lat_params<float>(nx, ny, *p);
         h->npt = p->storage == CLB_F32 ? 2 : 4;
+        bool tuned = false;
         {
             std::lock_guard<std::mutex> lk(g_tune_mu);
             auto it = g_tune_cache.find(std::make_tuple(p->storage, nx, ny));
@@ -459,7 +522,14 @@ extern "C" clb_status clb_create(int nx, int ny, const clb_params* p, void* stre
                 h->npt = it->second[2];
                 h->pipe_stages = it->second[3];
                 h->pipe_rows = it->second[4];
+                h->march = it->second[5];
+                tuned = true;
             }
+        }
+        if (!tuned) {
+            int sms = 0;
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+            h->march = march_rows_rule(nx, ny, *p, std::max(1, sms));
         }
         // the padding of each row's last chunk is never read, but keep it defined
         e = cudaMemsetAsync(h->mem, 0, L.snap, h->stream);
@@ -558,8 +628,14 @@ extern "C" clb_status clb_step(clb_handle* h, long n)
         n -= kGraphChunk;
         h->steps += kGraphChunk;
     }
+    const Launch L = current_launch(h);
+    for (; L.march > 0 && n >= 2; n -= 2) {
+        CLB_TRY(launch_two(h, h->cur, h->stream, L));
+        h->cur ^= 1;
+        h->steps += 2;
+    }
     for (; n > 0; --n) {
-        CLB_TRY(launch_step(h, h->cur, h->stream, current_launch(h)));
+        CLB_TRY(launch_step(h, h->cur, h->stream, L));
         h->cur ^= 1;
         h->steps++;
     }
@@ -771,7 +847,8 @@ clb_status apply_launch(clb_handle* h, const Launch& L)
 {
     CLB_TRY(check_launch(h, L));
     const Launch c = current_launch(h);
-    if (c.bx != L.bx || c.by != L.by || c.npt != L.npt || c.stages != L.stages || c.rows != L.rows) {
+    if (c.bx != L.bx || c.by != L.by || c.npt != L.npt || c.stages != L.stages || c.rows != L.rows ||
+        c.march != L.march) {
         DeviceGuard dg(h->device);
         cudaStreamSynchronize(h->stream);
         drop_graphs(h);
@@ -780,6 +857,7 @@ clb_status apply_launch(clb_handle* h, const Launch& L)
         h->npt = L.npt;
         h->pipe_stages = L.stages;
         h->pipe_rows = L.rows;
+        h->march = L.march;
     }
     return CLB_OK;
 }
@@ -793,6 +871,7 @@ extern "C" clb_status clb_set_launch(clb_handle* h, int block_x, int block_y, in
     if (block_y) L.by = block_y;
     if (nodes_per_thread) L.npt = nodes_per_thread;
     if (L.npt == 1) L.stages = 0;
+    L.march = 0;
     return apply_launch(h, L);
 }
 
@@ -802,6 +881,7 @@ extern "C" clb_status clb_set_pipeline(clb_handle* h, int stages, int rows)
     Launch L = current_launch(h);
     L.stages = stages;
     if (rows) L.rows = rows;
+    L.march = 0;
     return apply_launch(h, L);
 }
 
@@ -835,10 +915,14 @@ extern "C" clb_status clb_autotune(clb_handle* h, int* block_x, int* block_y, in
         std::vector<Launch> cands;
         const int shapes[][2] = {{64, 1}, {128, 1}, {256, 1}, {32, 4}, {64, 2}, {128, 2}};
         for (int npt : {1, 2, 4})
-            for (auto& sh : shapes) cands.push_back({sh[0], sh[1], npt, 0, 8});
+            for (auto& sh : shapes) cands.push_back({sh[0], sh[1], npt, 0, 8, 0});
         for (int npt : {2, 4})
             for (int st : {2, 3, 4})
-                for (int rows : {4, 8, 16}) cands.push_back({128, 1, npt, st, rows});
+                for (int rows : {4, 8, 16}) cands.push_back({128, 1, npt, st, rows, 0});
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+        if (const int rows = march_rows_rule(h->nx, h->ny, h->p, std::max(1, sms)))
+            cands.push_back({128, 1, 2, 0, 8, rows});  // two steps per launch
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
@@ -849,9 +933,11 @@ extern "C" clb_status clb_autotune(clb_handle* h, int* block_x, int* block_y, in
         for (const Launch& c : cands) {
             if (c.bx * c.npt > 2 * h->nx + 64 && c.bx * c.npt > 64) continue;  // far wider than the lattice
             if (c.stages > 0 && check_launch(h, c) != CLB_OK) continue;
-            for (int k = 0; k < 4 && st == CLB_OK; ++k) st = launch_step(h, (h->cur + k) & 1, h->stream, c);
+            const int per = c.march > 0 ? 2 : 1;  // steps per launch
+            const auto launch = [&](int from) { return per == 2 ? launch_two(h, from, h->stream, c) : launch_step(h, from, h->stream, c); };
+            for (int k = 0; k < 4 && st == CLB_OK; ++k) st = launch((h->cur + k) & 1);
             cudaEventRecord(e0, h->stream);
-            for (int k = 0; k < reps && st == CLB_OK; ++k) st = launch_step(h, (h->cur + k) & 1, h->stream, c);
+            for (int k = 0; k < reps / per && st == CLB_OK; ++k) st = launch((h->cur + k) & 1);
             cudaEventRecord(e1, h->stream);
             if (st != CLB_OK) break;
             cudaEventSynchronize(e1);
@@ -872,7 +958,7 @@ extern "C" clb_status clb_autotune(clb_handle* h, int* block_x, int* block_y, in
         CLB_TRY(apply_launch(h, bl));
         {
             std::lock_guard<std::mutex> lk(g_tune_mu);
-            g_tune_cache[std::make_tuple(h->p.storage, h->nx, h->ny)] = {bl.bx, bl.by, bl.npt, bl.stages, bl.rows};
+            g_tune_cache[std::make_tuple(h->p.storage, h->nx, h->ny)] = {bl.bx, bl.by, bl.npt, bl.stages, bl.rows, bl.march};
         }
         if (block_x) *block_x = bl.bx;
         if (block_y) *block_y = bl.by;

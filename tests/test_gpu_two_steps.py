@@ -1,0 +1,45 @@
+"""The FP32 kernel that takes two steps per launch (large lattices) against the one-step kernel, which
+an explicit launch shape selects: every population bitwise, over windows and rows of every kind (one
+and several windows per row, odd rows, a last window of one column, rows that end in mid-window,
+segments of every remainder), every wall layout, fixed and moving, both collision forms, and even
+and odd numbers of steps."""
+import numpy as np
+import pytest
+
+from paper_1710_10569_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+P, D, A = W.WALL_PERIODIC, W.WALL_DIRICHLET, W.WALL_ADIABATIC
+LAYOUTS = {"periodic": (P, P, P, P), "layer": (P, P, D, D), "box": (D, A, A, D), "cavity": (D, D, A, A), "sides": (A, D, P, P)}
+
+
+@pytest.fixture(scope="module")
+def clb():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_1710_10569_gb300 import clb as c
+    return c
+
+
+@pytest.mark.parametrize("shape,steps", [((53, 19001), 2), ((60, 17003), 7), ((59, 17200), 4), ((118, 8701), 3), ((121, 9002), 5),
+                                         ((1001, 1003), 7), ((2048, 517), 34), ((30011, 41), 6)],
+                         ids=lambda v: f"{v[0]}x{v[1]}" if isinstance(v, tuple) else f"{v}")
+@pytest.mark.parametrize("layout", sorted(LAYOUTS))
+def test_two_steps_per_launch_equal_one(clb, layout, shape, steps):
+    one = (shape[0] + steps) % 2 == 0
+    prob = W.random_problem(*shape, seed=shape[0] + steps, storage=W.STORAGE_F32, walls=LAYOUTS[layout], moving=not one)
+    if one:
+        prob.params.update(s_3=1.0, s_4=1.0, lambda2=1.0)
+    got = []
+    for shape_set in (False, True):
+        lat = clb.Lattice.from_problem(prob)
+        if shape_set:
+            lat.set_launch(128, 1, 2)
+        lat.step(steps)
+        got.append(lat.populations())
+        assert lat.steps == steps
+        lat.close()
+    for a, b in zip(*got):
+        assert np.isfinite(a).all() and np.array_equal(a, b)
