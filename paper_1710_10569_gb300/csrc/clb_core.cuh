@@ -68,6 +68,28 @@ __device__ __forceinline__ double fma_(double a, double b, double c) { return __
 __device__ __forceinline__ float rcp_(float a) { return __frcp_rn(a); }
 __device__ __forceinline__ double rcp_(double a) { return __drcp_rn(a); }
 
+// x / 2^N for a double by its exponent: integer instructions in place of a multiplication, which on
+// GB300 costs as much as any other FP64 instruction (64 clocks of an SM quarter's pipe per warp). Exact
+// where the result is a normal number; smaller ones give a signed zero, infinities and NaN stay.
+template <int N>
+__device__ __forceinline__ double scale_down(double x)
+{
+    const int hi = __double2hiint(x);
+    const unsigned e = (unsigned)hi >> 20 & 0x7ff;
+    const bool keep = e == 0x7ff, tiny = e <= N;
+    return __hiloint2double(keep ? hi : tiny ? hi & (int)0x80000000 : hi - (N << 20), !keep && tiny ? 0 : __double2loint(x));
+}
+// 1 / x from the hardware's approximation r (relative error e below 2^-19) by one step of Halley's
+// third-order iteration, r + r (e + e^2) with e = 1 - x r: three FMAs in place of the six of the
+// correctly rounded reciprocal, and within one unit of the last place of it.
+__device__ __forceinline__ double rcp_halley(double x)
+{
+    double r;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(r) : "d"(x));
+    const double e = __fma_rn(-x, r, 1.0);
+    return __fma_rn(r, __fma_rn(e, e, e), r);
+}
+
 // Two FP32 lanes (two lattice nodes) in one 64-bit register pair, operated on by the packed
 // FP32 instructions of sm_100-class GPUs (add/sub/mul/fma .rn.f32x2). Each lane is rounded exactly
 // as the scalar instruction would round it, so a node computed in a pair carries the same bits as
@@ -138,9 +160,20 @@ __device__ __forceinline__ F2 rcp_(F2 a)
     return F2(__frcp_rn(lo), __frcp_rn(hi));
 }
 
+// Constants of the FP64 collision (collide), formed once on the host: an FP64 instruction on uniform
+// values costs a warp as much as one on its nodes.
+template <typename A> struct CollideConsts {};
+template <> struct CollideConsts<double> {
+    double hFx, hFvy, hgb, qFx, eFx;  // Fv_x / 2, Fv_y / 2, gb / 2, Fv_x / 4, Fv_x / 8
+    double c3, hFc3;                  // (2 - s_3) / 3, and Fv_x / 2 times it (third-order forcing)
+    double hsp, hsm, om11;            // sp / 2, sm / 2, 1 - s_nu
+    double om3, qom3, s36, qom4;      // 1 - s_3 and its quarter, s_4 / 36, (1 - s_4) / 4
+    double hom1, hom2, heq;           // (1 - lambda1) / 2, (1 - lambda2) / 2, lambda2 cs2_T / 2
+};
+
 // Per-lattice constants in the arithmetic precision A.
 template <typename A>
-struct LatParams {
+struct LatParams : CollideConsts<A> {
     int nx, ny;
     long long crow;           // elements per chunked row (coupled lattice: see chunk_off)
     int pitch;                // thermal-only mode (plane-major): elements per row, 128-byte aligned
@@ -403,61 +436,108 @@ __device__ __forceinline__ void central_d2q9(const A f[9], A ux, A uy, A k[3][3]
     for (int a = 0; a < 3; ++a) central3(r0[a], rp[a], rm[a], uy, k[a][0], k[a][1], k[a][2]);
 }
 
-// D2Q5 collision in populations form (Eqs. 16-21) for temperature T and velocity u. HI1: lambda2 = 1,
-// so the second-order central moments relax to equilibrium whatever their value (not formed).
-template <bool HI1 = false, typename A>
-__device__ __forceinline__ void collide_d2q5(const LatParams<A>& P, A T, A ux, A uy, A g[5])
+// D2Q5 collision in populations form (Eqs. 16-21) for temperature T and velocity u, given the axis
+// sums s and differences d of g. The back transform takes the halves of the raw moments,
+// r1/2 = k1/2 + (u/2) T and r2/2 = k2/2 + u (k1/2 + r1/2). HI1: lambda2 = 1, so the second-order
+// central moments relax to equilibrium whatever their value (not formed).
+template <bool HI1 = false>
+__device__ __forceinline__ void collide_d2q5(const LatParams<double>& P, double T, double ux, double uy, double hux,
+                                             double huy, double s1, double d1, double s2, double d2, double g[5])
 {
-    const A d1 = g[1] - g[3], s1 = g[1] + g[3];
-    const A d2 = g[2] - g[4], s2 = g[2] + g[4];
-    const A t10 = fma_(-ux, T, d1);
-    const A t01 = fma_(-uy, T, d2);
-    const A t20 = fma_(ux * ux, T, fma_(A(-2) * ux, d1, s1));
-    const A t02 = fma_(uy * uy, T, fma_(A(-2) * uy, d2, s2));
-    const A om1 = A(1) - P.lambda1;
-    const A om2 = A(1) - P.lambda2;
-    const A eqT = P.lambda2 * T * P.cs2T;
-    if constexpr (HI1) back_d2q5(T, om1 * t10, om1 * t01, eqT, eqT, ux, uy, g);
-    else back_d2q5(T, om1 * t10, om1 * t01, fma_(om2, t20, eqT), fma_(om2, t02, eqT), ux, uy, g);
+    const double uT = hux * T, vT = huy * T;
+    const double k1 = P.hom1 * fma_(-ux, T, d1), k2 = P.hom1 * fma_(-uy, T, d2);
+    const double r1 = k1 + uT, r2 = k2 + vT;
+    const double eq = P.heq * T;
+    double h1 = fma_(ux, k1 + r1, eq), h2 = fma_(uy, k2 + r2, eq);
+    if constexpr (!HI1) {
+        h1 = fma_(P.hom2, fma_(ux * ux, T, fma_(-2.0 * ux, d1, s1)), h1);
+        h2 = fma_(P.hom2, fma_(uy * uy, T, fma_(-2.0 * uy, d2, s2)), h2);
+    }
+    g[0] = fma_(-2.0, h2, fma_(-2.0, h1, T));
+    g[1] = h1 + r1;
+    g[3] = h1 - r1;
+    g[2] = h2 + r2;
+    g[4] = h2 - r2;
 }
 
-// Collision of one node in place, populations form: Eqs. (6)-(11) for f, Eqs. (16)-(21) for g.
+// Collision of one node in place, populations form (FP64 storage): Eqs. (6)-(11) for f, Eqs. (16)-(21)
+// for g. FP64 instructions bound it (GB300 issues two per clock and SM), so it is written for the
+// fewest of them: 104 with HI1, 421 us per step on 2048 x 1024 (the transforms pass by pass took
+// 139.8, 544 us). The relaxed central moments go straight to raw moments about 0, in the halves (second
+// order, and the momentum) and quarters (order 3 and 4, and xy) that the back transform takes;
+// rho u = j + F/2 makes the first-order central moments -F/2, so they are not formed:
+//   k20 = m20 - u (j - F/2), r20 = m20 + 2 u F - (relaxation), k11 = m11 - u_x j_y + u_y F_x / 2,
+//   r21 = R21 + u_y r20 with R21 = k21* + 2 u_x k11* + u_x^2 k01*, and r12 alike with the axes swapped,
+//   r22 = R22 + u_y (2 R21 + u_y r20) with R22 = k22* + 2 u_x k12* + u_x^2 k02*.
 // HI1: the high-order rates are 1 (s_3 = s_4 = lambda2 = 1, the paper's setting, Sec. 3), so k~21,
 // k~12, k~22 and the second-order D2Q5 moments relax to their equilibrium and forcing terms
-// whatever their value; they are then not formed (the compiler drops that part of the forward
-// transforms). The results are the same as with HI1 = false: (1 - s) k is an exact zero for s = 1.
-template <bool HI1 = false, typename A>
-__device__ __forceinline__ void collide(const LatParams<A>& P, A f[9], A g[5], A Tb)
+// whatever their value; they are then not formed. The results are the same as with HI1 = false:
+// (1 - s) k is an exact zero for s = 1.
+template <bool HI1 = false>
+__device__ __forceinline__ void collide(const LatParams<double>& P, double f[9], double g[5])
 {
-    const Macro<A> m = macroscopic(P, f, g, Tb);
-    const A ux = m.ux, uy = m.uy, rho = m.rho, T = m.T;
-    const A cs2 = A(1) / A(3);
-    A k[3][3];
-    central_d2q9(f, ux, uy, k);
+    const double s0 = f[1] + f[3], d0 = f[1] - f[3];
+    const double sp = f[5] + f[6], dp = f[5] - f[6];
+    const double sm = f[8] + f[7], dm = f[8] - f[7];
+    const double rp = f[2] + sp, rm = f[4] + sm;
+    const double m02 = rp + rm, m20 = s0 + (sp + sm), m11 = dp - dm;
+    const double rho = (f[0] + s0) + m02;
+    // the momentum from differences of opposite populations: rp - rm, two additions fewer, rounds at the
+    // size of rp, and loses the slow growth of a roll near onset (Ra = 2500 between wet walls)
+    const double jx = (d0 + dp) + dm, jy = ((f[2] - f[4]) + sp) - sm;
+    const double s1 = g[1] + g[3], d1 = g[1] - g[3], s2 = g[2] + g[4], d2 = g[2] - g[4];
+    const double T = g[0] + (s1 + s2);
+    const double hFx = P.hFx, hFy = fma_(P.hgb, T - P.T0, P.hFvy);
+    const double inv = rcp_halley(rho);
+    const double qx = jx + hFx, qy = jy + hFy;  // rho u (Eq. 13)
+    const double ux = qx * inv, uy = qy * inv;
+    const double hux = scale_down<1>(ux), huy = scale_down<1>(uy);
+    double k21 = 0.0, k12 = 0.0, k22 = 0.0;
+    if constexpr (!HI1) {
+        double k[3][3];
+        central_d2q9(f, ux, uy, k);
+        k21 = k[2][1];
+        k12 = k[1][2];
+        k22 = k[2][2];
+    }
 
     // relaxation, Eq. (8), equilibrium Eq. (9), forcing Eq. (11)
-    const A a20 = fma_(-rho, cs2, k[2][0]);
-    const A a02 = fma_(-rho, cs2, k[0][2]);
-    A q[3][3];
-    q[0][0] = rho;
-    q[1][0] = k[1][0] + m.Fx;
-    q[0][1] = k[0][1] + m.Fy;
-    q[2][0] = fma_(-P.sm, a02, fma_(-P.sp, a20, k[2][0]));
-    q[0][2] = fma_(-P.sp, a02, fma_(-P.sm, a20, k[0][2]));
-    q[1][1] = (A(1) - P.s_nu) * k[1][1];
-    const A half3 = (A(1) - A(0.5) * P.s_3) * cs2;
-    if constexpr (HI1) {
-        q[2][1] = half3 * m.Fy;
-        q[1][2] = half3 * m.Fx;
-        q[2][2] = P.s_4 * rho * (cs2 * cs2);
-    } else {
-        q[2][1] = fma_(A(1) - P.s_3, k[2][1], half3 * m.Fy);
-        q[1][2] = fma_(A(1) - P.s_3, k[1][2], half3 * m.Fx);
-        q[2][2] = fma_(A(1) - P.s_4, k[2][2], P.s_4 * rho * (cs2 * cs2));
+    const double k20 = fma_(-ux, jx - hFx, m20), k02 = fma_(-uy, jy - hFy, m02);
+    const double a20 = fma_(-1.0 / 3.0, rho, k20), a02 = fma_(-1.0 / 3.0, rho, k02);
+    const double h20 = fma_(-P.hsm, a02, fma_(-P.hsp, a20, fma_(ux, P.Fvx, scale_down<1>(m20))));
+    const double q02 = fma_(-P.sm, a20, fma_(-P.sp, a02, k02));
+    const double h02 = fma_(huy, fma_(2.0, hFy, qy), scale_down<1>(q02));
+    const double h10 = fma_(0.5, jx, hFx), h01 = fma_(0.5, jy, hFy);
+    const double q11 = P.om11 * fma_(-ux, jy, fma_(uy, hFx, m11));
+    const double M11 = fma_(hux, h01, fma_(huy, P.qFx, scale_down<2>(q11)));
+    double R21 = fma_(hux, q11, scale_down<2>(hFy) * fma_(ux, ux, P.c3));
+    double R12 = fma_(huy, q11, P.eFx * fma_(uy, uy, P.c3));
+    double in = fma_(hux, q02, P.hFc3);
+    double e22 = P.s36 * rho;
+    if constexpr (!HI1) {
+        R21 = fma_(P.qom3, k21, R21);
+        R12 = fma_(P.qom3, k12, R12);
+        in = fma_(P.om3, k12, in);
+        e22 = fma_(P.qom4, k22, e22);
     }
-    back_d2q9(q, ux, uy, f);
+    const double M21 = fma_(huy, h20, R21), M12 = fma_(hux, h02, R12);
+    const double M22 = fma_(uy, R21 + M21, fma_(hux, in, e22));
 
-    collide_d2q5<HI1>(P, T, ux, uy, g);
+    // back transform from the scaled raw moments
+    const double p = M22 + M21, q = M22 - M21, r = M12 + M11, t = M12 - M11;
+    const double ex = fma_(-2.0, M22, h20), cx = fma_(-2.0, M12, h10);
+    const double ey = fma_(-2.0, M22, h02), cy = fma_(-2.0, M21, h01);
+    f[0] = fma_(4.0, M22, fma_(-2.0, h02, fma_(-2.0, h20, rho)));
+    f[1] = ex + cx;
+    f[3] = ex - cx;
+    f[2] = ey + cy;
+    f[4] = ey - cy;
+    f[5] = p + r;
+    f[6] = p - r;
+    f[7] = q - t;
+    f[8] = q + t;
+
+    collide_d2q5<HI1>(P, T, ux, uy, hux, huy, s1, d1, s2, d2, g);
 }
 
 // Deviation of the D2Q9 equilibrium from the rest state, f^eq_i(rho, u) - w_i rho_b, written as
@@ -604,7 +684,7 @@ template <bool DEV, bool HI1 = false, typename A>
 __device__ __forceinline__ void collide_any(const LatParams<A>& P, A f[9], A g[5], A Tb)
 {
     if constexpr (DEV) collide_dev<HI1>(P, f, g, Tb);
-    else collide<HI1>(P, f, g, Tb);
+    else collide<HI1>(P, f, g);  // FP64 populations: no base
 }
 
 // Equilibria in stored form, minus the rest state for deviation storage: f^eq(rho, u) (Eq. 9

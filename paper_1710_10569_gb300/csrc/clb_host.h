@@ -181,6 +181,25 @@ LatParams<A> make_lat_params(int nx, int ny, const clb_params& p)
     P.Fvy = A(p.Fv[1]);
     P.gb = A(p.rho0 * p.g_beta);
     P.T0 = A(p.T0);
+    if constexpr (sizeof(A) == sizeof(double)) {
+        P.hFx = 0.5 * p.Fv[0];
+        P.hFvy = 0.5 * p.Fv[1];
+        P.hgb = 0.5 * P.gb;
+        P.qFx = 0.25 * p.Fv[0];
+        P.eFx = 0.125 * p.Fv[0];
+        P.c3 = (2.0 - p.s_3) * (1.0 / 3.0);
+        P.hFc3 = P.hFx * P.c3;
+        P.hsp = 0.5 * P.sp;
+        P.hsm = 0.5 * P.sm;
+        P.om11 = 1.0 - s_nu;
+        P.om3 = 1.0 - p.s_3;
+        P.qom3 = 0.25 * P.om3;
+        P.s36 = p.s_4 * (1.0 / 36.0);
+        P.qom4 = 0.25 * (1.0 - p.s_4);
+        P.hom1 = 0.5 * (1.0 - P.lambda1);
+        P.hom2 = 0.5 * (1.0 - p.lambda2);
+        P.heq = 0.5 * p.lambda2 * p.cs2_T;
+    }
     return P;
 }
 

@@ -112,9 +112,13 @@ __device__ __forceinline__ void thermal_collide(const LatParams<typename Storage
                                                 typename Storage<ST>::A g[NT], typename Storage<ST>::A Tb)
 {
     using A = typename Storage<ST>::A;
-    const A dT = (g[0] + g[1]) + (g[2] + g[3]) + g[4];
-    if constexpr (Storage<ST>::DEV) collide_d2q5_dev(P, Tb + dT, dT, u, v, g);
-    else collide_d2q5(P, Tb + dT, u, v, g);
+    if constexpr (Storage<ST>::DEV) {
+        const A dT = (g[0] + g[1]) + (g[2] + g[3]) + g[4];
+        collide_d2q5_dev(P, Tb + dT, dT, u, v, g);
+    } else {
+        const double s1 = g[1] + g[3], d1 = g[1] - g[3], s2 = g[2] + g[4], d2 = g[2] - g[4];
+        collide_d2q5(P, g[0] + (s1 + s2), u, v, scale_down<1>(u), scale_down<1>(v), s1, d1, s2, d2, g);
+    }
 }
 
 // One time step, two neighbouring nodes x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x) and x0 + 1
