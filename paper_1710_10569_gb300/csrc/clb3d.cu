@@ -431,6 +431,7 @@ __global__ void __launch_bounds__(256) k_step3(const typename Storage<ST>::T* __
                                                typename Storage<ST>::T* __restrict__ dst,
                                                const Lat3<typename Storage<ST>::A> P, int xblocks)
 {
+    step_prologue();
     const int xb = blockIdx.x % xblocks, rb = blockIdx.x / xblocks;
     const int x = xb * blockDim.x + threadIdx.x;
     const int r = rb * blockDim.y + threadIdx.y;
@@ -777,6 +778,7 @@ __global__ void __launch_bounds__(256) k_thermal3_step(const typename Storage<ST
 {
     using A = typename Storage<ST>::A;
     using T = typename Storage<ST>::T;
+    step_prologue();
     const int xb = blockIdx.x % xblocks, rb = blockIdx.x / xblocks;
     const int x = xb * blockDim.x + threadIdx.x;
     const int r = rb * blockDim.y + threadIdx.y;
@@ -1004,22 +1006,21 @@ Lat3<A> make_lat3(int nx, int ny, int nz, const clb3d_params& p)
 int xblocks_of(const clb3d_lattice* h) { return (h->nx + h->bx - 1) / h->bx; }
 
 template <int ST, bool HIGH1>
-void launch3(const clb3d_lattice* h, int from, cudaStream_t s, unsigned grid, dim3 block, int xb)
+cudaError_t launch3(const clb3d_lattice* h, int from, cudaStream_t s, unsigned grid, dim3 block, int xb)
 {
     using T = typename Storage<ST>::T;
     if constexpr (ST == ST_F64)
-        k_step3<ST, HIGH1><<<grid, block, 0, s>>>((const T*)h->buf[from], (T*)h->buf[from ^ 1], h->Pd, xb);
+        return launch_chained(k_step3<ST, HIGH1>, grid, block, 0, s, (const T*)h->buf[from], (T*)h->buf[from ^ 1], h->Pd, xb);
     else
-        k_step3<ST, HIGH1><<<grid, block, 0, s>>>((const T*)h->buf[from], (T*)h->buf[from ^ 1], h->Pf, xb);
+        return launch_chained(k_step3<ST, HIGH1>, grid, block, 0, s, (const T*)h->buf[from], (T*)h->buf[from ^ 1], h->Pf, xb);
 }
 
 template <int ST>
-void launch3_rates(const clb3d_lattice* h, int from, cudaStream_t s, unsigned grid, dim3 block, int xb)
+cudaError_t launch3_rates(const clb3d_lattice* h, int from, cudaStream_t s, unsigned grid, dim3 block, int xb)
 {
     // the high-order rates all 1 (the paper's setting): the form that skips those moments
     const bool high1 = h->p.s_3 == 1.0 && h->p.s_4 == 1.0 && h->p.s_5 == 1.0 && h->p.s_6 == 1.0;
-    if (high1) launch3<ST, true>(h, from, s, grid, block, xb);
-    else launch3<ST, false>(h, from, s, grid, block, xb);
+    return high1 ? launch3<ST, true>(h, from, s, grid, block, xb) : launch3<ST, false>(h, from, s, grid, block, xb);
 }
 
 clb_status launch_step3(clb3d_lattice* h, int from, cudaStream_t s)
@@ -1028,10 +1029,9 @@ clb_status launch_step3(clb3d_lattice* h, int from, cudaStream_t s)
     const long long rb = ((long long)h->ny * h->nz + h->by - 1) / h->by;
     const dim3 block(h->bx, h->by);
     const unsigned grid = unsigned((long long)xb * rb);
-    if (h->p.storage == CLB_F64) launch3_rates<ST_F64>(h, from, s, grid, block, xb);
-    else if (h->p.storage == CLB_F32) launch3_rates<ST_F32>(h, from, s, grid, block, xb);
-    else launch3_rates<ST_F16DEV>(h, from, s, grid, block, xb);
-    CLB_CUDA(cudaGetLastError());
+    CLB_CUDA(h->p.storage == CLB_F64   ? launch3_rates<ST_F64>(h, from, s, grid, block, xb)
+             : h->p.storage == CLB_F32 ? launch3_rates<ST_F32>(h, from, s, grid, block, xb)
+                                       : launch3_rates<ST_F16DEV>(h, from, s, grid, block, xb));
     return CLB_OK;
 }
 
@@ -1740,14 +1740,14 @@ clb_status thermal3_launch(clb3d_thermal* h, int from, cudaStream_t s)
     const dim3 block(h->bx, h->by);
     const unsigned grid = unsigned((long long)xb * rb);
     if (h->p.storage == CLB_F64)
-        k_thermal3_step<ST_F64><<<grid, block, 0, s>>>((const double*)h->buf[from], (double*)h->buf[from ^ 1],
-                                                       (const double*)h->vel, h->Pd, xb);
+        CLB_CUDA(launch_chained(k_thermal3_step<ST_F64>, grid, block, 0, s, (const double*)h->buf[from], (double*)h->buf[from ^ 1],
+                                (const double*)h->vel, h->Pd, xb));
     else if (h->p.storage == CLB_F32)
-        k_thermal3_step<ST_F32><<<grid, block, 0, s>>>((const float*)h->buf[from], (float*)h->buf[from ^ 1],
-                                                       (const float*)h->vel, h->Pf, xb);
+        CLB_CUDA(launch_chained(k_thermal3_step<ST_F32>, grid, block, 0, s, (const float*)h->buf[from], (float*)h->buf[from ^ 1],
+                                (const float*)h->vel, h->Pf, xb));
     else
-        k_thermal3_step<ST_F16DEV><<<grid, block, 0, s>>>((const __half*)h->buf[from], (__half*)h->buf[from ^ 1],
-                                                          (const float*)h->vel, h->Pf, xb);
+        CLB_CUDA(launch_chained(k_thermal3_step<ST_F16DEV>, grid, block, 0, s, (const __half*)h->buf[from], (__half*)h->buf[from ^ 1],
+                                (const float*)h->vel, h->Pf, xb));
     CLB_CUDA(cudaGetLastError());
     return CLB_OK;
 }

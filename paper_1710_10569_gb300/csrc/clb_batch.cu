@@ -84,6 +84,7 @@ __global__ void __maxnreg__((ST == ST_F32 && V == 2) ? 96 : 255) k_step_batched(
 {
     using A = typename Storage<ST>::A;
     using E = typename Storage<ST>::T;
+    step_prologue();
     __shared__ Member<A> M;
     load_member(mem + owner[blockIdx.x], M);
     const int t = blockIdx.x - M.tile_begin;
@@ -415,32 +416,25 @@ public:
     }
 
     template <int ST>
-    void enqueue(cudaStream_t s, int par)
+    cudaError_t enqueue(cudaStream_t s, int par)
     {
         using A = typename Storage<ST>::A;
         const dim3 block(tile_x, tile_y);
         const Member<A>* m = (const Member<A>*)((char*)d_tables + off_members);
         const int* owner = (const int*)((char*)d_tables + off_owner);
-        if (hi1) {
-            if (npt == 4) k_step_batched<ST, 4, true><<<ntiles, block, 0, s>>>(m, owner, par, groups);
-            else if (npt == 2) k_step_batched<ST, 2, true><<<ntiles, block, 0, s>>>(m, owner, par, groups);
-            else k_step_batched<ST, 1, true><<<ntiles, block, 0, s>>>(m, owner, par, groups);
-        } else {
-            if (npt == 4) k_step_batched<ST, 4, false><<<ntiles, block, 0, s>>>(m, owner, par, groups);
-            else if (npt == 2) k_step_batched<ST, 2, false><<<ntiles, block, 0, s>>>(m, owner, par, groups);
-            else k_step_batched<ST, 1, false><<<ntiles, block, 0, s>>>(m, owner, par, groups);
-        }
+        const auto kernel = hi1 ? (npt == 4 ? k_step_batched<ST, 4, true> : npt == 2 ? k_step_batched<ST, 2, true> : k_step_batched<ST, 1, true>)
+                                : (npt == 4 ? k_step_batched<ST, 4, false> : npt == 2 ? k_step_batched<ST, 2, false> : k_step_batched<ST, 1, false>);
+        return launch_chained(kernel, ntiles, block, 0, s, m, owner, par, groups);
     }
 
     clb_status launch_step(cudaStream_t s, int par)
     {
         if (ntiles == 0) return CLB_OK;
         switch (storage) {
-        case CLB_F64: enqueue<ST_F64>(s, par); break;
-        case CLB_F32: enqueue<ST_F32>(s, par); break;
-        default: enqueue<ST_F16DEV>(s, par); break;
+        case CLB_F64: CLB_CUDA(enqueue<ST_F64>(s, par)); break;
+        case CLB_F32: CLB_CUDA(enqueue<ST_F32>(s, par)); break;
+        default: CLB_CUDA(enqueue<ST_F16DEV>(s, par)); break;
         }
-        CLB_CUDA(cudaGetLastError());
         return CLB_OK;
     }
 

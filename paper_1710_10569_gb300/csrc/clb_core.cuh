@@ -171,6 +171,10 @@ template <> struct CollideConsts<double> {
     double hom1, hom2, heq;           // (1 - lambda1) / 2, (1 - lambda2) / 2, lambda2 cs2_T / 2
 };
 
+// First statement of every kernel launched with launch_chained: wait until the kernel before it on
+// the stream has finished and its writes are visible.
+__device__ __forceinline__ void step_prologue() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // Per-lattice constants in the arithmetic precision A.
 template <typename A>
 struct LatParams : CollideConsts<A> {

@@ -50,6 +50,28 @@ void clear_error();
         if (s_ != CLB_OK) return s_;            \
     } while (0)
 
+// Launch a step kernel as a programmatic dependent of the kernel before it on the stream (in a captured
+// graph, a programmatic edge): it is set up while that kernel drains, and starts with step_prologue(),
+// which waits for it. Per step (FP32) 64 x 64 1.87 -> 1.68 us, 256 x 256 2.70 -> 2.57. No kernel
+// releases its successor before it ends: with a release at its start the waiting blocks take their
+// places while the running ones still hold theirs, and crowd onto few SMs (FP64 256 x 256: 16.6 ->
+// 25.4 us).
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, A... args)
+{
+    cudaLaunchAttribute at;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 constexpr long long kMaxNodes = 1LL << 30;  // index arithmetic and memory bound
 constexpr int kMaxEdge = 1 << 20;
 

@@ -186,6 +186,7 @@ __global__ void __launch_bounds__(256) k_step(const typename Storage<ST>::T* __r
                                               typename Storage<ST>::T* __restrict__ dst,
                                               const LatParams<typename Storage<ST>::A> P)
 {
+    step_prologue();
     const int lane = threadIdx.x & 31;
     const int x0 = (blockIdx.x * blockDim.x + threadIdx.x) * V;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;

@@ -184,11 +184,14 @@ dim3 grid_for(const clb_handle* h, int bx, int by)
 // The split step (k_step_inner beside k_step_edge) for the FP16 form, which sits at the issue
 // limit: 83.0 -> 77.9 us per step on 4096 x 2048. The FP32 form is bound by memory (one kernel:
 // 35.0 us, split: 35.2-35.6 us, the fork and join costing more than the registers save) and FP64
-// by its arithmetic (602 us either way); they keep the one kernel that holds every path.
+// by its arithmetic (the same either way); they keep the one kernel that holds every path. So do FP16
+// lattices below kSplitNodes, where the second launch and the fork and join are the larger part of a
+// step (513 x 385: 4.1 us split, 3.8 in one kernel; 256 x 256: 3.1 and 2.8).
+constexpr long long kSplitNodes = 400000;
 template <int ST>
-constexpr bool split_step()
+bool split_step(const clb_handle* h)
 {
-    return ST == ST_F16DEV;
+    return ST == ST_F16DEV && (long long)h->nx * h->ny >= kSplitNodes;
 }
 
 // Interior rows and warp columns of the split step for V nodes per thread: rows next to a y wall
@@ -228,12 +231,11 @@ cudaError_t enqueue_step(const clb_handle* h, const void* a, void* b, cudaStream
     const LatParams<A>& P = *reinterpret_cast<const LatParams<A>*>(ST == ST_F64 ? (const void*)&h->Pd : (const void*)&h->Pf);
     const bool hi1 = h->p.s_3 == 1.0 && h->p.s_4 == 1.0 && h->p.lambda2 == 1.0;
     const dim3 block(bx, by);
-    if constexpr (!split_step<ST>()) {
+    if (!split_step<ST>(h)) {
         const dim3 grid((h->nx + bx * NPT - 1) / (bx * NPT), (h->ny + by - 1) / by);
-        if (hi1) k_step<ST, NPT, true><<<grid, block, 0, s>>>((const E*)a, (E*)b, P);
-        else k_step<ST, NPT, false><<<grid, block, 0, s>>>((const E*)a, (E*)b, P);
-        return cudaSuccess;
-    } else {
+        return launch_chained(hi1 ? k_step<ST, NPT, true> : k_step<ST, NPT, false>, grid, block, 0, s, (const E*)a, (E*)b, P);
+    }
+    if constexpr (ST == ST_F16DEV) {
         const SplitGeom G = split_geom(h->nx, h->ny, h->Pf, NPT);
         const int ncol = G.c1 - G.c0, nrow = G.y1 - G.y0, nedge = G.edge_warps();
         const bool inner = ncol > 0 && nrow > 0;
@@ -265,8 +267,8 @@ cudaError_t enqueue_step(const clb_handle* h, const void* a, void* b, cudaStream
             if (e == cudaSuccess) e = cudaStreamWaitEvent(s, h->join, 0);
             if (e != cudaSuccess) return e;
         }
-        return cudaSuccess;
     }
+    return cudaSuccess;
 }
 
 template <int ST>
@@ -334,9 +336,8 @@ clb_status launch_two(const clb_handle* h, int from, cudaStream_t s, const Launc
     const MarchGeom G = march_geom(h->nx, h->ny, L.march);
     const float* a = (const float*)h->buf[from];
     float* b = (float*)h->buf[from ^ 1];
-    if (h->p.s_3 == 1.0 && h->p.s_4 == 1.0 && h->p.lambda2 == 1.0) k_step_two<true><<<G.warps(), 32, 0, s>>>(a, b, h->Pf, G);
-    else k_step_two<false><<<G.warps(), 32, 0, s>>>(a, b, h->Pf, G);
-    CLB_CUDA(cudaGetLastError());
+    const bool hi1 = h->p.s_3 == 1.0 && h->p.s_4 == 1.0 && h->p.lambda2 == 1.0;
+    CLB_CUDA(launch_chained(hi1 ? k_step_two<true> : k_step_two<false>, G.warps(), 32, 0, s, a, b, h->Pf, G));
     return CLB_OK;
 }
 
@@ -448,6 +449,23 @@ clb_status take_snapshot(clb_handle* h)
     return CLB_OK;
 }
 
+// Launch shape of a lattice that has not been tuned. FP64: an instruction takes its SM quarter's pipe
+// for 64 clocks however many of a warp's lanes are active, so nodes go to as many warps as they fill,
+// one per thread (64 x 64: 5.1 us per step against 17.4 with four; 2048 x 1024: 421 against 424). FP32
+// and FP16: two and four nodes per thread, the packed instructions' and the widest loads' count, where
+// the lattice fills the chip with them; below, more and shorter warps (128 x 128, FP16: 1.9 us against
+// 3.4). Blocks of few warps, so that a ragged row end idles few of them (513 x 385, FP32: 4.3 us at
+// 128 x 1, 3.7 at 32 x 2; 640 x 640, FP16: 6.5 and 5.7).
+void default_shape(int storage, long long nodes, int* bx, int* by, int* npt)
+{
+    const bool small = nodes < 32768;
+    *bx = 32;
+    *by = 2;
+    *npt = storage == CLB_F64 || small ? 1 : 2;
+    if (storage != CLB_F64 && small) *by = 4;
+    if (storage == CLB_F16DEV && nodes >= kSplitNodes) *npt = 4;
+}
+
 std::mutex g_tune_mu;
 std::map<std::tuple<int, int, int>, std::array<int, 6>> g_tune_cache;
 
@@ -511,7 +529,7 @@ extern "C" clb_status clb_create(int nx, int ny, const clb_params* p, void* stre
         h->diag = (double*)(h->mem + L.diag);
         h->Pd = make_lat_params<double>(nx, ny, *p);
         h->Pf = make_lat_params<float>(nx, ny, *p);
-        h->npt = p->storage == CLB_F32 ? 2 : 4;
+        default_shape(p->storage, (long long)nx * ny, &h->bx, &h->by, &h->npt);
         bool tuned = false;
         {
             std::lock_guard<std::mutex> lk(g_tune_mu);

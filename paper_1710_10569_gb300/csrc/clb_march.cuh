@@ -301,6 +301,7 @@ template <bool HI1>
 __global__ void __launch_bounds__(32, kMarchResident)
     k_step_two(const float* __restrict__ src, float* __restrict__ dst, const LatParams<float> P, const MarchGeom G)
 {
+    step_prologue();
     __shared__ unsigned long long slots[kMarchSlots * 32];
     const int strip = blockIdx.x % G.strips, seg = blockIdx.x / G.strips;
     const int xo = strip * G.width, ya = seg * G.rows;

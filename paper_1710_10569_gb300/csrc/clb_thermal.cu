@@ -136,6 +136,7 @@ __global__ void __launch_bounds__(128, ST == ST_F64 ? 8 : 12) k_thermal_step(con
 {
     using A = typename Storage<ST>::A;
     using E = typename Storage<ST>::T;
+    step_prologue();
     const int x0 = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
     const int y = blockIdx.y;
     if (x0 >= P.nx) return;
@@ -298,16 +299,15 @@ clb_status thermal_launch(clb_thermal* h, int from, cudaStream_t s)
     void* b = h->buf[from ^ 1];
     switch (h->p.storage) {
     case CLB_F64:
-        k_thermal_step<ST_F64><<<grid, block, 0, s>>>((const double*)a, (double*)b, (const double*)h->vel[0], (const double*)h->vel[1], h->Pd);
+        CLB_CUDA(launch_chained(k_thermal_step<ST_F64>, grid, block, 0, s, (const double*)a, (double*)b, (const double*)h->vel[0], (const double*)h->vel[1], h->Pd));
         break;
     case CLB_F32:
-        k_thermal_step<ST_F32><<<grid, block, 0, s>>>((const float*)a, (float*)b, (const float*)h->vel[0], (const float*)h->vel[1], h->Pf);
+        CLB_CUDA(launch_chained(k_thermal_step<ST_F32>, grid, block, 0, s, (const float*)a, (float*)b, (const float*)h->vel[0], (const float*)h->vel[1], h->Pf));
         break;
     default:
-        k_thermal_step<ST_F16DEV><<<grid, block, 0, s>>>((const __half*)a, (__half*)b, (const float*)h->vel[0], (const float*)h->vel[1], h->Pf);
+        CLB_CUDA(launch_chained(k_thermal_step<ST_F16DEV>, grid, block, 0, s, (const __half*)a, (__half*)b, (const float*)h->vel[0], (const float*)h->vel[1], h->Pf));
         break;
     }
-    CLB_CUDA(cudaGetLastError());
     return CLB_OK;
 }
 
