@@ -76,16 +76,17 @@ struct MarchCols {
     bool pairs;  // every lane's two columns load as one aligned pair: warp-uniform
     MarchWalls w;
 };
-__device__ __forceinline__ MarchCols march_cols(const LatParams<float>& P, int xo, int lane)
+// Columns start + 2 lane and the next (start even).
+__device__ __forceinline__ MarchCols march_cols(const LatParams<float>& P, int start, int lane)
 {
     MarchCols M;
-    const int x0 = xo - 2 + 2 * lane;
+    const int x0 = start + 2 * lane;
     // its own two where they exist (a periodic row wraps); lanes beyond an x wall, whose values reach
     // no stored node, load columns 0 and 1
     int xa = x0, xb = x0 + 1;
     if (P.per_x) {
-        xa = xa < 0 ? xa + P.nx : xa % P.nx;
-        xb = xb < 0 ? xb + P.nx : xb % P.nx;
+        xa = (xa % P.nx + P.nx) % P.nx;
+        xb = (xb % P.nx + P.nx) % P.nx;
     } else if (xa < 0 || xa >= P.nx) {
         xa = 0;
         xb = 1;
@@ -289,7 +290,7 @@ __device__ __forceinline__ void march_two(const float* __restrict__ src, float* 
                                           const LatParams<float>& P, int xo, int xe, int ya, int yb, int lane,
                                           unsigned long long* __restrict__ slots, int stride)
 {
-    const MarchCols M = march_cols(P, xo, lane);
+    const MarchCols M = march_cols(P, xo - 2, lane);
     if (M.pairs && !M.w.any_x && (P.per_y || (ya >= 2 && yb <= P.ny - 2)))
         march_rows<HI1, false>(src, dst, P, M, xo, xe, ya, yb, lane, slots, stride);
     else

@@ -7,8 +7,9 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <type_traits>
 
-#include "clb_kernels.cuh"
+#include "clb_march.cuh"
 
 using namespace clb;
 
@@ -186,6 +187,229 @@ __global__ void __launch_bounds__(128, ST == ST_F64 ? 8 : 12) k_thermal_step(con
     }
 }
 
+// ---------------------------------------------------------------------------------------------
+// kSteps time steps per launch (FP32 and FP16 forms, large lattices). One step moves 48 bytes a node
+// (FP32: 5 populations in and out, the velocity in) for some 45 operations and runs at the copy
+// bandwidth; what can give is the bytes per step. As in the coupled lattice's two-step kernel
+// (clb_march.cuh) a warp takes a window of 64 columns, two nodes per lane, and marches along y: level
+// k of the pipeline computes step k + 1 of row r - k from the rows that level k - 1 has just left. Here
+// a level hands on five populations only, so the rows between levels stay in registers (the
+// velocities, read once, in shared-memory slots private to the thread). Each step loses the outermost
+// column of the window (of 64 columns the inner 56 are stored) and a row at either end of the segment.
+// The arithmetic of a node is that of k_thermal_step, with the intermediate states rounded to the
+// storage type: bitwise the same. Measured on 4096 x 4096 (us per step, one step per launch -> four):
+// FP32 117.2 -> 45.9 (365 GLUPS), FP16 90.0 -> 47.8. It is then bound by the latency of a turn, whose
+// levels follow one another (some 110 instructions per pair of nodes and level, 45 of them packed
+// arithmetic, at 24 warps per SM). Tried: turns unrolled by two and four, which saves the moves of the
+// handed-on rows but takes 120 registers (51.8 at 16 warps per SM); the next row loaded a turn
+// ahead (54.2); velocities in registers (54.4).
+constexpr int kSteps = 4;                       // a power of two
+constexpr int kMarchOutT = 64 - 4 * ((kSteps + 1) / 2);
+constexpr int kLanesLost = (kSteps + 1) / 2;    // lanes at either end of a window that store nothing
+constexpr int kResidentT = 24;                  // warps per SM that the register bound of k_thermal_steps leaves
+
+__device__ __forceinline__ F2 load_pair(const float* p)
+{
+    F2 r;
+    r.u = *reinterpret_cast<const unsigned long long*>(p);
+    return r;
+}
+__device__ __forceinline__ F2 load_pair(const __half* p)
+{
+    const __half2 h = *reinterpret_cast<const __half2*>(p);
+    return F2(__low2float(h), __high2float(h));
+}
+__device__ __forceinline__ void store_pair(float* p, F2 v) { *reinterpret_cast<unsigned long long*>(p) = v.u; }
+__device__ __forceinline__ void store_pair(__half* p, F2 v)
+{
+    float a, b;
+    v.split(a, b);
+    *reinterpret_cast<__half2*>(p) = __floats2half2_rn(a, b);
+}
+// The values as the storage type holds them.
+__device__ __forceinline__ F2 as_stored(F2 v, const float*) { return v; }
+__device__ __forceinline__ F2 as_stored(F2 v, const __half*)
+{
+    float a, b;
+    v.split(a, b);
+    const __half2 h = __floats2half2_rn(a, b);
+    return F2(__low2float(h), __high2float(h));
+}
+
+// Pull and collide one row of a window: before the shift along x, g[i] holds population i of this
+// lane's nodes on the row it is pulled from (bounced at a y wall: the opposite one of the own row).
+template <bool HI1, bool WALLS>
+__device__ __forceinline__ void thermal_row(const LatParams<float>& P, F2 g[NT], const MarchWalls& w, F2 u, F2 v, float Tb)
+{
+    const F2 g1 = g[1], g3 = g[3];
+    g[1] = pull_shr(g1);
+    g[3] = pull_shl(g3);
+    if (WALLS && (w.bottom || w.top || w.any_x)) {
+        float a[NT], b[NT], oa, ob;
+#pragma unroll
+        for (int i = 0; i < NT; ++i) g[i].split(a[i], b[i]);
+        g3.split(oa, ob);
+        if (w.m0 & 1) a[1] = oa;
+        g1.split(oa, ob);
+        if (w.m0 & 2) a[3] = oa;
+        if (w.m1 & 2) b[3] = ob;
+        const auto rules = [&](float* q, int m) {
+            q[2] = w.bottom ? q[2] : q[2] - P.T_dyw;
+            q[4] = w.top ? q[4] : q[4] + P.T_dyw;
+            if ((m & 1) && P.kind[0] == WALL_DIRICHLET) q[1] = P.Tw_c2[0] - q[1];
+            if ((m & 2) && P.kind[1] == WALL_DIRICHLET) q[3] = P.Tw_c2[1] - q[3];
+            if (w.bottom && P.kind[2] == WALL_DIRICHLET) q[2] = P.Tw_c2[2] - q[2];
+            if (w.top && P.kind[3] == WALL_DIRICHLET) q[4] = P.Tw_c2[3] - q[4];
+        };
+        rules(a, w.m0);
+        rules(b, w.m1);
+#pragma unroll
+        for (int i = 0; i < NT; ++i) g[i] = F2(a[i], b[i]);
+    } else {
+        // re-based to this row (see thermal_gather)
+        g[2] = g[2] - F2(P.T_dyw);
+        g[4] = g[4] + F2(P.T_dyw);
+    }
+    const F2 dT = (g[0] + g[1]) + (g[2] + g[3]) + g[4];
+    collide_d2q5_dev<HI1>(P, F2(Tb) + dT, dT, u, v, g);
+}
+
+// What level k of the pipeline has left for level k + 1: g0, g1, g3 of its last row, g2 of its last two
+// (and g4 of its last, for a bounce at the bottom wall).
+struct ThermalPipe {
+    F2 c0[kSteps - 1], c1[kSteps - 1], c3[kSteps - 1], up[kSteps - 1], upp[kSteps - 1], dn[kSteps - 1];
+};
+
+// kSteps steps of rows [ya, yb), columns [xo, xe) by one warp (xo even, xe - xo <= kMarchOutT, xe even or
+// nx). WALLS = false: no row (ya - kSteps + 1 to yb + kSteps - 2) or column next to a wall, all columns load
+// as aligned pairs.
+template <int ST, bool HI1, bool WALLS>
+__device__ __forceinline__ void thermal_march(const typename Storage<ST>::T* __restrict__ src,
+                                              typename Storage<ST>::T* __restrict__ dst, const float* __restrict__ ux,
+                                              const float* __restrict__ uy, const LatParams<float>& P, const MarchCols& M,
+                                              int xo, int xe, int ya, int yb, int lane, F2* __restrict__ slots)
+{
+    using E = typename Storage<ST>::T;
+    constexpr int L = kSteps - 1;  // rows that a segment needs beyond its own at either end, for the first step
+    const int x0 = xo - 2 * kLanesLost + 2 * lane;
+    const bool pairs = !WALLS || M.pairs;
+    const bool vpairs = pairs && P.nx % 2 == 0;  // velocity rows are dense
+    MarchWalls w = M.w;
+    const bool store = lane >= kLanesLost && lane < 32 - kLanesLost && x0 < xe;
+    const bool store2 = !WALLS || x0 + 1 < P.nx;
+    const long long pl = P.plane;
+    const auto wrap = [&](int r) { return r < 0 ? r + P.ny : r >= P.ny ? r - P.ny : r; };
+    ThermalPipe S;
+#pragma unroll
+    for (int k = 0; k < L; ++k) S.c0[k] = S.c1[k] = S.c3[k] = S.up[k] = S.upp[k] = S.dn[k] = F2(0.0f, 0.0f);
+    const auto vel = [&](int row, int c) -> F2& { return slots[((row & (kSteps - 1)) * 2 + c) * 32]; };
+
+    // the populations that row r pulls and its velocity
+    const auto load_row = [&](int r, F2 g[NT], F2& u, F2& v) {
+        const int y = wrap(r);
+        const bool bottom = WALLS && !P.per_y && y == 0, top = WALLS && !P.per_y && y == P.ny - 1;
+        const E* sc = src + (long long)y * P.pitch;
+        // across a y wall the node's own opposite plane
+        const E* su = bottom ? sc + 2 * pl : src + (long long)(y > 0 ? y - 1 : P.ny - 1) * P.pitch;
+        const E* sd = top ? sc - 2 * pl : src + (long long)(y < P.ny - 1 ? y + 1 : 0) * P.pitch;
+        const auto load = [&](const E* p) { return pairs ? load_pair(p + M.xa) : F2(to_a(p[M.xa]), to_a(p[M.xb])); };
+        g[0] = load(sc);
+        g[1] = load(sc + pl);
+        g[3] = load(sc + 3 * pl);
+        g[2] = load(su + 2 * pl);
+        g[4] = load(sd + 4 * pl);
+        const long long n = (long long)y * P.nx;
+        u = vpairs ? load_pair(ux + n + M.xa) : F2(ux[n + M.xa], ux[n + M.xb]);
+        v = vpairs ? load_pair(uy + n + M.xa) : F2(uy[n + M.xa], uy[n + M.xb]);
+    };
+    // One turn of the pipeline: row r enters with its pulled populations in g, row r - L leaves. ALL:
+    // every level has its rows (not so in the first turns, nor beyond the top wall).
+    const auto turn = [&](auto all, int r, F2 g[NT], F2 u, F2 v) {
+        constexpr bool ALL = decltype(all)::value;
+        if (ALL || !WALLS || P.per_y || r < P.ny) {
+            w.bottom = WALLS && !P.per_y && r == 0;
+            w.top = WALLS && !P.per_y && r == P.ny - 1;
+            vel(r, 0) = u;
+            vel(r, 1) = v;
+            thermal_row<HI1, WALLS>(P, g, w, u, v, row_base(P, wrap(r)));
+        }
+        bool left = true;  // level k - 1 has just left row q + 1 in g
+#pragma unroll
+        for (int k = 1; k < kSteps; ++k) {
+            const int q = r - k;  // level k: step k + 1 of row q
+            w.bottom = WALLS && !P.per_y && q == 0;
+            w.top = WALLS && !P.per_y && q == P.ny - 1;
+            const F2 above = as_stored(g[4], src);
+            F2 h[NT];
+            h[0] = S.c0[k - 1];
+            h[1] = S.c1[k - 1];
+            h[3] = S.c3[k - 1];
+            h[2] = w.bottom ? S.dn[k - 1] : S.upp[k - 1];
+            h[4] = w.top ? S.up[k - 1] : above;
+            if (ALL || left) {
+                S.upp[k - 1] = S.up[k - 1];
+                S.up[k - 1] = as_stored(g[2], src);
+                S.c0[k - 1] = as_stored(g[0], src);
+                S.c1[k - 1] = as_stored(g[1], src);
+                S.c3[k - 1] = as_stored(g[3], src);
+                if (WALLS) S.dn[k - 1] = above;
+            }
+            left = left && q >= (WALLS && !P.per_y ? max(0, ya - L + k) : ya - L + k);
+            if (ALL || (left && (!WALLS || P.per_y || q < P.ny)))
+                thermal_row<HI1, WALLS>(P, h, w, vel(q, 0), vel(q, 1), row_base(P, wrap(q)));
+#pragma unroll
+            for (int i = 0; i < NT; ++i) g[i] = h[i];
+        }
+        if (ALL || left) {
+            if (store) {
+                E* dc = dst + (long long)(r - L) * P.pitch + x0;
+#pragma unroll
+                for (int i = 0; i < NT; ++i) {
+                    if (store2) {
+                        store_pair(dc + i * pl, g[i]);
+                    } else {
+                        float a, b;
+                        g[i].split(a, b);
+                        dc[i * pl] = from_a(a, (E*)nullptr);
+                    }
+                }
+            }
+        }
+    };
+    const int last = yb - 1 + L;
+    int r = WALLS && !P.per_y ? max(0, ya - L) : ya - L;
+    // the first turns fill the pipeline; with walls every turn is of this kind
+    const int full = WALLS ? last + 1 : r + 2 * L;
+    F2 g[NT], u, v;
+    for (; r < full; ++r) {
+        if (!WALLS || P.per_y || r < P.ny) load_row(r, g, u, v);
+        turn(std::false_type(), r, g, u, v);
+    }
+    if constexpr (!WALLS) {
+        for (; r <= last; ++r) {
+            load_row(r, g, u, v);
+            turn(std::true_type(), r, g, u, v);
+        }
+    }
+}
+
+// kSteps steps over a lattice: block (one warp) b takes strip b % strips of segment b / strips.
+template <int ST, bool HI1>
+__global__ void __launch_bounds__(32, kResidentT)
+    k_thermal_steps(const typename Storage<ST>::T* __restrict__ src, typename Storage<ST>::T* __restrict__ dst,
+                    const float* __restrict__ ux, const float* __restrict__ uy, const LatParams<float> P, const MarchGeom G)
+{
+    step_prologue();
+    __shared__ F2 slots[2 * kSteps * 32];
+    const int strip = blockIdx.x % G.strips, seg = blockIdx.x / G.strips;
+    const int xo = strip * G.width, xe = min(P.nx, xo + G.width), ya = seg * G.rows, yb = min(P.ny, ya + G.rows);
+    const MarchCols M = march_cols(P, xo - 2 * kLanesLost, threadIdx.x);
+    if (M.pairs && !M.w.any_x && (P.per_y || (ya >= kSteps && yb <= P.ny - kSteps)))
+        thermal_march<ST, HI1, false>(src, dst, ux, uy, P, M, xo, xe, ya, yb, threadIdx.x, slots + threadIdx.x);
+    else
+        thermal_march<ST, HI1, true>(src, dst, ux, uy, P, M, xo, xe, ya, yb, threadIdx.x, slots + threadIdx.x);
+}
+
 // g^eq(T, u) written to the slots the next pull reads (as k_init does for the coupled step), and
 // the velocity stored in the handle's precision.
 template <int ST>
@@ -273,6 +497,7 @@ struct clb_thermal {
     double* stage = nullptr;
     int cur = 0;
     long steps = 0;
+    int march = 0;  // > 0: kSteps steps per launch (k_thermal_steps), in segments of this many rows
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     LatParams<double> Pd{};
     LatParams<float> Pf{};
@@ -308,6 +533,60 @@ clb_status thermal_launch(clb_thermal* h, int from, cudaStream_t s)
         CLB_CUDA(launch_chained(k_thermal_step<ST_F16DEV>, grid, block, 0, s, (const __half*)a, (__half*)b, (const float*)h->vel[0], (const float*)h->vel[1], h->Pf));
         break;
     }
+    return CLB_OK;
+}
+
+MarchGeom thermal_geom(int nx, int ny, int rows)
+{
+    MarchGeom G;
+    G.strips = (nx + kMarchOutT - 1) / kMarchOutT;
+    G.width = ((nx + G.strips - 1) / G.strips + 1) & ~1;
+    G.strips = (nx + G.width - 1) / G.width;
+    G.rows = rows;
+    G.segs = (ny + rows - 1) / rows;
+    return G;
+}
+
+// Rows per segment of the kSteps-step kernel, 0 where one step per launch is the faster form (small
+// lattices: 512 x 512 2.8 us against 2.9, 700 x 700 4.1 against 3.3; few rows; rows that fill their
+// windows badly; wet walls, whose nodes pull through their neighbours; FP64, bound by its arithmetic).
+// A segment of R rows takes R + 2 (kSteps - 1) turns; the R of the least turns over the rounds of
+// resident warps is taken, counting two rounds at least: warps that all start together load and
+// compute in step, and one round runs at half the rate (2048 x 2048: one of 22 rows 17.2 us per step,
+// two of 12 to 14 rows 14.7 - 15.2; 4096 x 4096: two of 44 rows 45.9, three of 28 46.8).
+constexpr long long kMarchNodesT = 400000;
+int thermal_rows_rule(int nx, int ny, const clb_params& p, int sms)
+{
+    const bool wet = p.wall[0] == CLB_WALL_WET || p.wall[2] == CLB_WALL_WET;
+    if (p.storage == CLB_F64 || wet || (long long)nx * ny < kMarchNodesT || ny < 24) return 0;
+    if ((double)nx < 0.7 * kMarchOutT * thermal_geom(nx, ny, 6).strips) return 0;
+    int best = 6;
+    long long least = 1LL << 60;
+    for (int rows = 6; rows <= 64; ++rows) {
+        const long long warps = thermal_geom(nx, ny, rows).warps(), round = (long long)sms * kResidentT;
+        const long long turns = (rows + 2 * (kSteps - 1)) * std::max(2LL, (warps + round - 1) / round);
+        if (turns < least) {
+            least = turns;
+            best = rows;
+        }
+    }
+    return best;
+}
+
+// kSteps steps from buffer `from` into the other one.
+clb_status thermal_launch_steps(clb_thermal* h, int from, cudaStream_t s)
+{
+    const MarchGeom G = thermal_geom(h->nx, h->ny, h->march);
+    const void* a = h->buf[from];
+    void* b = h->buf[from ^ 1];
+    const float *u = (const float*)h->vel[0], *v = (const float*)h->vel[1];
+    const bool hi1 = h->p.lambda2 == 1.0;
+    if (h->p.storage == CLB_F32)
+        CLB_CUDA(launch_chained(hi1 ? k_thermal_steps<ST_F32, true> : k_thermal_steps<ST_F32, false>, G.warps(), 32, 0, s,
+                                (const float*)a, (float*)b, u, v, h->Pf, G));
+    else
+        CLB_CUDA(launch_chained(hi1 ? k_thermal_steps<ST_F16DEV, true> : k_thermal_steps<ST_F16DEV, false>, G.warps(), 32, 0,
+                                s, (const __half*)a, (__half*)b, u, v, h->Pf, G));
     return CLB_OK;
 }
 
@@ -363,6 +642,9 @@ extern "C" clb_status clb_thermal_create(int nx, int ny, const clb_params* p, vo
     h->stage = (double*)(h->mem + 2 * bb + 2 * vb);
     h->Pd = make_lat_params<double>(nx, ny, *p);
     h->Pf = make_lat_params<float>(nx, ny, *p);
+    int sms = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+    h->march = thermal_rows_rule(nx, ny, *p, std::max(1, sms));
     e = cudaMemsetAsync(h->mem, 0, 2 * bb, h->stream);
     if (e != cudaSuccess) {
         clb_thermal_destroy(h);
@@ -421,7 +703,9 @@ extern "C" clb_status clb_thermal_step(clb_thermal* h, long n)
         if (h->graph[par]) continue;
         CLB_CUDA(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
         clb_status st = CLB_OK;
-        for (int k = 0; k < kChunkT && st == CLB_OK; ++k) st = thermal_launch(h, par ^ (k & 1), h->cap);
+        const int per = h->march > 0 ? kSteps : 1;  // steps per launch; kChunkT / per launches are an even number
+        for (int k = 0; k < kChunkT / per && st == CLB_OK; ++k)
+            st = per > 1 ? thermal_launch_steps(h, par ^ (k & 1), h->cap) : thermal_launch(h, par ^ (k & 1), h->cap);
         cudaGraph_t g = nullptr;
         cudaError_t e = cudaStreamEndCapture(h->cap, &g);
         if (st != CLB_OK) {
@@ -437,6 +721,11 @@ extern "C" clb_status clb_thermal_step(clb_thermal* h, long n)
         CLB_CUDA(cudaGraphLaunch(h->graph[h->cur], h->stream));
         n -= kChunkT;
         h->steps += kChunkT;
+    }
+    for (; h->march > 0 && n >= kSteps; n -= kSteps) {
+        CLB_TRY(thermal_launch_steps(h, h->cur, h->stream));
+        h->cur ^= 1;
+        h->steps += kSteps;
     }
     for (; n > 0; --n) {
         CLB_TRY(thermal_launch(h, h->cur, h->stream));

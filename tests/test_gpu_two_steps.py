@@ -1,4 +1,6 @@
-"""The FP32 kernel that takes two steps per launch (large lattices) against the one-step kernel, which
+"""The kernels that take several steps per launch (large lattices) against one step per launch.
+
+The FP32 kernel that takes two steps per launch against the one-step kernel, which
 an explicit launch shape selects: every population bitwise, over windows and rows of every kind (one
 and several windows per row, odd rows, a last window of one column, rows that end in mid-window,
 segments of every remainder), every wall layout, fixed and moving, both collision forms, and even
@@ -43,3 +45,25 @@ def test_two_steps_per_launch_equal_one(clb, layout, shape, steps):
         lat.close()
     for a, b in zip(*got):
         assert np.isfinite(a).all() and np.array_equal(a, b)
+
+
+# The temperature equation alone: four steps per launch against the same number of calls of one step.
+@pytest.mark.parametrize("shape", [(8193, 49), (4096, 101), (1121, 358), (112, 3601), (55, 7301), (703, 702)],
+                         ids=lambda v: f"{v[0]}x{v[1]}")
+@pytest.mark.parametrize("layout", sorted(LAYOUTS))
+def test_four_thermal_steps_per_launch_equal_one(clb, layout, shape):
+    nx, ny = shape
+    storage = W.STORAGE_F32 if (nx + ny) % 2 == 0 else W.STORAGE_F16DEV
+    rng = np.random.default_rng(nx)
+    p = W.default_params(nu=0.05, kappa=0.03, storage=storage, wall=LAYOUTS[layout], T_wall=(0.3, -0.2, 0.5, -0.4),
+                         lambda2=1.0 if ny % 3 else 1.3, u_wall=((0, 0.02), (0, 0.01), (0.02, 0.03), (0.01, -0.02)))
+    T, ux, uy = rng.uniform(-0.5, 0.5, (ny, nx)), rng.uniform(-0.1, 0.1, (ny, nx)), rng.uniform(-0.1, 0.1, (ny, nx))
+    got = []
+    for calls in ([9], [1] * 9):
+        h = clb.Thermal(nx, ny, p)
+        h.init(T, ux, uy)
+        for n in calls:
+            h.step(n)
+        got.append(h.populations())
+        h.close()
+    assert np.isfinite(got[0]).all() and np.array_equal(*got)
