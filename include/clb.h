@@ -286,12 +286,13 @@ clb_status clb_batch_run(clb_batch *b, double tol, long max_steps, long interval
  * number of its last check, and its steps since init. Host arrays of n entries, any may be NULL.
  * Reads host bookkeeping only (no device work). */
 clb_status clb_batch_status(clb_batch *b, int *status, double *er, long *steps, double *nu);
-/* Tile shape of the batched launch: threads along x (32..256), rows (block_x * rows <= 256) and
- * nodes per thread (1, 2, 4). Each block steps 1, 2, 4, ... such groups of rows one after another
- * (it fetches its lattice's descriptor once): as many as keep a block at 2048 nodes or fewer and
- * the launch at 8 or more rounds of the blocks the device holds at once. clb_batch_autotune times
- * candidates over the whole batch (the populations are restored afterwards) and keeps the
- * fastest. Results do not depend on it. */
+/* Tile shape of the batched launch of one step: threads along x (32..256), rows (block_x * rows <=
+ * 256) and nodes per thread (1, 2, 4). FP32 batches of some size without wet walls take pairs of steps
+ * in one launch of its own shape, until a tile shape is set; clb_batch_autotune weighs both. Each
+ * block steps 1, 2, 4, ... such groups of rows one after another (it fetches its lattice's descriptor
+ * once): as many as keep a block at 2048 nodes or fewer and the launch at 8 or more rounds of the
+ * blocks the device holds at once. clb_batch_autotune times candidates over the whole batch (the
+ * populations are restored afterwards) and keeps the fastest. Results do not depend on it. */
 clb_status clb_batch_set_tile(clb_batch *b, int tile_x, int tile_y, int nodes_per_thread);
 clb_status clb_batch_autotune(clb_batch *b, int *tile_x, int *tile_y, int *nodes_per_thread);
 /* Launch geometry of the next batched step over the active instances: tile shape, groups of rows

@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "clb_diag.cuh"
+#include "clb_march.cuh"
 
 using namespace clb;
 
@@ -29,6 +30,7 @@ struct Member {
     int tiles_x;
     int tile_begin;
     int row_begin;
+    int strip_width, strips, march_begin;  // the two-step launch: strips and first block of the lattice
     int axis;
     double nodes, cells, H, dT, sign, kappa, u_ref, dT_ref;
 };
@@ -84,9 +86,9 @@ __global__ void __maxnreg__((ST == ST_F32 && V == 2) ? 96 : 255) k_step_batched(
 {
     using A = typename Storage<ST>::A;
     using E = typename Storage<ST>::T;
-    step_prologue();
     __shared__ Member<A> M;
-    load_member(mem + owner[blockIdx.x], M);
+    load_member(mem + owner[blockIdx.x], M);  // the tables are not written by steps: fetched before the wait
+    step_prologue();
     const int t = blockIdx.x - M.tile_begin;
     const int tx = t % M.tiles_x, ty = t / M.tiles_x;
     const int lane = threadIdx.x & 31;
@@ -140,6 +142,25 @@ __global__ void __maxnreg__((ST == ST_F32 && V == 2) ? 96 : 255) k_step_batched(
         collide_any<Storage<ST>::DEV, HI1>(M.P, f, g, row_base(M.P, y));
         store_node(dst, M.P, x, y, f, g);
     }
+}
+
+// Two time steps of every lattice (FP32, no wet walls; clb_march.cuh): block (one warp) b takes strip
+// t % strips of segment t / strips of lattice owner[b], t = b - march_begin. 48 cavities of edge 64 to 512
+// (3.3 million nodes): 68.5 us per step with one step per launch, 49.3 with two; 256 of them 307 and 222.
+// Bound by the FP32 pipe and the repeated columns of short rows (a lattice's columns are cut into equal
+// windows of 60 at most).
+template <bool HI1>
+__global__ void __launch_bounds__(32, kMarchResident)
+    k_step_two_batched(const Member<float>* __restrict__ mem, const int* __restrict__ owner, int parity, int rows)
+{
+    __shared__ Member<float> M;
+    __shared__ unsigned long long slots[kMarchSlots * 32];
+    load_member(mem + owner[blockIdx.x], M);
+    step_prologue();
+    const int t = blockIdx.x - M.march_begin;
+    const int xo = (t % M.strips) * M.strip_width, ya = (t / M.strips) * rows;
+    march_two<HI1>((const float*)M.buf[parity], (float*)M.buf[parity ^ 1], M.P, xo, min(M.P.nx, xo + M.strip_width), ya,
+                   min(M.P.ny, ya + rows), threadIdx.x, slots + threadIdx.x, 32);
 }
 
 // Blocks of k_step_batched<ST, V, HI1> resident on the whole device at once.
@@ -226,7 +247,7 @@ void carve(Lattice& L, char* base)
 }
 
 template <typename A>
-Member<A> make_member(const Lattice& L, int tile_x, int npt, int tile_begin, int row_begin, double* diag)
+Member<A> make_member(const Lattice& L, int tile_x, int npt, int tile_begin, int row_begin, int march_begin, double* diag)
 {
     Member<A> m;
     std::memset(&m, 0, sizeof(m));
@@ -239,6 +260,10 @@ Member<A> make_member(const Lattice& L, int tile_x, int npt, int tile_begin, int
     m.tiles_x = (L.nx + tile_x * npt - 1) / (tile_x * npt);
     m.tile_begin = tile_begin;
     m.row_begin = row_begin;
+    const MarchGeom mg = march_geom(L.nx, L.ny, 1);
+    m.strip_width = mg.width;
+    m.strips = mg.strips;
+    m.march_begin = march_begin;
     m.axis = L.axis;
     const NuGeom g = nu_geom(L.nx, L.ny, L.p, L.axis);
     m.nodes = double(L.nx) * L.ny;
@@ -270,6 +295,12 @@ long tiles_of(int nx, int ny, int tile_x, int tile_y, int npt)
     return (long)((nx + tile_x * npt - 1) / (tile_x * npt)) * ((ny + tile_y - 1) / tile_y);
 }
 
+// Batches of fewer nodes step one at a time (288,000 nodes in 48 cavities: 8.7 us against 8.2 at the best
+// number of rows and 9.4 at others; 400,000 in 12: 10.0 against 9.5; 1.1 million in 8: 27.1 against 18.5),
+// and any batch whose lattices fill their windows badly, by the time of
+// one step in us.
+constexpr double kMarchBatchNodes = 400000, kBatchStepUs = 3.0, kBatchNodeUs = 112.0 / 6.2e6;
+
 constexpr int kDiagStride = 16;  // doubles of diagnostics output per member
 
 // The set of resident lattices and the device tables of the batched launch. Every table is
@@ -284,6 +315,8 @@ public:
     int tile_x = 128, tile_y = 1, npt = 1;
     int groups = 1;  // row groups per block (kBlockNodes): a tile is (tile_x * npt) x (tile_y * groups) nodes
     bool hi1 = false;  // every active lattice has s_3 = s_4 = 1 (set by rebuild)
+    bool one_step = false;  // an explicit tile shape: one step per launch
+    int march = 0;  // > 0: pairs of steps in one launch, in segments of this many rows (set by rebuild)
     int parity = 0;  // every resident lattice holds its current data in buf[parity]
     std::vector<Lattice*> members;  // launch order
 
@@ -325,7 +358,9 @@ public:
         off_diag = align256(cap_members * msz);
         off_owner = off_diag + align256(cap_members * kDiagStride * sizeof(double));
         off_rows = off_owner + align256(cap_tiles * sizeof(int));
-        table_bytes = off_rows + align256(cap_rows * sizeof(int));
+        // a lattice's strips and segments (of kMarchRowsMin rows or more) are at most twice its tiles
+        off_march = off_rows + align256(cap_rows * sizeof(int));
+        table_bytes = off_march + (storage == CLB_F32 ? align256(2 * cap_tiles * sizeof(int)) : 0);
         cudaError_t e = cudaMalloc(&d_tables, table_bytes);
         if (e != cudaSuccess)
             return set_error(e == cudaErrorMemoryAllocation ? CLB_ENOMEM : CLB_ECUDA, "launch tables (%zu bytes): %s",
@@ -361,6 +396,31 @@ public:
         for (int g = 2; g * threads * npt <= kBlockNodes && tiles_with(g) >= kMinWaves * resident; g *= 2) groups = g;
     }
 
+    long march_warps(int rows) const
+    {
+        long t = 0;
+        for (const Lattice* L : active) t += march_geom(L->nx, L->ny, rows).warps();
+        return t;
+    }
+
+    // Rows per segment of the two-step launch, 0 for one step per launch: the rule of a single lattice
+    // (march_rows_for), over the warps of all members.
+    void choose_march()
+    {
+        march = 0;
+        if (storage != CLB_F32 || one_step) return;
+        double nodes = 0;
+        for (const Lattice* L : active) {
+            if (L->p.wall[0] == CLB_WALL_WET || L->p.wall[2] == CLB_WALL_WET) return;
+            nodes += double(L->nx) * L->ny;
+        }
+        if (nodes < kMarchBatchNodes) return;
+        int dev = 0, sms = 1;
+        cudaGetDevice(&dev);
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        march = march_rows_for([&](int rows) { return march_warps(rows); }, std::max(1, sms), kBatchStepUs + nodes * kBatchNodeUs);
+    }
+
     // Rebuild the tile and row tables for the active members (no allocation, no stream sync).
     clb_status rebuild()
     {
@@ -374,10 +434,12 @@ public:
                 hi1 = hi1 && L->p.s_3 == 1.0 && L->p.s_4 == 1.0 && L->p.lambda2 == 1.0;
             }
         choose_groups();
-        const long tiles = tiles_with(groups);
+        choose_march();
+        const long tiles = tiles_with(groups), warps = march ? march_warps(march) : 0;
         long rows = 0;
         for (const Lattice* L : active) rows += L->ny;
-        if (active.size() > cap_members || (size_t)tiles > cap_tiles || (size_t)rows > cap_rows)
+        if (active.size() > cap_members || (size_t)tiles > cap_tiles || (size_t)rows > cap_rows ||
+            (size_t)warps > 2 * cap_tiles)
             return set_error(CLB_ENOMEM, "batched launch tables: %zu members, %ld tiles, %ld rows exceed the reserved "
                                          "%zu, %zu, %zu", active.size(), tiles, rows, cap_members, cap_tiles, cap_rows);
         // the mirrors of the previous rebuild may still be in flight to the device
@@ -387,28 +449,37 @@ public:
         int* owner = (int*)((char*)h_tables + off_owner);
         int* row_owner = (int*)((char*)h_tables + off_rows);
         double* ddiag = (double*)((char*)d_tables + off_diag);
-        int t = 0, r = 0;
+        int* march_owner = (int*)((char*)h_tables + off_march);
+        int t = 0, r = 0, mw = 0;
         for (size_t k = 0; k < active.size(); ++k) {
             const Lattice& L = *active[k];
             const int tx = (L.nx + tile_x * npt - 1) / (tile_x * npt), ty = (L.ny + tile_y * groups - 1) / (tile_y * groups);
             if (storage == CLB_F64) {
-                Member<double> m = make_member<double>(L, tile_x, npt, t, r, ddiag + kDiagStride * k);
+                Member<double> m = make_member<double>(L, tile_x, npt, t, r, mw, ddiag + kDiagStride * k);
                 std::memcpy(hm + k * msz, &m, msz);
             } else {
-                Member<float> m = make_member<float>(L, tile_x, npt, t, r, ddiag + kDiagStride * k);
+                Member<float> m = make_member<float>(L, tile_x, npt, t, r, mw, ddiag + kDiagStride * k);
                 std::memcpy(hm + k * msz, &m, msz);
             }
             std::fill(owner + t, owner + t + tx * ty, int(k));
             std::fill(row_owner + r, row_owner + r + L.ny, int(k));
+            if (march) {
+                const int n = march_geom(L.nx, L.ny, march).warps();
+                std::fill(march_owner + mw, march_owner + mw + n, int(k));
+                mw += n;
+            }
             t += tx * ty;
             r += L.ny;
         }
         ntiles = t;
         nrows = r;
+        nmarch = mw;
         if (!active.empty()) {
             CLB_CUDA(cudaMemcpyAsync((char*)d_tables + off_members, hm, active.size() * msz, cudaMemcpyHostToDevice, stream));
             CLB_CUDA(cudaMemcpyAsync((char*)d_tables + off_owner, owner, (size_t)t * sizeof(int), cudaMemcpyHostToDevice, stream));
             CLB_CUDA(cudaMemcpyAsync((char*)d_tables + off_rows, row_owner, (size_t)r * sizeof(int), cudaMemcpyHostToDevice, stream));
+            if (march)
+                CLB_CUDA(cudaMemcpyAsync((char*)d_tables + off_march, march_owner, (size_t)mw * sizeof(int), cudaMemcpyHostToDevice, stream));
             CLB_CUDA(cudaEventRecord(copied, stream));
         }
         dirty = false;
@@ -438,6 +509,15 @@ public:
         return CLB_OK;
     }
 
+    // Two steps of every active member, buffers par to par ^ 1.
+    clb_status launch_two(cudaStream_t s, int par)
+    {
+        const Member<float>* m = (const Member<float>*)((char*)d_tables + off_members);
+        const int* owner = (const int*)((char*)d_tables + off_march);
+        CLB_CUDA(launch_chained(hi1 ? k_step_two_batched<true> : k_step_two_batched<false>, nmarch, 32, 0, s, m, owner, par, march));
+        return CLB_OK;
+    }
+
     clb_status step(long n)
     {
         CLB_TRY(rebuild());
@@ -447,7 +527,9 @@ public:
             if (graph[par]) continue;
             CLB_CUDA(cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal));
             clb_status st = CLB_OK;
-            for (int k = 0; k < kChunk && st == CLB_OK; ++k) st = launch_step(cap, par ^ (k & 1));
+            const int per = march ? 2 : 1;  // steps per launch; kChunk / per launches are an even number
+            for (int k = 0; k < kChunk / per && st == CLB_OK; ++k)
+                st = per == 2 ? launch_two(cap, par ^ (k & 1)) : launch_step(cap, par ^ (k & 1));
             cudaGraph_t g = nullptr;
             cudaError_t e = cudaStreamEndCapture(cap, &g);
             if (st != CLB_OK) {
@@ -463,6 +545,11 @@ public:
             CLB_CUDA(cudaGraphLaunch(graph[parity], stream));
             for (Lattice* L : active) L->steps += kChunk;
             n -= kChunk;
+        }
+        for (; march && n >= 2; n -= 2) {
+            CLB_TRY(launch_two(stream, parity));
+            parity ^= 1;
+            for (Lattice* L : active) L->steps += 2;
         }
         for (; n > 0; --n) {
             CLB_TRY(launch_step(stream, parity));
@@ -545,14 +632,14 @@ public:
         return CLB_OK;
     }
 
-    int ntiles = 0, nrows = 0;
+    int ntiles = 0, nrows = 0, nmarch = 0;
 
 private:
     bool dirty = true;
     std::vector<Lattice*> active;
     void* d_tables = nullptr;  // members | diagnostics outputs | tile owners | row owners
     void* h_tables = nullptr;  // pinned mirror of the same layout
-    size_t off_members = 0, off_diag = 0, off_owner = 0, off_rows = 0, table_bytes = 0;
+    size_t off_members = 0, off_diag = 0, off_owner = 0, off_rows = 0, off_march = 0, table_bytes = 0;
     size_t cap_members = 0, cap_tiles = 0, cap_rows = 0;
     cudaEvent_t copied = nullptr;  // recorded after the last copy of the mirrors
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
@@ -835,6 +922,7 @@ extern "C" clb_status clb_batch_set_tile(clb_batch* b, int tile_x, int tile_y, i
         b->E.tile_x = tile_x;
         b->E.tile_y = tile_y;
         b->E.npt = nodes_per_thread;
+        b->E.one_step = true;
         b->E.mark_dirty();
         return CLB_OK;
     } catch (const std::bad_alloc&) {
@@ -870,6 +958,7 @@ extern "C" clb_status clb_batch_autotune(clb_batch* b, int* tile_x, int* tile_y,
         cudaEventCreate(&e1);
         float best = 1e30f;
         int bt[3] = {E.tile_x, E.tile_y, E.npt};
+        E.one_step = true;
         clb_status st = CLB_OK;
         for (auto& sh : shapes) {
             E.tile_x = sh[0];
@@ -890,6 +979,22 @@ extern "C" clb_status clb_batch_autotune(clb_batch* b, int* tile_x, int* tile_y,
                 bt[0] = sh[0];
                 bt[1] = sh[1];
                 bt[2] = sh[2];
+            }
+        }
+        // two steps per launch, where the rule takes them (10 steps in 5 launches)
+        E.one_step = false;
+        E.mark_dirty();
+        if (st == CLB_OK) st = E.rebuild();
+        if (st == CLB_OK && E.march) {
+            for (int k = 0; k < 4 && st == CLB_OK; ++k) st = E.launch_two(E.stream, (E.parity + k) & 1);
+            cudaEventRecord(e0, E.stream);
+            for (int k = 0; k < 5 && st == CLB_OK; ++k) st = E.launch_two(E.stream, (E.parity + k) & 1);
+            cudaEventRecord(e1, E.stream);
+            if (st == CLB_OK) {
+                float ms = 0;
+                cudaEventSynchronize(e1);
+                cudaEventElapsedTime(&ms, e0, e1);
+                E.one_step = !(ms < best);
             }
         }
         cudaEventDestroy(e0);

@@ -289,18 +289,6 @@ Launch current_launch(const clb_handle* h)
     return {h->bx, h->by, h->npt, h->pipe_stages, h->pipe_rows, h->march};
 }
 
-// Strips and segments of the two-step kernel with segments of `rows` rows.
-MarchGeom march_geom(int nx, int ny, int rows)
-{
-    MarchGeom G;
-    G.strips = (nx + kMarchOut - 1) / kMarchOut;
-    G.width = ((nx + G.strips - 1) / G.strips + 1) & ~1;
-    G.strips = (nx + G.width - 1) / G.width;
-    G.rows = rows;
-    G.segs = (ny + rows - 1) / rows;
-    return G;
-}
-
 // Rows per segment of the two-step kernel, 0 where one step per launch is the faster form.
 // Longer segments repeat fewer rows of the first step, shorter ones fill the last round of resident
 // warps. With w warps per SM a warp takes 0.5 + 0.068 w us per row (fitted to 1 to 20 warps per SM),
@@ -315,19 +303,7 @@ int march_rows_rule(int nx, int ny, const clb_params& p, int sms)
 {
     const bool wet = p.wall[0] == CLB_WALL_WET || p.wall[2] == CLB_WALL_WET;
     if (p.storage != CLB_F32 || wet || (long long)nx * ny < kMarchNodes) return 0;
-    const int resident = sms * kMarchResident;
-    int best = 0;
-    double least = 1.0 + 112.0 * nx * ny / 6.7e6;
-    for (int rows = 4; rows <= 64; ++rows) {
-        const int warps = march_geom(nx, ny, rows).warps(), rest = warps % resident;
-        const double t = (rows + 1) * ((warps / resident) * (0.5 + 0.068 * kMarchResident) +
-                                       (rest ? 0.5 + 0.068 * rest / sms : 0.0));
-        if (t < least) {
-            least = t;
-            best = rows;
-        }
-    }
-    return best;
+    return march_rows_for([&](int rows) { return march_geom(nx, ny, rows).warps(); }, sms, 1.0 + 112.0 * nx * ny / 6.7e6);
 }
 
 // Enqueue two steps from buffer `from` into the other buffer on stream s.

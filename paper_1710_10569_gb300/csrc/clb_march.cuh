@@ -43,6 +43,40 @@ struct MarchGeom {
     __host__ __device__ int warps() const { return strips * segs; }
 };
 
+// Strips and segments of the two-step kernel with segments of `rows` rows.
+inline MarchGeom march_geom(int nx, int ny, int rows)
+{
+    MarchGeom G;
+    G.strips = (nx + kMarchOut - 1) / kMarchOut;
+    G.width = ((nx + G.strips - 1) / G.strips + 1) & ~1;
+    G.strips = (nx + G.width - 1) / G.width;
+    G.rows = rows;
+    G.segs = (ny + rows - 1) / rows;
+    return G;
+}
+
+// The rows per segment for which the warps (a function of it) take the least time, in us per step: a
+// round of w warps per SM takes 0.5 + 0.068 w us per row and step (fitted to 1 to 20 warps per SM), a
+// segment of R rows is R + 1 of these. 0 if none takes less than `one_step`, the time of one step per
+// launch.
+constexpr int kMarchRowsMin = 4, kMarchRowsMax = 64;
+template <typename Warps>
+inline int march_rows_for(const Warps& warps_of, int sms, double one_step)
+{
+    int best = 0;
+    double least = one_step;
+    for (int rows = kMarchRowsMin; rows <= kMarchRowsMax; ++rows) {
+        const long long warps = warps_of(rows), resident = (long long)sms * kMarchResident, rest = warps % resident;
+        const double t = (rows + 1) * ((warps / resident) * (0.5 + 0.068 * kMarchResident) +
+                                       (rest ? 0.5 + 0.068 * rest / sms : 0.0));
+        if (t < least) {
+            least = t;
+            best = rows;
+        }
+    }
+    return best;
+}
+
 // The pair of values pulled from x - 1 (shr) or x + 1 (shl): one from the neighbour lane.
 __device__ __forceinline__ F2 pull_shr(F2 v)
 {
@@ -112,62 +146,67 @@ template <bool HI1, bool WALLS>
 __device__ __forceinline__ void march_row(const LatParams<float>& P, F2 v[NPOP], const MarchWalls& w, F2 d5, F2 d6,
                                           F2 d7, F2 d8, float Tb)
 {
+    // shifts along x; next to an x wall the node's own opposite value comes in instead
+    const bool left = WALLS && (w.m0 & 1), right0 = WALLS && (w.m0 & 2), right1 = WALLS && (w.m1 & 2);
+    const auto from_left = [&](F2 x, F2 own) {
+        float a, b, o0, o1;
+        x.split(a, b);
+        own.split(o0, o1);
+        const float up = lane_up(b);
+        return F2(left ? o0 : up, a);
+    };
+    const auto from_right = [&](F2 x, F2 own) {
+        float a, b, o0, o1;
+        x.split(a, b);
+        own.split(o0, o1);
+        const float down = lane_down(a);
+        return F2(right0 ? o0 : b, right1 ? o1 : down);
+    };
     F2 f[9], g[5];
     f[0] = v[0];
     f[2] = v[2];
     f[4] = v[4];
+    f[1] = from_left(v[1], v[3]);
+    f[3] = from_right(v[3], v[1]);
+    f[5] = from_left(v[5], d7);
+    f[6] = from_right(v[6], d8);
+    f[7] = from_right(v[7], d5);
+    f[8] = from_left(v[8], d6);
     g[0] = v[9];
+    g[1] = from_left(v[10], WALLS && P.kind[0] == WALL_DIRICHLET ? F2(P.Tw_c2[0]) - v[12] : v[12]);
     g[2] = v[11];
+    g[3] = from_right(v[12], WALLS && P.kind[1] == WALL_DIRICHLET ? F2(P.Tw_c2[1]) - v[10] : v[10]);
     g[4] = v[13];
-    f[1] = pull_shr(v[1]);
-    f[3] = pull_shl(v[3]);
-    f[5] = pull_shr(v[5]);
-    f[6] = pull_shl(v[6]);
-    f[7] = pull_shl(v[7]);
-    f[8] = pull_shr(v[8]);
-    g[1] = pull_shr(v[10]);
-    g[3] = pull_shl(v[12]);
-    if (WALLS && (w.bottom || w.top || w.any_x)) {
-        // bounced values are not shifted
-        if (w.bottom) {
-            f[5] = v[5];
-            f[6] = v[6];
-        }
-        if (w.top) {
-            f[7] = v[7];
-            f[8] = v[8];
-        }
-        float a[NPOP], b[NPOP];
-#pragma unroll
-        for (int i = 0; i < NPOP; ++i) (i < 9 ? f[i] : g[i - 9]).split(a[i], b[i]);
-        if (w.any_x) {
-            float own[2];
-            const auto take = [&](int i, F2 o, int side) {
-                o.split(own[0], own[1]);
-                if (w.m0 & side) a[i] = own[0];
-                if (w.m1 & side) b[i] = own[1];
-            };
-            take(1, v[3], 1);
-            take(5, d7, 1);
-            take(8, d6, 1);
-            take(10, v[12], 1);
-            take(3, v[1], 2);
-            take(6, d8, 2);
-            take(7, d5, 2);
-            take(12, v[10], 2);
-        }
-        const int rows = (w.bottom ? 4 : 0) | (w.top ? 8 : 0);
-        float fa[9], ga[5], fb[9], gb[5];
-        finish_pull(P, a, rows | w.m0, fa, ga);
-        finish_pull(P, b, rows | w.m1, fb, gb);
-#pragma unroll
-        for (int i = 0; i < 9; ++i) f[i] = F2(fa[i], fb[i]);
-#pragma unroll
-        for (int i = 0; i < 5; ++i) g[i] = F2(ga[i], gb[i]);
+    // next to a y wall (whole rows): bounced values, not shifted; elsewhere g2 and g4 are re-based to
+    // this row (see finish_pull)
+    if (WALLS && w.bottom) {
+        f[5] = v[5];
+        f[6] = v[6];
+        if (P.kind[2] == WALL_DIRICHLET) g[2] = F2(P.Tw_c2[2]) - g[2];
     } else {
-        // re-based to this row (see finish_pull)
         g[2] = g[2] - F2(P.T_dyw);
+    }
+    if (WALLS && w.top) {
+        f[7] = v[7];
+        f[8] = v[8];
+        if (P.kind[3] == WALL_DIRICHLET) g[4] = F2(P.Tw_c2[3]) - g[4];
+    } else {
         g[4] = g[4] + F2(P.T_dyw);
+    }
+    if (WALLS && P.moving) {
+        // momentum of a moving wall; a diagonal that crosses two takes the y wall's
+        const auto add = [&](int i, bool x0, bool x1, int x_side, bool y, int y_side) {
+            const float c = y ? P.fbb[y_side][i] : P.fbb[x_side][i];
+            f[i] = f[i] + F2(x0 || y ? c : 0.0f, x1 || y ? c : 0.0f);
+        };
+        add(1, left, false, 0, false, 0);
+        add(3, right0, right1, 1, false, 0);
+        add(2, false, false, 0, w.bottom, 2);
+        add(4, false, false, 0, w.top, 3);
+        add(5, left, false, 0, w.bottom, 2);
+        add(6, right0, right1, 1, w.bottom, 2);
+        add(7, right0, right1, 1, w.top, 3);
+        add(8, left, false, 0, w.top, 3);
     }
     collide_dev<HI1>(P, f, g, F2(Tb));
 #pragma unroll
@@ -225,7 +264,7 @@ __device__ __forceinline__ void march_rows(const float* __restrict__ src, float*
                 }
             }
             F2 d5 = v[0], d6 = v[0], d7 = v[0], d8 = v[0];
-            if (WALLS && w.any_x) {
+            if (WALLS && (w.m0 | w.m1)) {
                 const auto own = [&](int i) { return F2(sc[i * kRowChunk + oa], sc[i * kRowChunk + ob]); };
                 d5 = own(5);
                 d6 = own(6);
@@ -240,7 +279,7 @@ __device__ __forceinline__ void march_rows(const float* __restrict__ src, float*
         w.bottom = WALLS && !P.per_y && q == 0;
         w.top = WALLS && !P.per_y && q == P.ny - 1;
         F2 d5 = v[0], d6 = v[0], d7 = v[0], d8 = v[0];
-        if (WALLS && w.any_x) {
+        if (WALLS && (w.m0 | w.m1)) {
             d5 = as_pair(keepU(q, 1));
             d6 = as_pair(keepU(q, 2));
             d7 = as_pair(keepD(1));

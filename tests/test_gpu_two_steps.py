@@ -67,3 +67,29 @@ def test_four_thermal_steps_per_launch_equal_one(clb, layout, shape):
         got.append(h.populations())
         h.close()
     assert np.isfinite(got[0]).all() and np.array_equal(*got)
+
+
+# Batches: pairs of steps in one launch against one step per launch (an explicit tile shape).
+@pytest.mark.parametrize("sizes", [[(512, 512), (61, 70), (333, 129), (64, 64), (2, 3), (120, 900)], [(700, 700)],
+                                   [(60, 35)] * 230, [(1025, 31)] * 15 + [(59, 300)] * 9], ids=["mixed", "one", "many", "wide"])
+@pytest.mark.parametrize("rates", [1.0, 1.2])
+def test_two_steps_per_batched_launch_equal_one(clb, sizes, rates):
+    layouts = list(LAYOUTS.values())
+    probs = [W.random_problem(nx, ny, seed=k, storage=W.STORAGE_F32, walls=layouts[k % len(layouts)], moving=rates != 1.0)
+             for k, (nx, ny) in enumerate(sizes)]
+    for p in probs:
+        p.params.update(s_3=rates, s_4=rates, lambda2=rates)
+        if min(p.nx, p.ny) < 4:
+            p.T, p.ux, p.uy = 0.01 * p.T, 0.01 * p.ux, 0.01 * p.uy
+    got = []
+    for tile in (None, (64, 2, 2)):
+        b = clb.Batch(probs)
+        if tile:
+            b.set_tile(*tile)
+        b.step(39)
+        got.append([b.fields(k) for k in range(len(probs))])
+        assert set(b.status()[2]) == {39}
+        b.close()
+    for k, (x, y) in enumerate(zip(*got)):
+        for a, b in zip(x, y):
+            assert np.isfinite(a).all() and np.array_equal(a, b), k
