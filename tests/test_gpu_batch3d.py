@@ -117,3 +117,25 @@ def test_member_cannot_be_stepped_alone(clb):
     b = clb.Batch3D(mixed3(F32)[:2])
     with pytest.raises(RuntimeError):
         b.member(0).step(1)
+
+
+@pytest.mark.parametrize("storage", [W.STORAGE_F64, W.STORAGE_F32, W.STORAGE_F16DEV])
+@pytest.mark.parametrize("shapes", [[(9, 7, 5), (33, 20, 17), (5, 4, 3)], [(96, 80, 70), (21, 9, 11), (64, 2, 40)]],
+                         ids=["small", "large"])
+def test_chained_graphs_equal_single_lattices_after_reinit(clb, storage, shapes):
+    """Graphs of one chain of launches per lattice (32 steps, or 8 for large batches), with steps left
+    over, and with one lattice initialised again while the others sit in their other buffer."""
+    probs = [W.random_problem3d(*s, seed=k, storage=storage) for k, s in enumerate(shapes)]
+    for p in probs:  # thin extents: gentle fields
+        p.ux, p.uy, p.uz, p.T = 0.2 * p.ux, 0.2 * p.uy, 0.2 * p.uz, 0.2 * p.T
+    b = clb.Batch3D(probs)
+    b.step(37)
+    b.init_fields(1, *probs[1].fields())
+    b.step(41)
+    for k, p in enumerate(probs):
+        lat = clb.Lattice3D.from_problem(p)
+        lat.step(41 if k == 1 else 78)
+        for x, y in zip(lat.populations(), b.member(k).populations()):
+            assert np.isfinite(x).all() and np.array_equal(x, y), k
+        lat.close()
+    b.close()
