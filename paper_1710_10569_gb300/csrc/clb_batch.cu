@@ -78,9 +78,8 @@ __device__ __forceinline__ void prefetch_pulls(const typename Storage<ST>::T* __
 // Register cap: the FP32 two-nodes-per-thread form (the default tile) is held at 96 registers so
 // that five 128-thread blocks stay resident per SM; the other forms take what they need (blocks
 // have at most 256 threads).
-// HI1: every lattice of the launch has s_3 = s_4 = lambda2 = 1 (the form of collide that does not
-// form the moments those rates discard).
-template <int ST, int V, bool HI1>
+// FORM: the collision form that fits every lattice of the launch (collide_form).
+template <int ST, int V, int FORM>
 __global__ void __maxnreg__((ST == ST_F32 && V == 2) ? 96 : 255) k_step_batched(const Member<typename Storage<ST>::A>* __restrict__ mem,
                                                       const int* __restrict__ owner, int parity, int groups)
 {
@@ -130,7 +129,7 @@ __global__ void __maxnreg__((ST == ST_F32 && V == 2) ? 96 : 255) k_step_batched(
             // the warp's next row to L2 first (one row ahead: 53.7 -> 55.7 GLUPS on 256 uneven
             // cavities; two rows ahead 53.4)
             if (y + (int)blockDim.y < y_end) prefetch_pulls<ST, V>(src, M.P, x0, y + blockDim.y);
-            step_warp_nodes<ST, V, true, HI1>(src, dst, M.P, x0, y, lane, keep);
+            step_warp_nodes<ST, V, true, FORM>(src, dst, M.P, x0, y, lane, keep);
         }
     }
     const int nrow = y_end - y0;
@@ -139,7 +138,7 @@ __global__ void __maxnreg__((ST == ST_F32 && V == 2) ? 96 : 255) k_step_batched(
         const int y = y0 + j % nrow, x = xs + j / nrow;
         A f[9], g[5];
         gather(src, M.P, x, y, f, g);
-        collide_any<Storage<ST>::DEV, HI1>(M.P, f, g, row_base(M.P, y));
+        collide_any<Storage<ST>::DEV, FORM>(M.P, f, g, row_base(M.P, y));
         store_node(dst, M.P, x, y, f, g);
     }
 }
@@ -163,30 +162,32 @@ __global__ void __launch_bounds__(32, kMarchResident)
                    min(M.P.ny, ya + rows), threadIdx.x, slots + threadIdx.x, 32);
 }
 
-// Blocks of k_step_batched<ST, V, HI1> resident on the whole device at once.
-template <int ST, int V, bool HI1>
-long resident_blocks_of(int threads)
+// The batched step kernel for npt nodes per thread and a collision form.
+template <int ST, int FORM>
+auto step_kernel(int npt)
+{
+    return npt == 4 ? k_step_batched<ST, 4, FORM> : npt == 2 ? k_step_batched<ST, 2, FORM> : k_step_batched<ST, 1, FORM>;
+}
+template <int ST>
+auto step_kernel(int npt, int form)
+{
+    if constexpr (ST == ST_F64)
+        if (form > 1) return form == 3 ? step_kernel<ST, 3>(npt) : step_kernel<ST, 2>(npt);
+    return form ? step_kernel<ST, 1>(npt) : step_kernel<ST, 0>(npt);
+}
+
+// Blocks of that kernel resident on the whole device at once.
+template <int ST>
+long resident_blocks(int npt, int threads, int form)
 {
     int dev = 0, sms = 1, per_sm = 1;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_step_batched<ST, V, HI1>, threads, 0) != cudaSuccess) {
+    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, step_kernel<ST>(npt, form), threads, 0) != cudaSuccess) {
         cudaGetLastError();
         per_sm = 1;
     }
     return (long)std::max(1, sms) * std::max(1, per_sm);
-}
-
-template <int ST, bool HI1>
-long resident_blocks_npt(int npt, int threads)
-{
-    return npt == 4 ? resident_blocks_of<ST, 4, HI1>(threads)
-                    : npt == 2 ? resident_blocks_of<ST, 2, HI1>(threads) : resident_blocks_of<ST, 1, HI1>(threads);
-}
-template <int ST>
-long resident_blocks_npt(int npt, int threads, bool hi1)
-{
-    return hi1 ? resident_blocks_npt<ST, true>(npt, threads) : resident_blocks_npt<ST, false>(npt, threads);
 }
 
 template <int ST>
@@ -314,7 +315,7 @@ public:
     cudaStream_t cap = nullptr;
     int tile_x = 128, tile_y = 1, npt = 1;
     int groups = 1;  // row groups per block (kBlockNodes): a tile is (tile_x * npt) x (tile_y * groups) nodes
-    bool hi1 = false;  // every active lattice has s_3 = s_4 = 1 (set by rebuild)
+    int form = 0;  // the collision form that fits every active lattice (set by rebuild)
     bool one_step = false;  // an explicit tile shape: one step per launch
     int march = 0;  // > 0: pairs of steps in one launch, in segments of this many rows (set by rebuild)
     int parity = 0;  // every resident lattice holds its current data in buf[parity]
@@ -389,9 +390,9 @@ public:
     void choose_groups()
     {
         const int threads = tile_x * tile_y;
-        const long resident = storage == CLB_F64 ? resident_blocks_npt<ST_F64>(npt, threads, hi1)
-                              : storage == CLB_F32 ? resident_blocks_npt<ST_F32>(npt, threads, hi1)
-                                                   : resident_blocks_npt<ST_F16DEV>(npt, threads, hi1);
+        const long resident = storage == CLB_F64 ? resident_blocks<ST_F64>(npt, threads, form)
+                              : storage == CLB_F32 ? resident_blocks<ST_F32>(npt, threads, form)
+                                                   : resident_blocks<ST_F16DEV>(npt, threads, form);
         groups = 1;
         for (int g = 2; g * threads * npt <= kBlockNodes && tiles_with(g) >= kMinWaves * resident; g *= 2) groups = g;
     }
@@ -427,11 +428,11 @@ public:
         if (!dirty) return CLB_OK;
         drop_graphs();
         active.clear();
-        hi1 = true;
+        form = 3;
         for (Lattice* L : members)
             if (L->active) {
                 active.push_back(L);
-                hi1 = hi1 && L->p.s_3 == 1.0 && L->p.s_4 == 1.0 && L->p.lambda2 == 1.0;
+                form = std::min(form, collide_form(L->p));
             }
         choose_groups();
         choose_march();
@@ -493,8 +494,7 @@ public:
         const dim3 block(tile_x, tile_y);
         const Member<A>* m = (const Member<A>*)((char*)d_tables + off_members);
         const int* owner = (const int*)((char*)d_tables + off_owner);
-        const auto kernel = hi1 ? (npt == 4 ? k_step_batched<ST, 4, true> : npt == 2 ? k_step_batched<ST, 2, true> : k_step_batched<ST, 1, true>)
-                                : (npt == 4 ? k_step_batched<ST, 4, false> : npt == 2 ? k_step_batched<ST, 2, false> : k_step_batched<ST, 1, false>);
+        const auto kernel = step_kernel<ST>(npt, form);
         return launch_chained(kernel, ntiles, block, 0, s, m, owner, par, groups);
     }
 
@@ -514,7 +514,7 @@ public:
     {
         const Member<float>* m = (const Member<float>*)((char*)d_tables + off_members);
         const int* owner = (const int*)((char*)d_tables + off_march);
-        CLB_CUDA(launch_chained(hi1 ? k_step_two_batched<true> : k_step_two_batched<false>, nmarch, 32, 0, s, m, owner, par, march));
+        CLB_CUDA(launch_chained(form ? k_step_two_batched<true> : k_step_two_batched<false>, nmarch, 32, 0, s, m, owner, par, march));
         return CLB_OK;
     }
 

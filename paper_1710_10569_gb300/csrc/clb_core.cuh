@@ -79,6 +79,13 @@ __device__ __forceinline__ double scale_down(double x)
     const bool keep = e == 0x7ff, tiny = e <= N;
     return __hiloint2double(keep ? hi : tiny ? hi & (int)0x80000000 : hi - (N << 20), !keep && tiny ? 0 : __double2loint(x));
 }
+// 2 x by its exponent (zero and subnormal numbers, which lack the hidden bit, by an addition).
+__device__ __forceinline__ double scale_up1(double x)
+{
+    const int hi = __double2hiint(x);
+    const unsigned e = (unsigned)hi >> 20 & 0x7ff;
+    return e == 0 ? __hiloint2double(hi & (int)0x80000000, 0) : e >= 0x7fe ? x : __hiloint2double(hi + (1 << 20), __double2loint(x));
+}
 // 1 / x from the hardware's approximation r (relative error e below 2^-19) by one step of Halley's
 // third-order iteration, r + r (e + e^2) with e = 1 - x r: three FMAs in place of the six of the
 // correctly rounded reciprocal, and within one unit of the last place of it.
@@ -168,7 +175,11 @@ template <> struct CollideConsts<double> {
     double c3, hFc3;                  // (2 - s_3) / 3, and Fv_x / 2 times it (third-order forcing)
     double hsp, hsm, om11;            // sp / 2, sm / 2, 1 - s_nu
     double om3, qom3, s36, qom4;      // 1 - s_3 and its quarter, s_4 / 36, (1 - s_4) / 4
-    double hom1, hom2, heq;           // (1 - lambda1) / 2, (1 - lambda2) / 2, lambda2 cs2_T / 2
+    double hom1, hl1, hl1h;           // (1 - lambda1) / 2, lambda1 / 2, lambda1 - 1 / 2
+    double hom2, heq;                 // (1 - lambda2) / 2, lambda2 cs2_T / 2
+    // wet walls, per side with inward normal n: half the force along the normal and along the wall at
+    // T_w, the wall's velocity along both, 1 / (1 - n u_n), and g^eq(T_w, u_w)
+    double wFn[4], wFt[4], wun[4], wut[4], winv[4], wg[4][5];
 };
 
 // First statement of every kernel launched with launch_chained: wait until the kernel before it on
@@ -273,9 +284,12 @@ __device__ __forceinline__ void finish_pull(const LatParams<A>& P, const T raw[N
     for (int i = 0; i < 9; ++i) f[i] = to_a(raw[i]);
 #pragma unroll
     for (int i = 0; i < 5; ++i) g[i] = to_a(raw[9 + i]);
-    // g2 (g4) pulled from the row below (above) is re-based to this row; bounced values are not
-    g[2] = (wall_mask & 4) ? g[2] : g[2] - P.T_dyw;
-    g[4] = (wall_mask & 8) ? g[4] : g[4] + P.T_dyw;
+    // g2 (g4) pulled from the row below (above) is re-based to this row; bounced values are not (FP64
+    // populations have no base)
+    if constexpr (sizeof(A) < sizeof(double)) {
+        g[2] = (wall_mask & 4) ? g[2] : g[2] - P.T_dyw;
+        g[4] = (wall_mask & 8) ? g[4] : g[4] + P.T_dyw;
+    }
     if (wall_mask) {
         if ((wall_mask & 1) && P.kind[0] == WALL_DIRICHLET) g[1] = P.Tw_c2[0] - g[1];
         if ((wall_mask & 2) && P.kind[1] == WALL_DIRICHLET) g[3] = P.Tw_c2[1] - g[3];
@@ -441,18 +455,19 @@ __device__ __forceinline__ void central_d2q9(const A f[9], A ux, A uy, A k[3][3]
 }
 
 // D2Q5 collision in populations form (Eqs. 16-21) for temperature T and velocity u, given the axis
-// sums s and differences d of g. The back transform takes the halves of the raw moments,
-// r1/2 = k1/2 + (u/2) T and r2/2 = k2/2 + u (k1/2 + r1/2). HI1: lambda2 = 1, so the second-order
+// sums s and differences d of g. The back transform takes the halves of the raw moments: with k1 =
+// (1 - lambda1)(d - u T), r1/2 = k1/2 + (u/2) T and r2/2 = k2/2 + u (k1/2 + r1/2), whose inner sum is
+// (1 - lambda1) d + (lambda1 - 1/2) u T. HI1: lambda2 = 1, so the second-order
 // central moments relax to equilibrium whatever their value (not formed).
 template <bool HI1 = false>
-__device__ __forceinline__ void collide_d2q5(const LatParams<double>& P, double T, double ux, double uy, double hux,
-                                             double huy, double s1, double d1, double s2, double d2, double g[5])
+__device__ __forceinline__ void collide_d2q5(const LatParams<double>& P, double T, double ux, double uy, double s1,
+                                             double d1, double s2, double d2, double g[5])
 {
-    const double uT = hux * T, vT = huy * T;
-    const double k1 = P.hom1 * fma_(-ux, T, d1), k2 = P.hom1 * fma_(-uy, T, d2);
-    const double r1 = k1 + uT, r2 = k2 + vT;
+    const double uT = ux * T, vT = uy * T;
+    const double t1 = P.hom1 * d1, t2 = P.hom1 * d2;
+    const double r1 = fma_(P.hl1, uT, t1), r2 = fma_(P.hl1, vT, t2);
     const double eq = P.heq * T;
-    double h1 = fma_(ux, k1 + r1, eq), h2 = fma_(uy, k2 + r2, eq);
+    double h1 = fma_(ux, fma_(P.hl1h, uT, scale_up1(t1)), eq), h2 = fma_(uy, fma_(P.hl1h, vT, scale_up1(t2)), eq);
     if constexpr (!HI1) {
         h1 = fma_(P.hom2, fma_(ux * ux, T, fma_(-2.0 * ux, d1, s1)), h1);
         h2 = fma_(P.hom2, fma_(uy * uy, T, fma_(-2.0 * uy, d2, s2)), h2);
@@ -466,18 +481,19 @@ __device__ __forceinline__ void collide_d2q5(const LatParams<double>& P, double 
 
 // Collision of one node in place, populations form (FP64 storage): Eqs. (6)-(11) for f, Eqs. (16)-(21)
 // for g. FP64 instructions bound it (GB300 issues two per clock and SM), so it is written for the
-// fewest of them: 104 with HI1, 421 us per step on 2048 x 1024 (the transforms pass by pass took
-// 139.8, 544 us). The relaxed central moments go straight to raw moments about 0, in the halves (second
+// fewest of them: 103 in form 1, 94 in form 2 (363.8 us per step on 2048 x 1024), 87 in form 3; the
+// transforms pass by pass took 139.8 (544 us). The relaxed central moments go straight to raw moments about 0, in the halves (second
 // order, and the momentum) and quarters (order 3 and 4, and xy) that the back transform takes;
 // rho u = j + F/2 makes the first-order central moments -F/2, so they are not formed:
 //   k20 = m20 - u (j - F/2), r20 = m20 + 2 u F - (relaxation), k11 = m11 - u_x j_y + u_y F_x / 2,
 //   r21 = R21 + u_y r20 with R21 = k21* + 2 u_x k11* + u_x^2 k01*, and r12 alike with the axes swapped,
 //   r22 = R22 + u_y (2 R21 + u_y r20) with R22 = k22* + 2 u_x k12* + u_x^2 k02*.
-// HI1: the high-order rates are 1 (s_3 = s_4 = lambda2 = 1, the paper's setting, Sec. 3), so k~21,
-// k~12, k~22 and the second-order D2Q5 moments relax to their equilibrium and forcing terms
-// whatever their value; they are then not formed. The results are the same as with HI1 = false:
-// (1 - s) k is an exact zero for s = 1.
-template <bool HI1 = false>
+// FORM: 0 for any parameters; 1 (and above) for high-order rates of 1 (s_3 = s_4 = lambda2 = 1, the
+// paper's setting, Sec. 3), where k~21, k~12, k~22 and the second-order D2Q5 moments relax to their
+// equilibrium and forcing terms whatever their value and are not formed; 2 also without a body force
+// along x and with T0 = 0 (buoyant convection), 3 without any force (no buoyancy either). The results
+// are the same in every form that fits: what is left out is an exact zero, or adds one.
+template <int FORM = 0>
 __device__ __forceinline__ void collide(const LatParams<double>& P, double f[9], double g[5])
 {
     const double s0 = f[1] + f[3], d0 = f[1] - f[3];
@@ -491,9 +507,11 @@ __device__ __forceinline__ void collide(const LatParams<double>& P, double f[9],
     const double jx = (d0 + dp) + dm, jy = ((f[2] - f[4]) + sp) - sm;
     const double s1 = g[1] + g[3], d1 = g[1] - g[3], s2 = g[2] + g[4], d2 = g[2] - g[4];
     const double T = g[0] + (s1 + s2);
-    const double hFx = P.hFx, hFy = fma_(P.hgb, T - P.T0, P.hFvy);
+    constexpr bool HI1 = FORM != 0, FX = FORM < 2, FY = FORM < 3;
+    const double hFx = FX ? P.hFx : 0.0;
+    const double hFy = FX ? fma_(P.hgb, T - P.T0, P.hFvy) : FY ? fma_(P.hgb, T, P.hFvy) : 0.0;
     const double inv = rcp_halley(rho);
-    const double qx = jx + hFx, qy = jy + hFy;  // rho u (Eq. 13)
+    const double qx = FX ? jx + hFx : jx, qy = FY ? jy + hFy : jy;  // rho u (Eq. 13)
     const double ux = qx * inv, uy = qy * inv;
     const double hux = scale_down<1>(ux), huy = scale_down<1>(uy);
     double k21 = 0.0, k12 = 0.0, k22 = 0.0;
@@ -506,17 +524,17 @@ __device__ __forceinline__ void collide(const LatParams<double>& P, double f[9],
     }
 
     // relaxation, Eq. (8), equilibrium Eq. (9), forcing Eq. (11)
-    const double k20 = fma_(-ux, jx - hFx, m20), k02 = fma_(-uy, jy - hFy, m02);
+    const double k20 = fma_(-ux, FX ? jx - hFx : jx, m20), k02 = fma_(-uy, FY ? jy - hFy : jy, m02);
     const double a20 = fma_(-1.0 / 3.0, rho, k20), a02 = fma_(-1.0 / 3.0, rho, k02);
-    const double h20 = fma_(-P.hsm, a02, fma_(-P.hsp, a20, fma_(ux, P.Fvx, scale_down<1>(m20))));
+    const double h20 = fma_(-P.hsm, a02, fma_(-P.hsp, a20, FX ? fma_(ux, P.Fvx, scale_down<1>(m20)) : scale_down<1>(m20)));
     const double q02 = fma_(-P.sm, a20, fma_(-P.sp, a02, k02));
-    const double h02 = fma_(huy, fma_(2.0, hFy, qy), scale_down<1>(q02));
-    const double h10 = fma_(0.5, jx, hFx), h01 = fma_(0.5, jy, hFy);
-    const double q11 = P.om11 * fma_(-ux, jy, fma_(uy, hFx, m11));
-    const double M11 = fma_(hux, h01, fma_(huy, P.qFx, scale_down<2>(q11)));
-    double R21 = fma_(hux, q11, scale_down<2>(hFy) * fma_(ux, ux, P.c3));
-    double R12 = fma_(huy, q11, P.eFx * fma_(uy, uy, P.c3));
-    double in = fma_(hux, q02, P.hFc3);
+    const double h02 = fma_(huy, FY ? fma_(2.0, hFy, qy) : qy, scale_down<1>(q02));
+    const double h10 = FX ? fma_(0.5, jx, hFx) : scale_down<1>(jx), h01 = FY ? fma_(0.5, jy, hFy) : scale_down<1>(jy);
+    const double q11 = P.om11 * fma_(-ux, jy, FX ? fma_(uy, hFx, m11) : m11);
+    const double M11 = fma_(hux, h01, FX ? fma_(huy, P.qFx, scale_down<2>(q11)) : scale_down<2>(q11));
+    double R21 = FY ? fma_(hux, q11, scale_down<2>(hFy) * fma_(ux, ux, P.c3)) : hux * q11;
+    double R12 = FX ? fma_(huy, q11, P.eFx * fma_(uy, uy, P.c3)) : huy * q11;
+    double in = FX ? fma_(hux, q02, P.hFc3) : hux * q02;
     double e22 = P.s36 * rho;
     if constexpr (!HI1) {
         R21 = fma_(P.qom3, k21, R21);
@@ -541,7 +559,7 @@ __device__ __forceinline__ void collide(const LatParams<double>& P, double f[9],
     f[7] = q - t;
     f[8] = q + t;
 
-    collide_d2q5<HI1>(P, T, ux, uy, hux, huy, s1, d1, s2, d2, g);
+    collide_d2q5<FORM != 0>(P, T, ux, uy, s1, d1, s2, d2, g);
 }
 
 // Deviation of the D2Q9 equilibrium from the rest state, f^eq_i(rho, u) - w_i rho_b, written as
@@ -684,11 +702,11 @@ __device__ __forceinline__ void collide_dev(const LatParams<S>& P, A f[9], A g[5
     collide_d2q5_dev<HI1>(P, T, dT, ux, uy, g);
 }
 
-template <bool DEV, bool HI1 = false, typename A>
+template <bool DEV, int FORM = 0, typename A>
 __device__ __forceinline__ void collide_any(const LatParams<A>& P, A f[9], A g[5], A Tb)
 {
-    if constexpr (DEV) collide_dev<HI1>(P, f, g, Tb);
-    else collide<HI1>(P, f, g);  // FP64 populations: no base
+    if constexpr (DEV) collide_dev<FORM != 0>(P, f, g, Tb);
+    else collide<FORM>(P, f, g);  // FP64 populations: no base
 }
 
 // Equilibria in stored form, minus the rest state for deviation storage: f^eq(rho, u) (Eq. 9
@@ -816,14 +834,72 @@ __device__ __forceinline__ void gather_wet(const T* __restrict__ src, const LatP
     for (int i = 0; i < 5; ++i) g[i] = geqb[i] + (gq[i] - geqq[i]);
 }
 
+// gather_wet for FP64 populations on one wet wall (not in a corner), written for few FP64 instructions
+// (75 instead of some 200: 60 x 31 nodes, whose steps wait for the wall rows, 11.5 -> 7.4 us per step).
+// The populations that would come from beyond the wall: U0 along the normal, U1 and U2 on the diagonals
+// that lead along the wall's + and - direction; O their opposites. With s = n u'_n and A = 1/3 + u'_t^2 the
+// differences of the equilibria are rho s (1 - A) for U0 and rho (A s +- B u'_t) / 2 on the diagonals,
+// whose second term the closure of the tangential momentum rho u'_t replaces.
+__device__ __forceinline__ void gather_wet_f64(const double* __restrict__ src, const LatParams<double>& P, int x, int y,
+                                               bool onx, double f[9], double g[5])
+{
+    const bool low = onx ? x == 0 : y == 0;
+    const int side = (onx ? 0 : 2) + (low ? 0 : 1);
+    double fq[9], gq[5];
+    gather_pull(src, P, x, y, f, g);
+    gather_pull(src, P, onx ? (low ? 1 : x - 1) : x, onx ? y : (low ? 1 : y - 1), fq, gq);
+
+    const double tp = onx ? f[2] : f[1], tm = onx ? f[4] : f[3];
+    const double O0 = onx ? (low ? f[3] : f[1]) : (low ? f[4] : f[2]);
+    const double O1 = onx ? (low ? f[7] : f[8]) : (low ? f[7] : f[6]);
+    const double O2 = onx ? (low ? f[6] : f[5]) : (low ? f[8] : f[5]);
+    const double num = fma_(2.0, (O0 + O1) + O2, (f[0] + tp) + tm);
+    const double rho = (low ? num - P.wFn[side] : num + P.wFn[side]) * P.winv[side];
+    const double inv = rcp_halley(rho);
+    const double un = fma_(-P.wFn[side], inv, P.wun[side]), ut = fma_(-P.wFt[side], inv, P.wut[side]);
+    const double rs = rho * (low ? un : -un), ru = rho * ut;
+    const double hAs = scale_down<1>(rs) * fma_(ut, ut, 1.0 / 3.0);
+    const double hv = scale_down<1>(ru - (tp - tm));
+    const double U0 = O0 + fma_(-2.0, hAs, rs), U1 = (O1 + hAs) + hv, U2 = (O2 + hAs) - hv;
+    if (onx) {
+        if (low) f[1] = U0, f[5] = U1, f[8] = U2;
+        else f[3] = U0, f[6] = U1, f[7] = U2;
+    } else {
+        if (low) f[2] = U0, f[5] = U1, f[6] = U2;
+        else f[4] = U0, f[8] = U1, f[7] = U2;
+    }
+
+    // g: the wall's equilibrium plus the fluid node's non-equilibrium part
+    const double sp = fq[5] + fq[6], sm = fq[8] + fq[7];
+    const double rhoq = ((fq[0] + (fq[1] + fq[3])) + (fq[2] + sp)) + (fq[4] + sm);
+    const double jx = ((fq[1] - fq[3]) + (fq[5] - fq[6])) + (fq[8] - fq[7]), jy = ((fq[2] - fq[4]) + sp) - sm;
+    const double T = (gq[0] + (gq[1] + gq[3])) + (gq[2] + gq[4]);
+    const double invq = rcp_halley(rhoq);
+    const double ux = (jx + P.hFx) * invq, uy = (jy + fma_(P.hgb, T - P.T0, P.hFvy)) * invq;
+    const double hT = scale_down<1>(T);
+    const double x2 = hT * fma_(ux, ux, P.cs2T), x1 = hT * ux, y2 = hT * fma_(uy, uy, P.cs2T), y1 = hT * uy;
+    const double* wg = P.wg[side];
+    g[0] = wg[0] + (gq[0] - fma_(-2.0, y2, fma_(-2.0, x2, T)));
+    g[1] = wg[1] + (gq[1] - (x2 + x1));
+    g[3] = wg[3] + (gq[3] - (x2 - x1));
+    g[2] = wg[2] + (gq[2] - (y2 + y1));
+    g[4] = wg[4] + (gq[4] - (y2 - y1));
+}
+
 // Pre-collision populations of node (x, y) at the current time, wall rules included.
 template <typename T, typename A>
 __device__ __forceinline__ void gather(const T* __restrict__ src, const LatParams<A>& P, int x, int y,
                                        A f[9], A g[5])
 {
     constexpr bool DEV = sizeof(T) < sizeof(double);
-    if ((P.wet_y && (y == 0 || y == P.ny - 1)) || (P.wet_x && (x == 0 || x == P.nx - 1)))
-        gather_wet<DEV>(src, P, x, y, f, g);
+    const bool onx = P.wet_x && (x == 0 || x == P.nx - 1), ony = P.wet_y && (y == 0 || y == P.ny - 1);
+    if constexpr (!DEV) {
+        if (onx != ony) {
+            gather_wet_f64(src, P, x, y, onx, f, g);
+            return;
+        }
+    }
+    if (onx || ony) gather_wet<DEV>(src, P, x, y, f, g);
     else gather_pull(src, P, x, y, f, g);
 }
 

@@ -219,10 +219,34 @@ LatParams<A> make_lat_params(int nx, int ny, const clb_params& p)
         P.s36 = p.s_4 * (1.0 / 36.0);
         P.qom4 = 0.25 * (1.0 - p.s_4);
         P.hom1 = 0.5 * (1.0 - P.lambda1);
+        P.hl1 = 0.5 * P.lambda1;
+        P.hl1h = P.lambda1 - 0.5;
         P.hom2 = 0.5 * (1.0 - p.lambda2);
         P.heq = 0.5 * p.lambda2 * p.cs2_T;
+        for (int s = 0; s < 4; ++s) {
+            const double u = p.u_wall[s][0], v = p.u_wall[s][1], T = p.T_wall[s], n = s % 2 ? -1.0 : 1.0;
+            const double hFy = P.hFvy + P.hgb * (T - p.T0), c = p.cs2_T;
+            P.wFn[s] = s < 2 ? P.hFx : hFy;
+            P.wFt[s] = s < 2 ? hFy : P.hFx;
+            P.wun[s] = s < 2 ? u : v;
+            P.wut[s] = s < 2 ? v : u;
+            P.winv[s] = 1.0 / (1.0 - n * P.wun[s]);
+            const double g[5] = {T - T * (c + u * u) - T * (c + v * v), 0.5 * (T * (c + u * u) + u * T),
+                                 0.5 * (T * (c + v * v) + v * T), 0.5 * (T * (c + u * u) - u * T),
+                                 0.5 * (T * (c + v * v) - v * T)};
+            for (int i = 0; i < 5; ++i) P.wg[s][i] = g[i];
+        }
     }
     return P;
+}
+
+// The form of the collision kernels that fits a lattice's parameters (see collide): 0 in general, 1 for
+// high-order rates of 1; FP64 also 2 without a force along x and with T0 = 0, 3 without any force.
+inline int collide_form(const clb_params& p)
+{
+    if (p.s_3 != 1.0 || p.s_4 != 1.0 || p.lambda2 != 1.0) return 0;
+    if (p.storage != CLB_F64 || p.Fv[0] != 0.0 || p.T0 != 0.0) return 1;
+    return p.g_beta == 0.0 && p.Fv[1] == 0.0 ? 3 : 2;
 }
 
 // Nusselt geometry of Eq. (29) for one axis: H, dT and the sign making heat flow from the hot

@@ -33,7 +33,7 @@ __device__ __forceinline__ E lane_down(E v) { return __shfl_down_sync(0xffffffff
 //
 // warp_vector is the vector body. WALLS = false is the interior of the lattice (no wall next to any node of the
 // warp), where every wall term folds away at compile time.
-template <int ST, int V, bool WALLS, bool HI1 = false>
+template <int ST, int V, bool WALLS, int FORM = 0>
 __device__ __forceinline__ void warp_vector(const typename Storage<ST>::T* __restrict__ src,
                                             typename Storage<ST>::T* __restrict__ dst,
                                             const LatParams<typename Storage<ST>::A>& P, int x0, int y,
@@ -120,7 +120,7 @@ __device__ __forceinline__ void warp_vector(const typename Storage<ST>::T* __res
                 for (int i = 0; i < 9; ++i) f[i] = F2(fa[i], fb[i]);
 #pragma unroll
                 for (int i = 0; i < 5; ++i) g[i] = F2(ga[i], gb[i]);
-                collide_dev<HI1>(P, f, g, F2(Tb));
+                collide_dev<FORM != 0>(P, f, g, F2(Tb));
 #pragma unroll
                 for (int i = 0; i < NPOP; ++i) from_a2(i < 9 ? f[i] : g[i - 9], out[i].e[k], out[i].e[k + 1]);
             }
@@ -129,7 +129,7 @@ __device__ __forceinline__ void warp_vector(const typename Storage<ST>::T* __res
             for (int k = 0; k < V; ++k) {
                 A f[9], g[5];
                 finish_pull(P, raw[k], mask[k], f, g);
-                collide_any<Storage<ST>::DEV, HI1>(P, f, g, Tb);
+                collide_any<Storage<ST>::DEV, FORM>(P, f, g, Tb);
 #pragma unroll
                 for (int i = 0; i < 9; ++i) out[i].e[k] = from_a(f[i], (E*)nullptr);
 #pragma unroll
@@ -148,7 +148,7 @@ __device__ __forceinline__ void warp_vector(const typename Storage<ST>::T* __res
 // the wall terms, and interior warps take the lean copy (fewer instructions; the FP16 form is
 // issue-limited). Nodes x < keep are computed but not stored (they belong to another warp: see the
 // shifted last tile of a row in the batched kernel).
-template <int ST, int V, bool SPLIT = true, bool HI1 = false>
+template <int ST, int V, bool SPLIT = true, int FORM = 0>
 __device__ __forceinline__ void step_warp_nodes(const typename Storage<ST>::T* __restrict__ src,
                                                 typename Storage<ST>::T* __restrict__ dst,
                                                 const LatParams<typename Storage<ST>::A>& P, int x0,
@@ -160,8 +160,8 @@ __device__ __forceinline__ void step_warp_nodes(const typename Storage<ST>::T* _
     if (wx1 < P.nx && !(P.wet_y && (y == 0 || y == P.ny - 1)) && !(P.wet_x && (wx0 == 0 || wx1 == P.nx - 1))) {
         const bool walls =
             (!P.per_y && (y == 0 || y == P.ny - 1)) || (!P.per_x && (wx0 == 0 || wx1 == P.nx - 1));
-        if (!SPLIT || walls) warp_vector<ST, V, true, HI1>(src, dst, P, x0, y, lane, keep);
-        else warp_vector<ST, V, false, HI1>(src, dst, P, x0, y, lane, keep);
+        if (!SPLIT || walls) warp_vector<ST, V, true, FORM>(src, dst, P, x0, y, lane, keep);
+        else warp_vector<ST, V, false, FORM>(src, dst, P, x0, y, lane, keep);
     } else {
 #pragma unroll
         for (int k = 0; k < V; ++k) {
@@ -169,7 +169,7 @@ __device__ __forceinline__ void step_warp_nodes(const typename Storage<ST>::T* _
             if (x < P.nx && x >= keep) {
                 A f[9], g[5];
                 gather(src, P, x, y, f, g);
-                collide_any<Storage<ST>::DEV, HI1>(P, f, g, row_base(P, y));
+                collide_any<Storage<ST>::DEV, FORM>(P, f, g, row_base(P, y));
                 store_node(dst, P, x, y, f, g);
             }
         }
@@ -179,9 +179,8 @@ __device__ __forceinline__ void step_warp_nodes(const typename Storage<ST>::T* _
 // One time step over the lattice: thread (tx, ty) of block (bx, by) updates nodes
 // x0 = (bx * blockDim.x + tx) * V .. x0 + V - 1 of row by * blockDim.y + ty. blockDim.x is a
 // multiple of 32, so each warp lies in one row.
-// HI1: the form for high-order rates of 1 (see collide), which the host picks when
-// s_3 = s_4 = lambda2 = 1.
-template <int ST, int V, bool HI1>
+// FORM: the collision form that fits the lattice's parameters (collide_form).
+template <int ST, int V, int FORM>
 __global__ void __launch_bounds__(256) k_step(const typename Storage<ST>::T* __restrict__ src,
                                               typename Storage<ST>::T* __restrict__ dst,
                                               const LatParams<typename Storage<ST>::A> P)
@@ -191,7 +190,7 @@ __global__ void __launch_bounds__(256) k_step(const typename Storage<ST>::T* __r
     const int x0 = (blockIdx.x * blockDim.x + threadIdx.x) * V;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     if (y >= P.ny || x0 - lane * V >= P.nx) return;  // whole warps only
-    step_warp_nodes<ST, V, true, HI1>(src, dst, P, x0, y, lane);
+    step_warp_nodes<ST, V, true, FORM>(src, dst, P, x0, y, lane);
 }
 
 // Split step. The warps of the interior of the lattice (32 V nodes inside the row, no wall next to
@@ -213,7 +212,7 @@ struct SplitGeom {
 
 // Interior warps: thread (tx, ty) of block (bx, by) is lane tx % 32 of warp column
 // c0 + (bx blockDim.x + tx) / 32 in row y0 + by blockDim.y + ty.
-template <int ST, int V, bool HI1>
+template <int ST, int V, int FORM>
 __global__ void __launch_bounds__(256) k_step_inner(const typename Storage<ST>::T* __restrict__ src,
                                                     typename Storage<ST>::T* __restrict__ dst,
                                                     const LatParams<typename Storage<ST>::A> P, int y0, int y1,
@@ -223,7 +222,7 @@ __global__ void __launch_bounds__(256) k_step_inner(const typename Storage<ST>::
     const int c = c0 + (int)((blockIdx.x * blockDim.x + threadIdx.x) >> 5);
     const int y = y0 + blockIdx.y * blockDim.y + threadIdx.y;
     if (y >= y1 || c >= c1) return;  // whole warps only
-    warp_vector<ST, V, false, HI1>(src, dst, P, c * 32 * V + lane * V, y, lane, 0);
+    warp_vector<ST, V, false, FORM>(src, dst, P, c * 32 * V + lane * V, y, lane, 0);
 }
 
 // The FP16 form with 4 nodes per thread (its default) and high-order rates of 1, held at 96
@@ -240,7 +239,7 @@ static __global__ void __maxnreg__(96) k_step_inner_f16x4_hi1(const __half* __re
 
 // Edge warps, one per 32 threads: the wall rows first (every column), then the edge columns of the
 // interior rows.
-template <int ST, int V, bool HI1>
+template <int ST, int V, int FORM>
 __global__ void __launch_bounds__(128) k_step_edge(const typename Storage<ST>::T* __restrict__ src,
                                                    typename Storage<ST>::T* __restrict__ dst,
                                                    const LatParams<typename Storage<ST>::A> P, const SplitGeom G)
@@ -258,7 +257,7 @@ __global__ void __launch_bounds__(128) k_step_edge(const typename Storage<ST>::T
         y = G.y0 + v / G.ncb;
         c = G.cb[v % G.ncb];
     }
-    step_warp_nodes<ST, V, true, HI1>(src, dst, P, c * 32 * V + lane * V, y, lane);
+    step_warp_nodes<ST, V, true, FORM>(src, dst, P, c * 32 * V + lane * V, y, lane);
 }
 
 // ---------------------------------------------------------------------------------------------

@@ -229,11 +229,14 @@ cudaError_t enqueue_step(const clb_handle* h, const void* a, void* b, cudaStream
     using E = typename Storage<ST>::T;
     using A = typename Storage<ST>::A;
     const LatParams<A>& P = *reinterpret_cast<const LatParams<A>*>(ST == ST_F64 ? (const void*)&h->Pd : (const void*)&h->Pf);
-    const bool hi1 = h->p.s_3 == 1.0 && h->p.s_4 == 1.0 && h->p.lambda2 == 1.0;
+    const int form = collide_form(h->p);
+    const bool hi1 = form > 0;
     const dim3 block(bx, by);
     if (!split_step<ST>(h)) {
         const dim3 grid((h->nx + bx * NPT - 1) / (bx * NPT), (h->ny + by - 1) / by);
-        return launch_chained(hi1 ? k_step<ST, NPT, true> : k_step<ST, NPT, false>, grid, block, 0, s, (const E*)a, (E*)b, P);
+        auto kernel = hi1 ? k_step<ST, NPT, 1> : k_step<ST, NPT, 0>;
+        if constexpr (ST == ST_F64) kernel = form == 3 ? k_step<ST, NPT, 3> : form == 2 ? k_step<ST, NPT, 2> : kernel;
+        return launch_chained(kernel, grid, block, 0, s, (const E*)a, (E*)b, P);
     }
     if constexpr (ST == ST_F16DEV) {
         const SplitGeom G = split_geom(h->nx, h->ny, h->Pf, NPT);
@@ -427,18 +430,30 @@ clb_status take_snapshot(clb_handle* h)
 
 // Launch shape of a lattice that has not been tuned. FP64: an instruction takes its SM quarter's pipe
 // for 64 clocks however many of a warp's lanes are active, so nodes go to as many warps as they fill,
-// one per thread (64 x 64: 5.1 us per step against 17.4 with four; 2048 x 1024: 421 against 424). FP32
+// one per thread (64 x 64: 4.7 us per step, 7.8 with two, 17.4 with four); two where the busiest quarter
+// steps no more nodes with them (256 x 256: 14.4 us against 15.2; 2048 x 1024: 371.7 against 378.5). FP32
 // and FP16: two and four nodes per thread, the packed instructions' and the widest loads' count, where
 // the lattice fills the chip with them; below, more and shorter warps (128 x 128, FP16: 1.9 us against
 // 3.4). Blocks of few warps, so that a ragged row end idles few of them (513 x 385, FP32: 4.3 us at
 // 128 x 1, 3.7 at 32 x 2; 640 x 640, FP16: 6.5 and 5.7).
-void default_shape(int storage, long long nodes, int* bx, int* by, int* npt)
+void default_shape(int storage, int nx, int ny, int sms, int* bx, int* by, int* npt)
 {
+    const long long nodes = (long long)nx * ny;
     const bool small = nodes < 32768;
     *bx = 32;
     *by = 2;
-    *npt = storage == CLB_F64 || small ? 1 : 2;
-    if (storage != CLB_F64 && small) *by = 4;
+    if (storage == CLB_F64) {
+        // nodes that the busiest SM quarter steps one after another, with one and with two per thread
+        const auto serial = [&](int v) {
+            const long long warps = (long long)((nx + 32 * v - 1) / (32 * v)) * ny;
+            return v * ((warps + 4 * sms - 1) / (4 * sms));
+        };
+        *npt = serial(1) >= 4 && serial(2) <= serial(1) ? 2 : 1;
+        if (*npt == 2) *by = 1;
+        return;
+    }
+    *npt = small ? 1 : 2;
+    if (small) *by = 4;
     if (storage == CLB_F16DEV && nodes >= kSplitNodes) *npt = 4;
 }
 
@@ -505,7 +520,9 @@ extern "C" clb_status clb_create(int nx, int ny, const clb_params* p, void* stre
         h->diag = (double*)(h->mem + L.diag);
         h->Pd = make_lat_params<double>(nx, ny, *p);
         h->Pf = make_lat_params<float>(nx, ny, *p);
-        default_shape(p->storage, (long long)nx * ny, &h->bx, &h->by, &h->npt);
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+        default_shape(p->storage, nx, ny, std::max(1, sms), &h->bx, &h->by, &h->npt);
         bool tuned = false;
         {
             std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -521,8 +538,6 @@ extern "C" clb_status clb_create(int nx, int ny, const clb_params* p, void* stre
             }
         }
         if (!tuned) {
-            int sms = 0;
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
             h->march = march_rows_rule(nx, ny, *p, std::max(1, sms));
         }
         // the padding of each row's last chunk is never read, but keep it defined

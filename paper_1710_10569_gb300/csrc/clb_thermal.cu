@@ -118,7 +118,7 @@ __device__ __forceinline__ void thermal_collide(const LatParams<typename Storage
         collide_d2q5_dev(P, Tb + dT, dT, u, v, g);
     } else {
         const double s1 = g[1] + g[3], d1 = g[1] - g[3], s2 = g[2] + g[4], d2 = g[2] - g[4];
-        collide_d2q5(P, g[0] + (s1 + s2), u, v, scale_down<1>(u), scale_down<1>(v), s1, d1, s2, d2, g);
+        collide_d2q5(P, g[0] + (s1 + s2), u, v, s1, d1, s2, d2, g);
     }
 }
 
