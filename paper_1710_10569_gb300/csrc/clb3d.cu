@@ -1418,7 +1418,8 @@ extern "C" clb_status clb3d_buffers(clb3d_lattice* h, void** current, long long*
 // over their concatenated tiles, replayed from CUDA graphs of kChunk steps.
 
 // Chains of the graphs of a batch at most, and the steps per graph of batches of many nodes.
-constexpr int kMaxChains = 32, kShortChunk = 8;
+constexpr size_t kMaxChains = 32;
+constexpr int kShortChunk = 8;
 
 struct clb3d_batch {
     int storage = CLB_F64;
@@ -1435,9 +1436,6 @@ struct clb3d_batch {
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     bool chains = true;          // graphs hold chains of single-lattice launches (until a tile shape is set)
     int chunk = kChunk;          // steps per graph
-    std::vector<cudaStream_t> side;  // the chains' streams (capture only), forked from cap and joined to it
-    std::vector<cudaEvent_t> join;
-    cudaEvent_t fork = nullptr;
 };
 
 namespace {
@@ -1553,59 +1551,59 @@ clb_status batch3_launch(clb3d_batch* b, int par, cudaStream_t s)
     return CLB_OK;
 }
 
-// b->chunk steps of every lattice, captured on b->cap and the side streams that fork from it. The
-// lattices of a batch do not depend on one another, so a graph holds them as chains of launches of the
+// A graph of b->chunk steps of every lattice, each lattice's steps a child graph of its own. The lattices of a batch do not depend on one another, so they are chains of launches of the
 // single-lattice step, which reads its parameters from the constant bank where the batched kernel
 // reads them from shared memory under a register cap, and lets the hardware run the chains side by
 // side: 12 boxes of edge 24 to 128 (3.1 million nodes) 175.0 -> 138.6 us per step in FP32, 194.7 -> 111.6 in
 // FP16; 12 of edge 16 to 48 33.6 -> 16.2; 48 of edge 16 to 32 62.8 -> 35.9 (16 chains). Fewer chains leave
-// the chip idle (12 boxes: 4 chains 150.5, 2 166.7). Lattices go to chains largest first, each to the
-// least loaded. Steps that fill no graph go through the batched kernel, one launch for all lattices;
-// graphs of large batches are therefore short (their launch is small against kShortChunk steps).
-clb_status batch3_chains(clb3d_batch* b, int start)
+// the chip idle (12 boxes: 4 chains 150.5, 2 166.7). At most kMaxChains run at once, largest first.
+// Steps that fill no graph go through the batched kernel, one launch for all lattices; graphs of large
+// batches are therefore short (their launch is small against kShortChunk steps).
+clb_status batch3_chains(clb3d_batch* b, int start, cudaGraph_t g)
 {
     std::vector<int> order(b->lat.size());
     for (size_t k = 0; k < order.size(); ++k) order[k] = (int)k;
     std::sort(order.begin(), order.end(), [&](int i, int j) { return nodes_of(b->lat[i]) > nodes_of(b->lat[j]); });
-    std::vector<long long> load(b->side.size(), 0);
-    CLB_CUDA(cudaEventRecord(b->fork, b->cap));
-    for (cudaStream_t t : b->side) CLB_CUDA(cudaStreamWaitEvent(t, b->fork, 0));
-    for (int k : order) {
-        const size_t c = std::min_element(load.begin(), load.end()) - load.begin();
-        load[c] += nodes_of(b->lat[k]);
-        for (int q = 0; q < b->chunk; ++q) CLB_TRY(launch_step3(b->lat[k], start ^ b->flip[k] ^ (q & 1), b->side[c]));
-    }
-    for (size_t c = 0; c < b->side.size(); ++c) {
-        CLB_CUDA(cudaEventRecord(b->join[c], b->side[c]));
-        CLB_CUDA(cudaStreamWaitEvent(b->cap, b->join[c], 0));
+    std::vector<cudaGraphNode_t> nodes(order.size());
+    for (size_t i = 0; i < order.size(); ++i) {
+        const int k = order[i];
+        CLB_CUDA(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
+        clb_status st = CLB_OK;
+        for (int q = 0; q < b->chunk && st == CLB_OK; ++q) st = launch_step3(b->lat[k], start ^ b->flip[k] ^ (q & 1), b->cap);
+        cudaGraph_t child = nullptr;
+        cudaError_t e = cudaStreamEndCapture(b->cap, &child);
+        if (st == CLB_OK && e == cudaSuccess)
+            e = cudaGraphAddChildGraphNode(&nodes[i], g, i < kMaxChains ? nullptr : &nodes[i - kMaxChains], i < kMaxChains ? 0 : 1, child);
+        if (child) cudaGraphDestroy(child);
+        if (st != CLB_OK) return st;
+        if (e != cudaSuccess) return set_error(CLB_ECUDA, "graph of lattice %d: %s", k, cudaGetErrorString(e));
     }
     return CLB_OK;
 }
 
 clb_status batch3_graph(clb3d_batch* b, int start)
 {
-    CLB_CUDA(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
+    cudaGraph_t g = nullptr;
     clb_status st = CLB_OK;
     if (b->chains) {
+        CLB_CUDA(cudaGraphCreate(&g, 0));
         try {
-            st = batch3_chains(b, start);
+            st = batch3_chains(b, start, g);
         } catch (const std::bad_alloc&) {
             st = set_error(CLB_ENOMEM, "host allocation failed");
         }
     } else {
+        CLB_CUDA(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
         for (int k = 0; k < b->chunk && st == CLB_OK; ++k) st = batch3_launch(b, start ^ (k & 1), b->cap);
+        const cudaError_t e = cudaStreamEndCapture(b->cap, &g);
+        if (st == CLB_OK && e != cudaSuccess) st = set_error(CLB_ECUDA, "graph capture: %s", cudaGetErrorString(e));
     }
-    cudaGraph_t g = nullptr;
-    const cudaError_t e = cudaStreamEndCapture(b->cap, &g);
-    if (st != CLB_OK) {
-        if (g) cudaGraphDestroy(g);
-        return st;
+    if (st == CLB_OK) {
+        const cudaError_t e = cudaGraphInstantiate(&b->graph[start], g, 0);
+        if (e != cudaSuccess) st = set_error(CLB_ECUDA, "graph instantiate: %s", cudaGetErrorString(e));
     }
-    if (e != cudaSuccess) return set_error(CLB_ECUDA, "graph capture: %s", cudaGetErrorString(e));
-    const cudaError_t e2 = cudaGraphInstantiate(&b->graph[start], g, 0);
-    cudaGraphDestroy(g);
-    if (e2 != cudaSuccess) return set_error(CLB_ECUDA, "graph instantiate: %s", cudaGetErrorString(e2));
-    return CLB_OK;
+    if (g) cudaGraphDestroy(g);
+    return st;
 }
 
 #define CHECK_B3(b) \
@@ -1642,19 +1640,11 @@ extern "C" clb_status clb3d_batch_create(int n, const int* nx, const int* ny, co
                 b->flip.push_back(0);
             }
         }
-        cudaError_t e = st == CLB_OK ? cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) : cudaSuccess;
-        if (st == CLB_OK && e == cudaSuccess) e = cudaEventCreateWithFlags(&b->fork, cudaEventDisableTiming);
-        const size_t nchains = std::min(n, kMaxChains);
-        b->side.assign(nchains, nullptr);
-        b->join.assign(nchains, nullptr);
-        for (size_t c = 0; c < nchains && st == CLB_OK && e == cudaSuccess; ++c) {
-            e = cudaStreamCreateWithFlags(&b->side[c], cudaStreamNonBlocking);
-            if (e == cudaSuccess) e = cudaEventCreateWithFlags(&b->join[c], cudaEventDisableTiming);
-        }
+        if (st == CLB_OK && cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess)
+            st = set_error(CLB_ECUDA, "batch set-up: %s", cudaGetErrorString(cudaGetLastError()));
         long long nodes = 0;
         for (const clb3d_lattice* h : b->lat) nodes += nodes_of(h);
         if (nodes >= 500000) b->chunk = kShortChunk;
-        if (e != cudaSuccess) st = set_error(CLB_ECUDA, "batch set-up: %s", cudaGetErrorString(e));
         if (st == CLB_OK) st = batch3_tables(b);
     } catch (const std::bad_alloc&) {
         st = set_error(CLB_ENOMEM, "host allocation failed");
@@ -1676,11 +1666,6 @@ extern "C" void clb3d_batch_destroy(clb3d_batch* b)
     cudaFree(b->d_members);
     cudaFree(b->d_owner);
     if (b->cap) cudaStreamDestroy(b->cap);
-    for (auto& t : b->side)
-        if (t) cudaStreamDestroy(t);
-    for (auto& t : b->join)
-        if (t) cudaEventDestroy(t);
-    if (b->fork) cudaEventDestroy(b->fork);
     delete b;
 }
 
