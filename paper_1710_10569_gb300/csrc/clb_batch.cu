@@ -655,10 +655,10 @@ private:
 };
 
 // Device addresses where the four host fields of a member are staged for its initialisation, and
-// where its fields are written for the host at retirement: rho, u_x, u_y in the population buffer
-// that the next step would write (at least 28 bytes per node in every storage form, 24 needed)
-// and T in the T slot of the residual snapshot, which k_fields rewrites only after k_init has read
-// it (stream order). No extra device memory is needed.
+// where its fields are written for the host at retirement: one after another in the population
+// buffer that the next step would write (56 bytes per node or more, 32 needed), but in the FP16 form
+// (28 bytes per node) T in the T slot of the residual snapshot, which k_snap rewrites only after
+// k_init has read it (stream order). No extra device memory is needed.
 void own_stage(const Lattice* L, int parity, double* dev[4])
 {
     const size_t N = (size_t)L->nx * L->ny;
@@ -666,14 +666,27 @@ void own_stage(const Lattice* L, int parity, double* dev[4])
     dev[0] = spare;
     dev[1] = spare + N;
     dev[2] = spare + 2 * N;
-    dev[3] = L->snap + 2 * N;
+    dev[3] = L->p.storage == CLB_F16DEV ? L->snap + 2 * N : spare + 3 * N;
+}
+
+// A request's four fields between its host array (rho, u_x, u_y, T one after another) and the member's
+// staging addresses, as one copy where these lie one after another too: a copy from or to pageable
+// memory costs the host some 10 us whatever its size (24 requests of 8,000 nodes, beside 730 us of
+// stepping: admission 1,140 -> 990 us, retirement 1,200 -> 380 us).
+template <typename D, typename S>
+clb_status copy_request(D* const* dst, S* const* src, size_t N, cudaMemcpyKind kind, cudaStream_t stream)
+{
+    const int first = dst[3] == dst[0] + 3 * N && src[3] == src[0] + 3 * N ? 4 : 3;
+    CLB_CUDA(cudaMemcpyAsync(dst[0], src[0], first * N * sizeof(double), kind, stream));
+    if (first == 3) CLB_CUDA(cudaMemcpyAsync(dst[3], src[3], N * sizeof(double), kind, stream));
+    return CLB_OK;
 }
 
 // Copy host fields (any may be NULL) into the member's own staging addresses and initialise it.
-// With `wait`, returns after the copies are done (the caller may then reuse its host arrays even
-// when they are pinned); otherwise the copies are only ordered on the stream.
+// Returns after the copies are done (the caller may then reuse its host arrays even when they are
+// pinned).
 clb_status init_from_host(Ensemble& E, Lattice* L, const double* rho, const double* ux, const double* uy,
-                          const double* T, bool wait)
+                          const double* T)
 {
     const size_t N = (size_t)L->nx * L->ny;
     const double* src[4] = {rho, ux, uy, T};
@@ -686,7 +699,7 @@ clb_status init_from_host(Ensemble& E, Lattice* L, const double* rho, const doub
             dev[k] = stage[k];
         }
     CLB_TRY(E.init_member(L, dev[0], dev[1], dev[2], dev[3]));
-    if (wait) CLB_CUDA(cudaStreamSynchronize(E.stream));
+    CLB_CUDA(cudaStreamSynchronize(E.stream));
     return CLB_OK;
 }
 
@@ -771,7 +784,7 @@ extern "C" clb_status clb_batch_init_fields(clb_batch* b, int k, const double* r
         }
         L->status = CLB_OK;
         L->er = INFINITY;
-        return init_from_host(b->E, L, rho, ux, uy, T, true);
+        return init_from_host(b->E, L, rho, ux, uy, T);
     } catch (const std::bad_alloc&) {
         return host_alloc_failed();
     }
@@ -800,11 +813,13 @@ extern "C" clb_status clb_batch_fields(clb_batch* b, int k, double* rho, double*
         double* spare = (double*)L->buf[b->E.parity ^ 1];
         double* dev[4];
         for (int i = 0; i < 4; ++i) dev[i] = nullptr;
+        const bool f16 = L->p.storage == CLB_F16DEV;
         for (int i = 0, slot = 0; i < 4; ++i)
-            if (host[i]) dev[i] = spare + (slot++ % 3) * N;
-        // at most three fields fit the spare buffer at once: fetch in two rounds when all four are asked
+            if (host[i]) dev[i] = spare + (f16 ? slot++ % 3 : slot++) * N;
+        // only three fields fit the spare buffer of the FP16 form (28 bytes per node): fetch in two
+        // rounds when all four are asked
         const int n_asked = (rho != nullptr) + (ux != nullptr) + (uy != nullptr) + (T != nullptr);
-        if (n_asked == 4) {
+        if (f16 && n_asked == 4) {
             CLB_TRY(b->E.fields(L, dev[0], dev[1], dev[2], nullptr));
             for (int i = 0; i < 3; ++i)
                 CLB_CUDA(cudaMemcpyAsync(host[i], dev[i], N * sizeof(double), cudaMemcpyDeviceToHost, b->E.stream));
@@ -1047,12 +1062,12 @@ namespace {
 struct Request {
     long id;
     std::unique_ptr<Lattice> L;
-    std::vector<double> init;  // 4 * N host copy, released at admission
+    std::unique_ptr<double[]> init;  // 4 * N host copy, released at admission
     long cap;
     double tol;
     long tiles = 0;  // entries of the tile-owner table at one group of rows per block
     int done = 0;
-    std::vector<double> result;  // 4 * N after retirement
+    std::unique_ptr<double[]> result;  // 4 * N after retirement
 };
 
 // Best-fit sub-allocation of one device reservation in 256-byte blocks; a released block merges
@@ -1190,12 +1205,12 @@ extern "C" clb_status clb_serve_submit(clb_server* s, int nx, int ny, const clb_
         r->tol = tol;
         r->tiles = tiles;
         const size_t N = (size_t)nx * ny;
-        r->init.assign(4 * N, 0.0);
+        r->init.reset(new double[4 * N]);
         const double* src[4] = {rho, ux, uy, T};
         const double dflt[4] = {1.0, 0.0, 0.0, p->T0};
         for (int k = 0; k < 4; ++k) {
-            if (src[k]) std::memcpy(r->init.data() + k * N, src[k], N * sizeof(double));
-            else std::fill(r->init.begin() + k * N, r->init.begin() + (k + 1) * N, dflt[k]);
+            if (src[k]) std::memcpy(r->init.get() + k * N, src[k], N * sizeof(double));
+            else std::fill_n(r->init.get() + k * N, N, dflt[k]);
         }
         if (req_id) *req_id = r->id;
         s->queue.push_back(r.get());
@@ -1246,10 +1261,14 @@ extern "C" clb_status clb_serve_progress(clb_server* s, long chunk, int* active,
             const size_t N = (size_t)r->L->nx * r->L->ny;
             // keep the padding of each row's last chunk defined (it is never read)
             CLB_CUDA(cudaMemsetAsync(mem, 0, 2 * buffer_slot_bytes(r->L->nx, r->L->ny, r->L->p.storage), s->E.stream));
-            const double* h = r->init.data();
+            const double* h = r->init.get();
             // pageable source: the copies have left the host array when they return
-            CLB_TRY(init_from_host(s->E, r->L.get(), h, h + N, h + 2 * N, h + 3 * N, false));
-            std::vector<double>().swap(r->init);
+            const double* src[4] = {h, h + N, h + 2 * N, h + 3 * N};
+            double* dev[4];
+            own_stage(r->L.get(), s->E.parity, dev);
+            CLB_TRY(copy_request(dev, src, N, cudaMemcpyHostToDevice, s->E.stream));
+            CLB_TRY(s->E.init_member(r->L.get(), dev[0], dev[1], dev[2], dev[3]));
+            r->init.reset();
             s->used += r->L->bytes;
             s->tiles_used += r->tiles;
             s->rows_used += r->L->ny;
@@ -1273,11 +1292,11 @@ extern "C" clb_status clb_serve_progress(clb_server* s, long chunk, int* active,
                 const size_t N = (size_t)L->nx * L->ny;
                 double* dev[4];
                 own_stage(L, s->E.parity, dev);
-                r->result.assign(4 * N, 0.0);
+                r->result.reset(new double[4 * N]);
                 CLB_TRY(s->E.fields(L, dev[0], dev[1], dev[2], dev[3]));
-                for (int k = 0; k < 4; ++k)
-                    CLB_CUDA(cudaMemcpyAsync(r->result.data() + k * N, dev[k], N * sizeof(double), cudaMemcpyDeviceToHost,
-                                             s->E.stream));
+                double* host[4];
+                for (int k = 0; k < 4; ++k) host[k] = r->result.get() + k * N;
+                CLB_TRY(copy_request(host, dev, N, cudaMemcpyDeviceToHost, s->E.stream));
             }
             if (!leaving.empty()) CLB_CUDA(cudaStreamSynchronize(s->E.stream));
             for (Request* r : leaving) {
@@ -1345,7 +1364,7 @@ extern "C" clb_status clb_serve_fetch(clb_server* s, long req_id, double* rho, d
         const size_t N = (size_t)r->L->nx * r->L->ny;
         double* out[4] = {rho, ux, uy, T};
         for (int k = 0; k < 4; ++k)
-            if (out[k]) std::memcpy(out[k], r->result.data() + k * N, N * sizeof(double));
+            if (out[k]) std::memcpy(out[k], r->result.get() + k * N, N * sizeof(double));
         s->all.erase(it);
         return CLB_OK;
     } catch (const std::bad_alloc&) {

@@ -138,10 +138,10 @@ __device__ __forceinline__ void reduce_row(const E* __restrict__ src, const LatP
 // sums are FP64 and GB300 issues FP64 slowly, so each thread takes 8 nodes (the warp tree's
 // FP64 adds per thread are shared by 8 nodes); the register cap keeps 4 blocks per SM so that
 // enough gathers are in flight. For nx <= kDiagNodes the order is that of reduce_row. The FP64 pipe
-// bounds it: per node 5 additions for the FP32 and FP16 forms (10 instructions while the terms were
-// converted by it) and 1 per node for the tree (4 before the exchange in block_sum). With the
-// read-back a pass takes 78.9 us on 2048 x 1024 FP32 nodes (103.0 before), 213 on 4096 x 2048 FP16
-// (304), 31.5 on 513 x 385 FP32 (43.0).
+// bounded it: per node 5 additions for the FP32 and FP16 forms (10 instructions while the terms were
+// converted by it) and 1 per node for the tree (4 before the exchange in block_sum). It is 50% busy
+// now, DRAM 46%, and the wait for the gathers is what is left. With the read-back a pass takes 78.9 us
+// on 2048 x 1024 FP32 nodes (103.0 before), 213 on 4096 x 2048 FP16 (304), 31.5 on 513 x 385 FP32 (43.0).
 constexpr int kDiagNodes = kReduceThreads * 8;
 
 template <int ST>
