@@ -523,7 +523,7 @@ extern "C" clb_status clb_create(int nx, int ny, const clb_params* p, void* stre
         int sms = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
         default_shape(p->storage, nx, ny, std::max(1, sms), &h->bx, &h->by, &h->npt);
-        bool tuned = false;
+        h->march = march_rows_rule(nx, ny, *p, std::max(1, sms));
         {
             std::lock_guard<std::mutex> lk(g_tune_mu);
             auto it = g_tune_cache.find(std::make_tuple(p->storage, nx, ny));
@@ -533,12 +533,9 @@ extern "C" clb_status clb_create(int nx, int ny, const clb_params* p, void* stre
                 h->npt = it->second[2];
                 h->pipe_stages = it->second[3];
                 h->pipe_rows = it->second[4];
-                h->march = it->second[5];
-                tuned = true;
+                // two steps per launch only where these walls allow it (the cache knows sizes alone)
+                if (h->march > 0) h->march = it->second[5];
             }
-        }
-        if (!tuned) {
-            h->march = march_rows_rule(nx, ny, *p, std::max(1, sms));
         }
         // the padding of each row's last chunk is never read, but keep it defined
         e = cudaMemsetAsync(h->mem, 0, L.snap, h->stream);

@@ -47,6 +47,26 @@ def test_two_steps_per_launch_equal_one(clb, layout, shape, steps):
         assert np.isfinite(a).all() and np.array_equal(a, b)
 
 
+# The autotuner's choice is kept by storage form and size: a lattice of that size with wet walls, which the
+# two-step kernel does not know, steps as under an explicit shape whatever another lattice's tuning chose.
+def test_wet_walls_after_tuning_the_same_size(clb):
+    prob = W.random_problem(2048, 600, seed=5, storage=W.STORAGE_F32, walls=LAYOUTS["layer"])
+    lat = clb.Lattice.from_problem(prob)
+    lat.autotune()
+    lat.close()
+    prob.params.update(wall=(P, P, W.WALL_WET, W.WALL_WET))
+    got = []
+    for shape_set in (False, True):
+        lat = clb.Lattice.from_problem(prob)
+        if shape_set:
+            lat.set_launch(128, 1, 2)
+        lat.step(6)
+        got.append(lat.populations())
+        lat.close()
+    for a, b in zip(*got):
+        assert np.isfinite(a).all() and np.array_equal(a, b)
+
+
 # The temperature equation alone: four steps per launch against the same number of calls of one step.
 @pytest.mark.parametrize("shape", [(8193, 49), (4096, 101), (1121, 358), (112, 3601), (55, 7301), (703, 702)],
                          ids=lambda v: f"{v[0]}x{v[1]}")
