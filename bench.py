@@ -5,13 +5,15 @@ Dirichlet walls T = +-0.5 at the bottom/top, Ra = 1e7, Pr = 0.71, u_c = 0.1, see
 1e-3, FP32 population storage and FP32 arithmetic. One bench step = one time step of the whole
 lattice (every node: pull, macroscopics, D2Q9 and D2Q5 central-moment collision, store).
 
-Metric: MLUPS (million coupled node updates per second), with the fused step kernel's fraction of
-the measured HBM copy bandwidth. The timed region runs K steps through clb_run (the fused step every
-step, the FP64 Nusselt number and residual every 100 steps and after the last one) on the lattice's
-stream; the two population buffers (2 x 117 MB in FP32) exceed the 129 MB L2. The roofline times the
-step kernel alone over a fixed window of 2048 graph-replayed launches (both graph parities captured
-before the window), and the DRAM bytes per launch measured by ncu are reported beside the
-algorithmic bytes.
+Metric: MLUPS (million coupled node updates per second), with the step kernel's fraction of the
+measured HBM copy bandwidth. The timed region runs K steps through clb_run (every step of the whole
+lattice; the FP64 Nusselt number and residual every 100 steps and after the last one) on the
+lattice's stream; the two population buffers (2 x 117 MB in FP32) exceed the 129 MB L2. An FP32
+lattice of this size advances two time steps per kernel launch (every node is collided and streamed
+twice, the state between the two steps staying on the chip), so the populations cross HBM once per
+two steps. The roofline times the step kernel alone over a fixed window of 2048 graph-replayed steps
+(both graph parities captured before the window), its bytes are those that one launch has to move,
+and the DRAM bytes per launch measured by ncu are reported beside them.
 
 Usage: python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
 For N > 1 (torchrun) every rank steps its own replica of the lattice (replicas only: the
@@ -57,7 +59,8 @@ DTYPE = {W.STORAGE_F64: "f64", W.STORAGE_F32: "f32", W.STORAGE_F16DEV: "f16dev s
 # 56 B per node, so at 2048 x 1024 a step's 117 MB would fit the 129 MB L2; it runs at 4096 x 2048.
 VARIANT_SIZE = {W.STORAGE_F64: (2048, 1024), W.STORAGE_F32: (2048, 1024), W.STORAGE_F16DEV: (4096, 2048)}
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "k_step_traffic.json")
-KERNEL_SOURCES = ["paper_1710_10569_gb300/csrc/clb_core.cuh", "paper_1710_10569_gb300/csrc/clb_kernels.cuh"]
+KERNEL_SOURCES = ["paper_1710_10569_gb300/csrc/clb_core.cuh", "paper_1710_10569_gb300/csrc/clb_kernels.cuh",
+                  "paper_1710_10569_gb300/csrc/clb_march.cuh"]
 KERNEL3D_SOURCES = ["paper_1710_10569_gb300/csrc/clb_core.cuh", "paper_1710_10569_gb300/csrc/clb3d.cu"]
 
 
@@ -106,16 +109,13 @@ def profile_counts():
     return d if d.get("kernel_source_hash") == kernel_hash() else {}
 
 
-def flops_per_node():
-    """Floating-point operations per node update (an FMA counted as two), from the FP64 step's
-    committed ncu instruction counts, if they were taken on the current kernel source (else None).
-    The FP32 and FP16 forms evaluate the same expressions except the ten 1-D inverse pairs
-    (s + d)/2, (s - d)/2 per node, which their packed pairs form as two sums and two halvings (4
-    flops) where FP64 uses one halving and two FMAs (5 flops): 8 flops fewer per node."""
-    ops = profile_counts().get("fp64_ops_per_node")
-    if not ops:
-        return None
-    return 2 * ops["dfma"] + ops["dadd"] + ops["dmul"]
+def flops_per_node(storage: int):
+    """Floating-point operations per node update (an FMA counted as two, a packed FP32 instruction
+    as two of its kind) of the storage form's step kernel, from its committed ncu instruction counts
+    (the two-step kernel's halo nodes included), if they were taken on the current kernel source
+    (else None)."""
+    ops = profile_counts().get("launches", {}).get(W.STORAGE_NAMES[storage], {}).get("flops_per_node")
+    return float(ops) if ops else None
 
 
 def traffic_per_launch(storage: int, nx: int, ny: int):
@@ -223,15 +223,27 @@ def aggregate(units: float, seconds: float, world: int):
     return float(u.item()), float(s.item())
 
 
-def kernels_per_step(storage: int) -> int:
-    """Kernels one step launches on a Rayleigh-Benard lattice: the FP16 form splits the step into
-    an interior kernel and an edge kernel (wall rows) that run side by side."""
-    return 2 if storage == W.STORAGE_F16DEV else 1
+def steps_per_launch(storage: int, nodes: int) -> int:
+    """Time steps that one launch advances a Rayleigh-Benard lattice by under the library's default:
+    two for FP32 lattices of a million nodes or more."""
+    return 2 if storage == W.STORAGE_F32 and nodes >= 1_000_000 else 1
 
 
-def step_kernel_name(storage: int) -> str:
+def step_kernels(storage: int, nodes: int, steps: int) -> int:
+    """Step kernels that clb_run launches over `steps` steps (DIAG_INTERVAL at a time) on a
+    Rayleigh-Benard lattice: an odd step is a launch by itself where launches take two, and an FP16
+    lattice of this size splits its step into an interior kernel and an edge kernel (wall rows) that
+    run side by side."""
+    per = steps_per_launch(storage, nodes)
+    parts = [min(DIAG_INTERVAL, steps - k) for k in range(0, steps, DIAG_INTERVAL)]
+    return sum(-(-n // per) for n in parts) * (2 if storage == W.STORAGE_F16DEV else 1)
+
+
+def step_kernel_name(storage: int, nodes: int) -> str:
     if storage == W.STORAGE_F16DEV:
         return "k_step_inner_f16x4_hi1 + k_step_edge<f16dev> (one step)"
+    if steps_per_launch(storage, nodes) == 2:
+        return f"k_step_two ({W.STORAGE_NAMES[storage]}, two steps)"
     return f"k_step<{W.STORAGE_NAMES[storage]}>"
 
 
@@ -266,7 +278,7 @@ def time_run(lat, steps: int, warmup: int, world: int):
     return e0.elapsed_time(e1) / 1e3
 
 
-KERNEL_WINDOW = 2048  # launches of the step kernel timed for the roofline (64 graph replays)
+KERNEL_WINDOW = 2048  # steps of the step kernel timed for the roofline (64 graph replays)
 
 
 def diag_checks(steps: int) -> int:
@@ -276,7 +288,7 @@ def diag_checks(steps: int) -> int:
 
 
 def time_steps(lat, steps: int, warmup: int, world: int):
-    """Device time of `steps` launches of the fused step kernel alone (graph replays). The
+    """Device time of `steps` steps of the fused step kernel alone (graph replays). The
     warm-up runs 64 steps first: the library captures the graphs of both buffer parities on its
     first 32-step chunk, so no capture or instantiation falls inside the timed window."""
     import torch
@@ -348,7 +360,8 @@ def e2e_run(storage: int, steps: int, nx: int, ny: int):
 
 def thermal_run(storage: int, steps: int, nx: int = 4096, ny: int = 4096):
     """The D2Q5-only step with a prescribed velocity (a cellular flow of amplitude 0.1) on a
-    Rayleigh-Benard temperature field: 5 populations in and out plus the node's velocity. The
+    Rayleigh-Benard temperature field: 5 populations in and out plus the node's velocity, per launch
+    (four steps in the FP32 and FP16 forms). The
     lattice is 4096 x 4096 so that a step's working set (two 336 MB FP32 buffers and 134 MB of
     velocities) is several times the 129 MB L2; at 2048 x 1024 it would fit."""
     import torch
@@ -372,17 +385,18 @@ def thermal_run(storage: int, steps: int, nx: int = 4096, ny: int = 4096):
     dt = e0.elapsed_time(e1) / 1e3
     th.close()
     per_node = {W.STORAGE_F64: 96, W.STORAGE_F32: 48, W.STORAGE_F16DEV: 28}[storage]
+    per = 1 if storage == W.STORAGE_F64 else 4  # steps per launch of a lattice of this size
     peak, _ = measured_peaks()
-    gbs = per_node * nx * ny * steps / dt / 1e9
+    gbs = per_node * nx * ny * steps / per / dt / 1e9
     return {"workload": f"thermal_only_{nx}x{ny}_cellular_flow", "mlups": nx * ny * steps / dt / 1e6,
-            "bytes_per_node": per_node, "achieved_gbs": gbs, "hbm_frac": gbs / peak, "steps": steps,
-            "storage": W.STORAGE_NAMES[storage]}
+            "bytes_per_node": per_node, "steps_per_launch": per, "achieved_gbs": gbs, "hbm_frac": gbs / peak,
+            "steps": steps, "storage": W.STORAGE_NAMES[storage]}
 
 
 def batched_run(storage: int, count: int = 256, steps: int = 1000, seq_subset: int = 32):
     """Many side-heated cavities of uneven sizes (edge log-uniform 64-512, Ra log-uniform 1e3-1e6,
-    Pr uniform 0.71-7) stepped in one launch per time step, against the same instances stepped one
-    after another through single-lattice handles (a seeded subset of `seq_subset` instances is timed
+    Pr uniform 0.71-7) stepped in one launch per time step (FP32: per two time steps), against the
+    same instances stepped one after another through single-lattice handles (a seeded subset of `seq_subset` instances is timed
     both ways)."""
     import torch
     from paper_1710_10569_gb300 import clb
@@ -411,6 +425,7 @@ def batched_run(storage: int, count: int = 256, steps: int = 1000, seq_subset: i
         return dt, launch
 
     dt_all, launch = time_batch(probs, steps)
+    per = 2 if storage == W.STORAGE_F32 else 1  # steps per launch of a batch of this size
     peak, _ = measured_peaks()
     sub = probs[:seq_subset]
     sub_nodes = sum(p.nodes for p in sub)
@@ -429,8 +444,8 @@ def batched_run(storage: int, count: int = 256, steps: int = 1000, seq_subset: i
     return {"instances": count, "nodes": nodes, "steps": steps, "storage": W.STORAGE_NAMES[storage],
             "tile": list(launch["tile"]), "row_groups_per_block": launch["groups"],
             "blocks_per_launch": launch["blocks"], "mlups": nodes * steps / dt_all / 1e6,
-            "hbm_frac": nodes * steps * BYTES_PER_NODE[storage] / dt_all / 1e9 / peak,
-            "instance_steps_per_s": count * steps / dt_all,
+            "hbm_frac": nodes * steps / per * BYTES_PER_NODE[storage] / dt_all / 1e9 / peak,
+            "steps_per_launch": per, "instance_steps_per_s": count * steps / dt_all,
             "subset": {"instances": seq_subset, "batched_mlups": sub_nodes * steps / dt_sub / 1e6,
                        "sequential_mlups": sub_nodes * steps / dt_seq / 1e6,
                        "speedup": dt_seq / dt_sub}}
@@ -475,8 +490,8 @@ def three_d_run(steps: int, nx: int = 256, ny: int = 256, nz: int = 128):
 
 def batched3d_run(steps: int, count: int = 48, seq_subset: int = 12):
     """A 3-D batch: 48 Rayleigh-Benard boxes with extents log-uniform in 24-128 (each axis drawn
-    separately), FP32, one k_step3_batched launch per step, against a seeded subset stepped one
-    lattice after another through single-lattice launches; CUDA events on the batch's stream."""
+    separately), FP32, its lattices' chains of steps side by side in one graph, against a seeded
+    subset stepped one lattice after another through single-lattice launches; CUDA events on the batch's stream."""
     import torch
     from paper_1710_10569_gb300 import clb
     peak, _ = measured_peaks()
@@ -691,14 +706,16 @@ def run_ours(args):
     with ClockSampler(local) as clocks:
         secs = time_run(lat, args.steps, args.warmup, world)
         # the dominant kernel alone, for the roofline: its average launch duration over a fixed
-        # window of graph-replayed launches, whatever --steps is
+        # window of graph-replayed steps, whatever --steps is
         k_steps = KERNEL_WINDOW
         secs_kernel = time_steps(lat, k_steps, 3, world)
     nodes = prob.nodes
     units, tmax = aggregate(float(nodes) * args.steps, secs, world)
     mlups = units / tmax / 1e6
     peak, peak_kind = measured_peaks()
-    per_launch_s = secs_kernel / k_steps
+    per = steps_per_launch(storage, nodes)
+    launches = k_steps // per
+    per_launch_s = secs_kernel / launches
     alg_bytes = BYTES_PER_NODE[storage] * nodes
     achieved = alg_bytes / per_launch_s / 1e9
     traffic = traffic_per_launch(storage, prob.nx, prob.ny)
@@ -715,12 +732,13 @@ def run_ours(args):
                 l2.autotune()
             k = max(200, args.steps // (8 if st == W.STORAGE_F64 else 2))
             s2 = time_steps(l2, k, max(3, args.warmup // 4), 1)
+            per2 = steps_per_launch(st, p2.nodes)
             variants[W.STORAGE_NAMES[st]] = {
                 "workload": f"rayleigh_benard_{p2.nx}x{p2.ny}_Ra1e7_Pr0.71",
                 "mlups": p2.nodes * k / s2 / 1e6,
-                "achieved_gbs": BYTES_PER_NODE[st] * p2.nodes / (s2 / k) / 1e9,
-                "hbm_frac": BYTES_PER_NODE[st] * p2.nodes / (s2 / k) / 1e9 / peak,
-                "steps": k, "dram_bytes_per_launch": traffic_per_launch(st, p2.nx, p2.ny),
+                "achieved_gbs": BYTES_PER_NODE[st] * p2.nodes * k / per2 / s2 / 1e9,
+                "hbm_frac": BYTES_PER_NODE[st] * p2.nodes * k / per2 / s2 / 1e9 / peak,
+                "steps_per_launch": per2, "steps": k, "dram_bytes_per_launch": traffic_per_launch(st, p2.nx, p2.ny),
                 "working_set_mb": BYTES_PER_NODE[st] * p2.nodes / 1e6,
                 "launch": list(l2.launch())}
             ops = profile_counts().get("fp64_ops_per_node")
@@ -749,30 +767,31 @@ def run_ours(args):
             "scaling": "weak", "vs_baseline": None, "dtype": DTYPE[storage], "data": "synthetic",
             "config": {"workload": f"rayleigh_benard_{prob.nx}x{prob.ny}_Ra1e7_Pr0.71",
                        "nodes": nodes, "storage": W.STORAGE_NAMES[storage],
-                       "step": "fused collide-and-stream every step; FP64 Nusselt number and residual "
+                       "step": f"fused collide-and-stream of every node every step, {per} step(s) per "
+                               "launch; FP64 Nusselt number and residual "
                                f"reduced and read back every {DIAG_INTERVAL} steps and after the last "
                                f"step (clb_run): {diag_checks(args.steps)} check(s) inside the timed "
                                f"{args.steps} steps",
                        "diag_checks_timed": diag_checks(args.steps),
                        "launch": list(lat.launch()),
-                       "l2": "no flush: each step reads one population buffer and writes the "
+                       "l2": "no flush: each launch reads one population buffer and writes the "
                              f"other ({alg_bytes / 2 / 1e6:.0f} MB each, {alg_bytes / 1e6:.0f} MB "
-                             "per step against the 129 MB L2); roofline.traffic is the ncu DRAM "
+                             "per launch against the 129 MB L2); roofline.traffic is the ncu DRAM "
                              "bytes per launch",
                        "parallelism": f"replicas x{world}"},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                          "frac": achieved / peak, "traffic": traffic,
-                         "kernel_launches_timed": k_steps,
+                         "steps_per_launch": per, "kernel_launches_timed": launches,
                          "kernel_us_per_launch": per_launch_s * 1e6,
                          "algorithmic_bytes_per_launch": alg_bytes,
-                         "kernel": step_kernel_name(storage),
-                         "flops_per_node": flops_per_node(),
+                         "kernel": step_kernel_name(storage, nodes),
+                         "flops_per_node": flops_per_node(storage),
                          "peak_kind": f"{peak_kind} HBM copy bandwidth (MEASURED_PEAKS.json hbm_gbs)"},
             "cpu_baseline": cpu,
             "e2e": e2e,
-            # every step's fused kernel (the FP16 form: the interior and edge kernels), plus the
-            # two reduction kernels of each check
-            "gpu_launches": args.steps * kernels_per_step(storage) + 2 * diag_checks(args.steps),
+            # the step kernels (two steps each in the FP32 form at this size; the FP16 form: an interior
+            # and an edge kernel per step), plus the two reduction kernels of each check
+            "gpu_launches": step_kernels(storage, nodes, args.steps) + 2 * diag_checks(args.steps),
             "clocks": clocks.summary(),
             "variants": variants,
             "thermal_only": thermal,
