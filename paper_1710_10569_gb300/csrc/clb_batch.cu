@@ -449,7 +449,7 @@ public:
         char* hm = (char*)h_tables + off_members;
         int* owner = (int*)((char*)h_tables + off_owner);
         int* row_owner = (int*)((char*)h_tables + off_rows);
-        double* ddiag = (double*)((char*)d_tables + off_diag);
+        double* ddiag = (double*)((char*)h_tables + off_diag);  // written by the last kernel of a check
         int* march_owner = (int*)((char*)h_tables + off_march);
         int t = 0, r = 0, mw = 0;
         for (size_t k = 0; k < active.size(); ++k) {
@@ -560,7 +560,7 @@ public:
     }
 
     // Nu and E_R (snapshot retaken when update) of every active member; sets L->nu, L->er, status.
-    // The outputs of all members come back in one copy.
+    // The last kernel writes the outputs of all members to the pinned mirror.
     clb_status diagnostics(int update)
     {
         CLB_TRY(rebuild());
@@ -578,9 +578,7 @@ public:
         else
             k_reduce_final_batched<float><<<(int)active.size(), kReduceThreads, 0, stream>>>((const Member<float>*)m);
         CLB_CUDA(cudaGetLastError());
-        double* hd = (double*)((char*)h_tables + off_diag);
-        CLB_CUDA(cudaMemcpyAsync(hd, (char*)d_tables + off_diag, active.size() * kDiagStride * sizeof(double),
-                                 cudaMemcpyDeviceToHost, stream));
+        const double* hd = (const double*)((char*)h_tables + off_diag);
         CLB_CUDA(cudaStreamSynchronize(stream));
         for (size_t k = 0; k < active.size(); ++k) {
             Lattice* L = active[k];

@@ -140,8 +140,9 @@ __device__ __forceinline__ void reduce_row(const E* __restrict__ src, const LatP
 // enough gathers are in flight. For nx <= kDiagNodes the order is that of reduce_row. The FP64 pipe
 // bounded it: per node 5 additions for the FP32 and FP16 forms (10 instructions while the terms were
 // converted by it) and 1 per node for the tree (4 before the exchange in block_sum). It is 50% busy
-// now, DRAM 46%, and the wait for the gathers is what is left. With the read-back a pass takes 78.9 us
-// on 2048 x 1024 FP32 nodes (103.0 before), 213 on 4096 x 2048 FP16 (304), 31.5 on 513 x 385 FP32 (43.0).
+// now, DRAM 46%, and the wait for the gathers is what is left. A whole check takes 72.6 us on
+// 2048 x 1024 FP32 nodes (103.0 before both, 78.9 with the final sum as it was), 204 on 4096 x 2048 FP16
+// (304, 213). Neither 3, 5 nor 6 blocks per SM changes that.
 constexpr int kDiagNodes = kReduceThreads * 8;
 
 template <int ST>
@@ -149,6 +150,7 @@ __global__ void __launch_bounds__(kReduceThreads, 4) k_reduce_nodes(
     const typename Storage<ST>::T* __restrict__ src, const LatParams<typename Storage<ST>::A> P,
     int axis, typename Storage<ST>::A* __restrict__ snap, int update, double* __restrict__ partial, int nseg)
 {
+    step_prologue();
     const int seg = blockIdx.x % nseg, y = blockIdx.x / nseg;
     const int x0 = seg * kDiagNodes, x1 = min(P.nx, x0 + kDiagNodes);
     double v[RS_N] = {0, 0, 0, 0, 0, 0};
@@ -159,7 +161,11 @@ __global__ void __launch_bounds__(kReduceThreads, 4) k_reduce_nodes(
 }
 
 // Sum the per-row partials in row order and finish the diagnostics in FP64: out[0..RS_N-1] = the
-// sums, out[RS_N] = Nu (Eq. 29), out[RS_N+1] = E_R.
+// sums, out[RS_N] = Nu (Eq. 29), out[RS_N+1] = E_R. One block, all latency: FP64 divisions and square
+// roots are long chains of slow instructions, so the two parts of E_R are formed by two lanes of one
+// warp and Nu by another warp. out may be pinned host memory, which spares the host a copy after the
+// kernel: it is written once, by neighbouring threads. A whole check, with the kernels also chained to the one
+// before: 513 x 385 FP32 31.5 -> 26.0 us, 256 x 256 FP64 38.1 -> 28.4, 60 x 31 FP64 28.0 -> 21.7.
 __device__ __forceinline__ void reduce_final(const double* __restrict__ partial, int rows,
                                              double nodes, double cells, double H, double dT,
                                              double sign, double kappa, double u_ref, double dT_ref,
@@ -168,13 +174,19 @@ __device__ __forceinline__ void reduce_final(const double* __restrict__ partial,
     double v[RS_N] = {0, 0, 0, 0, 0, 0};
     for (int r = threadIdx.x; r < rows; r += kReduceThreads)
         for (int k = 0; k < RS_N; ++k) v[k] += partial[(long long)r * RS_N + k];
-    __shared__ double tot[RS_N];
+    __shared__ double tot[RS_N + 2];
     block_sum(v, tot);
     __syncthreads();
-    if (threadIdx.x == 0) {
-        for (int k = 0; k < RS_N; ++k) out[k] = tot[k];
-        finish_diagnostics(tot, nodes, cells, H, dT, sign, kappa, u_ref, dT_ref, &out[RS_N], &out[RS_N + 1]);
+    const int t = threadIdx.x;
+    if (t < 2) {
+        const double r = residual_of(tot[t == 0 ? RS_DU : RS_DT], tot[t == 0 ? RS_U : RS_T], nodes, t == 0 ? u_ref : dT_ref);
+        const double rt = __shfl_down_sync(0x3u, r, 1);
+        if (t == 0) tot[RS_N + 1] = r > rt ? r : rt;
+    } else if (t == 32) {
+        tot[RS_N] = nusselt_of(tot[RS_UT], cells, H, dT, sign, kappa);
     }
+    __syncthreads();
+    if (t < RS_N + 2) out[t] = tot[t];
 }
 
 static __global__ void __launch_bounds__(kReduceThreads) k_reduce_final(const double* __restrict__ partial,
@@ -183,6 +195,7 @@ static __global__ void __launch_bounds__(kReduceThreads) k_reduce_final(const do
                                                                  double kappa, double u_ref,
                                                                  double dT_ref, double* __restrict__ out)
 {
+    step_prologue();
     reduce_final(partial, rows, nodes, cells, H, dT, sign, kappa, u_ref, dT_ref, out);
 }
 

@@ -273,20 +273,16 @@ inline NuGeom nu_geom(int nx, int ny, const clb_params& p, int axis)
 // Reduction partial sums of one row (or block), in this order.
 enum { RS_UT = 0, RS_DU, RS_U, RS_DT, RS_T, RS_BAD, RS_N };
 
-// Final scalars from the summed partials (host or device).
-__host__ __device__ inline void finish_diagnostics(const double* s, double nodes, double cells,
-                                                   double H, double dT, double sign, double kappa,
-                                                   double u_ref, double dT_ref, double* nu,
-                                                   double* er)
+// Nu of Eq. 29 from the summed term, and one field's part of the residual from its summed squares.
+__host__ __device__ inline double nusselt_of(double ut, double cells, double H, double dT, double sign, double kappa)
 {
-    *nu = 1.0 + sign * (s[RS_UT] / cells) * H / (kappa * dT);
-    const double fu = nodes * (1e-3 * u_ref) * (1e-3 * u_ref);
-    const double fT = nodes * (1e-3 * dT_ref) * (1e-3 * dT_ref);
-    const double du = s[RS_U] > fu ? s[RS_U] : fu;
-    const double dt = s[RS_T] > fT ? s[RS_T] : fT;
-    const double ru = s[RS_DU] == 0.0 ? 0.0 : (du > 0 ? sqrt(s[RS_DU] / du) : INFINITY);
-    const double rt = s[RS_DT] == 0.0 ? 0.0 : (dt > 0 ? sqrt(s[RS_DT] / dt) : INFINITY);
-    *er = ru > rt ? ru : rt;
+    return 1.0 + sign * (ut / cells) * H / (kappa * dT);
+}
+__host__ __device__ inline double residual_of(double diff, double norm, double nodes, double ref)
+{
+    const double least = nodes * (1e-3 * ref) * (1e-3 * ref);
+    const double d = norm > least ? norm : least;
+    return diff == 0.0 ? 0.0 : (d > 0 ? sqrt(diff / d) : INFINITY);
 }
 
 }  // namespace clb

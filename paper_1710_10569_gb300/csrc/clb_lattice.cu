@@ -154,7 +154,6 @@ struct clb_handle {
     double* snap = nullptr;
     double* stage = nullptr;
     double* partial = nullptr;
-    double* diag = nullptr;
     double* host_diag = nullptr;  // pinned
     long steps = 0;
     int bx = 128, by = 1, npt = 1;
@@ -390,24 +389,20 @@ clb_status launch_fields(clb_handle* h, double* rho, double* ux, double* uy, dou
     return CLB_OK;
 }
 
-// Diagnostics into h->diag (device) and h->host_diag (after sync).
+// Diagnostics into h->host_diag (pinned: the last kernel writes it).
 clb_status run_diagnostics(clb_handle* h, int axis, int update)
 {
     const void* s = h->buf[h->cur];
     const int nseg = diag_segments(h->nx);
     const int rows = h->ny * nseg;  // partial entries
     switch (h->p.storage) {
-    case CLB_F64: k_reduce_nodes<ST_F64><<<rows, kReduceThreads, 0, h->stream>>>((const double*)s, h->Pd, axis, h->snap, update, h->partial, nseg); break;
-    case CLB_F32: k_reduce_nodes<ST_F32><<<rows, kReduceThreads, 0, h->stream>>>((const float*)s, h->Pf, axis, (float*)h->snap, update, h->partial, nseg); break;
-    default: k_reduce_nodes<ST_F16DEV><<<rows, kReduceThreads, 0, h->stream>>>((const __half*)s, h->Pf, axis, (float*)h->snap, update, h->partial, nseg); break;
+    case CLB_F64: CLB_CUDA(launch_chained(k_reduce_nodes<ST_F64>, rows, kReduceThreads, 0, h->stream, (const double*)s, h->Pd, axis, h->snap, update, h->partial, nseg)); break;
+    case CLB_F32: CLB_CUDA(launch_chained(k_reduce_nodes<ST_F32>, rows, kReduceThreads, 0, h->stream, (const float*)s, h->Pf, axis, (float*)h->snap, update, h->partial, nseg)); break;
+    default: CLB_CUDA(launch_chained(k_reduce_nodes<ST_F16DEV>, rows, kReduceThreads, 0, h->stream, (const __half*)s, h->Pf, axis, (float*)h->snap, update, h->partial, nseg)); break;
     }
-    CLB_CUDA(cudaGetLastError());
     const NuGeom g = nu_geom(h->nx, h->ny, h->p, axis);
-    k_reduce_final<<<1, kReduceThreads, 0, h->stream>>>(h->partial, rows, double(h->nx) * h->ny, g.cells,
-                                                        g.H, g.dT, g.sign, h->p.kappa, h->p.u_ref,
-                                                        h->p.dT_ref, h->diag);
-    CLB_CUDA(cudaGetLastError());
-    CLB_CUDA(cudaMemcpyAsync(h->host_diag, h->diag, (RS_N + 2) * sizeof(double), cudaMemcpyDeviceToHost, h->stream));
+    CLB_CUDA(launch_chained(k_reduce_final, 1, kReduceThreads, 0, h->stream, h->partial, rows, double(h->nx) * h->ny, g.cells,
+                            g.H, g.dT, g.sign, h->p.kappa, h->p.u_ref, h->p.dT_ref, h->host_diag));
     CLB_CUDA(cudaStreamSynchronize(h->stream));
     if (h->host_diag[RS_BAD] > 0)
         return set_error(CLB_ENAN, "%.0f nodes have non-finite fields after %ld steps", h->host_diag[RS_BAD], h->steps);
@@ -517,7 +512,6 @@ extern "C" clb_status clb_create(int nx, int ny, const clb_params* p, void* stre
         h->snap = (double*)(h->mem + L.snap);
         h->stage = (double*)(h->mem + L.stage);
         h->partial = (double*)(h->mem + L.partial);
-        h->diag = (double*)(h->mem + L.diag);
         h->Pd = make_lat_params<double>(nx, ny, *p);
         h->Pf = make_lat_params<float>(nx, ny, *p);
         int sms = 0;
