@@ -348,20 +348,21 @@ public:
     }
 
     // One device allocation (and one pinned host mirror) for the member descriptors, the
-    // diagnostics outputs and the tile- and row-owner tables, at the given capacities.
-    clb_status reserve(size_t max_members, size_t max_tiles, size_t max_rows)
+    // diagnostics outputs and the tile- and row-owner tables, at the given capacities. Lattices of more
+    // than max_march windows and segments step one step per launch.
+    clb_status reserve(size_t max_members, size_t max_tiles, size_t max_rows, size_t max_march)
     {
         cap_members = std::max<size_t>(1, max_members);
         cap_tiles = std::max<size_t>(1, max_tiles);
         cap_rows = std::max<size_t>(1, max_rows);
+        cap_march = storage == CLB_F32 ? max_march : 0;
         const size_t msz = std::max(sizeof(Member<double>), sizeof(Member<float>));
         off_members = 0;
         off_diag = align256(cap_members * msz);
         off_owner = off_diag + align256(cap_members * kDiagStride * sizeof(double));
         off_rows = off_owner + align256(cap_tiles * sizeof(int));
-        // a lattice's strips and segments (of kMarchRowsMin rows or more) are at most twice its tiles
         off_march = off_rows + align256(cap_rows * sizeof(int));
-        table_bytes = off_march + (storage == CLB_F32 ? align256(2 * cap_tiles * sizeof(int)) : 0);
+        table_bytes = off_march + align256(cap_march * sizeof(int));
         cudaError_t e = cudaMalloc(&d_tables, table_bytes);
         if (e != cudaSuccess)
             return set_error(e == cudaErrorMemoryAllocation ? CLB_ENOMEM : CLB_ECUDA, "launch tables (%zu bytes): %s",
@@ -420,6 +421,7 @@ public:
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         march = march_rows_for([&](int rows) { return march_warps(rows); }, std::max(1, sms), kBatchStepUs + nodes * kBatchNodeUs);
+        if (march && (size_t)march_warps(march) > cap_march) march = 0;
     }
 
     // Rebuild the tile and row tables for the active members (no allocation, no stream sync).
@@ -436,11 +438,10 @@ public:
             }
         choose_groups();
         choose_march();
-        const long tiles = tiles_with(groups), warps = march ? march_warps(march) : 0;
+        const long tiles = tiles_with(groups);
         long rows = 0;
         for (const Lattice* L : active) rows += L->ny;
-        if (active.size() > cap_members || (size_t)tiles > cap_tiles || (size_t)rows > cap_rows ||
-            (size_t)warps > 2 * cap_tiles)
+        if (active.size() > cap_members || (size_t)tiles > cap_tiles || (size_t)rows > cap_rows)
             return set_error(CLB_ENOMEM, "batched launch tables: %zu members, %ld tiles, %ld rows exceed the reserved "
                                          "%zu, %zu, %zu", active.size(), tiles, rows, cap_members, cap_tiles, cap_rows);
         // the mirrors of the previous rebuild may still be in flight to the device
@@ -638,7 +639,7 @@ private:
     void* d_tables = nullptr;  // members | diagnostics outputs | tile owners | row owners
     void* h_tables = nullptr;  // pinned mirror of the same layout
     size_t off_members = 0, off_diag = 0, off_owner = 0, off_rows = 0, off_march = 0, table_bytes = 0;
-    size_t cap_members = 0, cap_tiles = 0, cap_rows = 0;
+    size_t cap_members = 0, cap_tiles = 0, cap_rows = 0, cap_march = 0;
     cudaEvent_t copied = nullptr;  // recorded after the last copy of the mirrors
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
 
@@ -731,7 +732,8 @@ extern "C" clb_status clb_batch_create(int n, const int* nx, const int* ny, cons
         auto b = std::make_unique<clb_batch>();
         cudaGetDevice(&b->device);
         CLB_TRY(b->E.init(storage, (cudaStream_t)stream));
-        CLB_TRY(b->E.reserve(n, max_tiles, rows));
+        // (segments of four rows or more: no more windows and segments than tiles of one row)
+        CLB_TRY(b->E.reserve(n, max_tiles, rows, max_tiles));
         CLB_CUDA(cudaMalloc((void**)&b->mem, total));
         CLB_CUDA(cudaMemsetAsync(b->mem, 0, total, b->E.stream));
         size_t off = 0;
@@ -1159,7 +1161,9 @@ extern "C" clb_status clb_serve_open(size_t hbm_budget_bytes, int max_slots, int
         // budget holds in lattices of ordinary shape; a request that would overflow them waits.
         const size_t tiles_cap = std::max<size_t>(size_t(1) << 20, hbm_budget_bytes / 16384);
         const size_t rows_cap = std::max<size_t>(size_t(1) << 18, hbm_budget_bytes / 65536);
-        CLB_TRY(s->E.reserve(max_slots, tiles_cap, rows_cap));
+        // an entry per window and segment of some 960 nodes (108 KB of populations in both buffers)
+        const size_t march_cap = std::max<size_t>(size_t(1) << 16, hbm_budget_bytes / 110000);
+        CLB_TRY(s->E.reserve(max_slots, tiles_cap, rows_cap, march_cap));
         CLB_TRY(s->pool.open(hbm_budget_bytes));
         *out = s.release();
         return CLB_OK;
