@@ -636,7 +636,7 @@ public:
 private:
     bool dirty = true;
     std::vector<Lattice*> active;
-    void* d_tables = nullptr;  // members | diagnostics outputs | tile owners | row owners
+    void* d_tables = nullptr;  // members | (diagnostics outputs: in the mirror) | tile, row and march owners
     void* h_tables = nullptr;  // pinned mirror of the same layout
     size_t off_members = 0, off_diag = 0, off_owner = 0, off_rows = 0, off_march = 0, table_bytes = 0;
     size_t cap_members = 0, cap_tiles = 0, cap_rows = 0, cap_march = 0;

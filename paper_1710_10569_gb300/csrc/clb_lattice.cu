@@ -181,7 +181,7 @@ dim3 grid_for(const clb_handle* h, int bx, int by)
 }
 
 // The split step (k_step_inner beside k_step_edge) for the FP16 form, which sits at the issue
-// limit: 83.0 -> 77.9 us per step on 4096 x 2048. The FP32 form is bound by memory (one kernel:
+// limit: 83.0 -> 77.9 us per step on 4096 x 2048 (72.9 since its collision works on halves). The FP32 form is bound by memory (one kernel:
 // 35.0 us, split: 35.2-35.6 us, the fork and join costing more than the registers save) and FP64
 // by its arithmetic (the same either way); they keep the one kernel that holds every path. So do FP16
 // lattices below kSplitNodes, where the second launch and the fork and join are the larger part of a

@@ -7,7 +7,9 @@
 // it (the first step), then pulls row r - 1 of that intermediate state and collides it (the second
 // step), so a population crosses HBM once for two steps. Every node's arithmetic is that of the
 // one-step kernels (collide_dev on packed pairs, the same pull and wall rules), so the results are
-// bitwise the same. It is then bound by the FP32 pipe (73% busy; HBM 62% at 4096 x 2048).
+// bitwise the same. It is then bound by the FP32 pipe (73% busy; HBM 62% at 4096 x 2048), and on
+// lattices that fill one round of resident warps by the wait for a row's loads (FP32 pipe 53%, HBM 61% at
+// 2048 x 1024).
 //
 // Where the intermediate state lives. The second step at row q needs, of the intermediate state, the
 // populations with e_y = 0 of row q, those with e_y = +1 of row q - 1 and those with e_y = -1 of row
@@ -20,7 +22,7 @@
 // rows takes R + 2 rows of the first step. Windows and segments overlap by that much and repeat the
 // work (6.7% and 1/R); no two warps exchange anything.
 //
-// Measured (us per step, one step per launch -> two): 2048 x 1024 34.8 -> 24.2 (86.7 GLUPS), 4096 x
+// Measured (us per step, one step per launch -> two): 2048 x 1024 34.8 -> 23.9 (87.8 GLUPS), 4096 x
 // 2048 131.8 -> 86.5 (97 GLUPS). The FP16 form moves half the bytes and is at the FP32 pipe's limit
 // with one step per launch (72.9 us at 4096 x 2048, 80.5 with two): it keeps that. Tried: the next
 // row staged by cp.async (2048 x 1024: 35.8; two more shared-memory passes per population) and by
