@@ -142,7 +142,7 @@ __device__ __forceinline__ void reduce_row(const E* __restrict__ src, const LatP
 // converted by it) and 1 per node for the tree (4 before the exchange in block_sum). It is 50% busy
 // now, DRAM 46%, and the wait for the gathers is what is left. A whole check takes 72.6 us on
 // 2048 x 1024 FP32 nodes (103.0 before both, 78.9 with the final sum as it was), 204 on 4096 x 2048 FP16
-// (304, 213). Neither 3, 5 nor 6 blocks per SM changes that.
+// (304, 213). With 5 blocks per SM: 77.4 and 205.
 constexpr int kDiagNodes = kReduceThreads * 8;
 
 template <int ST>

@@ -182,9 +182,11 @@ __device__ __forceinline__ void step_warp_nodes(const typename Storage<ST>::T* _
 // FORM: the collision form that fits the lattice's parameters (collide_form).
 // The FP32 two-node form for general rates is held at 80 registers (92 without the bound, 8 bytes of
 // spills): 24 warps per SM instead of 20, so that mid-sized lattices are one round of warps (513 x 385
-// 4.43 -> 3.93 us per step, 640 x 640 6.74 -> 6.35, 1024 x 950 16.5 -> 15.3; 512 x 512 4.88 -> 5.01).
+// 4.43 -> 3.93 us per step, 640 x 640 6.74 -> 6.35, 1024 x 950 16.5 -> 15.3; 512 x 512 4.88 -> 5.01). The
+// other forms have no bound at all: one of 1 block per SM moves the FP32 form for rates of 1 from 76 to 80
+// registers and 1024 x 950 from 13.7 to 15.1 us.
 template <int ST, int V, int FORM>
-__global__ void __launch_bounds__(256, ST == ST_F32 && V == 2 && FORM == 0 ? 3 : 1) k_step(const typename Storage<ST>::T* __restrict__ src,
+__global__ void __launch_bounds__(256, ST == ST_F32 && V == 2 && FORM == 0 ? 3 : 0) k_step(const typename Storage<ST>::T* __restrict__ src,
                                               typename Storage<ST>::T* __restrict__ dst,
                                               const LatParams<typename Storage<ST>::A> P)
 {
