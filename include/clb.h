@@ -199,8 +199,9 @@ clb_status clb_load(clb_handle *h, const void *buf, size_t bytes);
  * afterwards; it allocates one buffer-sized scratch with cudaMallocAsync) and keeps the fastest;
  * results are cached per (storage, nx, ny) for later clb_create calls. The shape never changes
  * the results (the per-node arithmetic does not depend on it). Lattices whose default takes two
- * steps per launch step one at a time, with the given shape, after clb_set_launch or
- * clb_set_pipeline; clb_autotune weighs both. */
+ * steps per launch step one at a time, with the given shape, once clb_set_launch or
+ * clb_set_pipeline has changed it (the present shape set again changes nothing), until
+ * clb_set_steps_per_launch(h, 0) or clb_autotune, which weighs both. */
 clb_status clb_set_launch(clb_handle *h, int block_x, int block_y, int nodes_per_thread);
 clb_status clb_get_launch(clb_handle *h, int *block_x, int *block_y, int *nodes_per_thread);
 clb_status clb_autotune(clb_handle *h, int *block_x, int *block_y, int *nodes_per_thread);
@@ -211,6 +212,13 @@ clb_status clb_autotune(clb_handle *h, int *block_x, int *block_y, int *nodes_pe
  * the direct kernel. clb_autotune also tries pipelined shapes and reports them here. */
 clb_status clb_set_pipeline(clb_handle *h, int stages, int rows);
 clb_status clb_get_pipeline(clb_handle *h, int *stages, int *rows);
+
+/* Time steps that a launch of clb_step advances the lattice by: 2 where the handle takes pairs of
+ * steps in one launch (an odd last step is a launch of its own), else 1. clb_set_steps_per_launch
+ * takes 1, or 0 for the library's own choice by size, storage and walls. Results do not depend on
+ * it. */
+clb_status clb_set_steps_per_launch(clb_handle *h, int steps);
+clb_status clb_get_steps_per_launch(clb_handle *h, int *steps);
 
 /* The CUDA stream the handle enqueues on (to time its work with events on that stream). */
 void *clb_stream(clb_handle *h);
@@ -254,6 +262,11 @@ void clb_thermal_destroy(clb_thermal *h);
  * [ny][nx]; NULL means T = T0, u = 0. Synchronous; resets the step count. */
 clb_status clb_thermal_init(clb_thermal *h, const double *T, const double *ux, const double *uy);
 clb_status clb_thermal_step(clb_thermal *h, long n);
+/* Time steps that a launch of clb_thermal_step advances: 4 on large FP32 and FP16 lattices (the rest of
+ * n goes one by one), else 1. clb_thermal_set_steps_per_launch takes 1, or 0 for the library's own
+ * choice. Results do not depend on it. */
+clb_status clb_thermal_set_steps_per_launch(clb_thermal *h, int steps);
+clb_status clb_thermal_get_steps_per_launch(clb_thermal *h, int *steps);
 /* T (Eq. 23) at the current time into a host array. Synchronous. */
 clb_status clb_thermal_fields(clb_thermal *h, double *T);
 /* Pre-collision populations g[5][ny][nx] at the current time. Synchronous. */
@@ -288,14 +301,18 @@ clb_status clb_batch_run(clb_batch *b, double tol, long max_steps, long interval
 clb_status clb_batch_status(clb_batch *b, int *status, double *er, long *steps, double *nu);
 /* Tile shape of the batched launch of one step: threads along x (32..256), rows (block_x * rows <=
  * 256) and nodes per thread (1, 2, 4). FP32 batches of some size without wet walls take pairs of steps
- * in one launch of its own shape, until a tile shape is set; clb_batch_autotune weighs both. Each
+ * in one launch of its own shape, until another tile shape is set; clb_batch_autotune weighs both. Each
  * block steps 1, 2, 4, ... such groups of rows one after another (it fetches its lattice's descriptor
  * once): as many as keep a block at 2048 nodes or fewer and the launch at 8 or more rounds of the
  * blocks the device holds at once. clb_batch_autotune times candidates over the whole batch (the
  * populations are restored afterwards) and keeps the fastest. Results do not depend on it. */
 clb_status clb_batch_set_tile(clb_batch *b, int tile_x, int tile_y, int nodes_per_thread);
 clb_status clb_batch_autotune(clb_batch *b, int *tile_x, int *tile_y, int *nodes_per_thread);
-/* Launch geometry of the next batched step over the active instances: tile shape, groups of rows
+/* Time steps that a launch over the active instances advances: 2 for pairs of steps, else 1.
+ * clb_batch_set_steps_per_launch takes 1, or 0 for the library's own choice. */
+clb_status clb_batch_set_steps_per_launch(clb_batch *b, int steps);
+clb_status clb_batch_get_steps_per_launch(clb_batch *b, int *steps);
+/* Launch geometry of the next launch of one step over the active instances: tile shape, groups of rows
  * per block and blocks per launch. Any pointer may be NULL. */
 clb_status clb_batch_get_launch(clb_batch *b, int *tile_x, int *tile_y, int *nodes_per_thread,
                                 int *groups, long *blocks);

@@ -159,8 +159,10 @@ clb_status clb3d_batch_init_fields(clb3d_batch* b, int k, const double* rho, con
 /* n >= 0 time steps of every lattice, enqueued on the stream. */
 clb_status clb3d_batch_step(clb3d_batch* b, long n);
 /* Steps are replayed from graphs that hold a chain of single-lattice launches per lattice, side by
- * side; the steps left over go through one launch for all lattices. Setting a tile sends every step
- * through the latter. */
+ * side (chains = 1, the default), or one launch per step for all lattices (chains = 0); the steps left
+ * over go through the latter. Setting another tile sets chains to 0. Results do not depend on it. */
+clb_status clb3d_batch_set_chains(clb3d_batch* b, int chains);
+clb_status clb3d_batch_get_chains(clb3d_batch* b, int* chains);
 /* Thread block of the batched step: block_x threads along x (a multiple of 32, <= 256) times block_y
  * rows (block_x * block_y <= 256). Each block steps 1, 2, 4, ... groups of block_y rows one after
  * another: as many as keep a block at 2048 nodes or fewer and the launch at 8 or more rounds of the

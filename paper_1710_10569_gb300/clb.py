@@ -86,6 +86,8 @@ _SIGS = {
     "clb_autotune": [_VP, _P(_I), _P(_I), _P(_I)],
     "clb_set_pipeline": [_VP, _I, _I],
     "clb_get_pipeline": [_VP, _P(_I), _P(_I)],
+    "clb_set_steps_per_launch": [_VP, _I],
+    "clb_get_steps_per_launch": [_VP, _P(_I)],
     "clb_stream": [_VP],
     "clb_buffers": [_VP, _P(_VP), _P(_VP), _P(_S), _P(_I)],
     "clb_step_partition": [_I, _I, _P(clb_params), _I, _P(_I)],
@@ -95,6 +97,8 @@ _SIGS = {
     "clb_thermal_destroy": [_VP],
     "clb_thermal_init": [_VP, _D, _D, _D],
     "clb_thermal_step": [_VP, _L],
+    "clb_thermal_set_steps_per_launch": [_VP, _I],
+    "clb_thermal_get_steps_per_launch": [_VP, _P(_I)],
     "clb_thermal_fields": [_VP, _D],
     "clb_thermal_populations": [_VP, _D],
     "clb_thermal_sync": [_VP],
@@ -107,6 +111,8 @@ _SIGS = {
     "clb_batch_run": [_VP, ctypes.c_double, _L, _L, _P(_L), _D, _P(_I)],
     "clb_batch_status": [_VP, _P(_I), _D, _P(_L), _D],
     "clb_batch_set_tile": [_VP, _I, _I, _I],
+    "clb_batch_set_steps_per_launch": [_VP, _I],
+    "clb_batch_get_steps_per_launch": [_VP, _P(_I)],
     "clb_batch_autotune": [_VP, _P(_I), _P(_I), _P(_I)],
     "clb_batch_get_launch": [_VP, _P(_I), _P(_I), _P(_I), _P(_I), _P(ctypes.c_long)],
     "clb_serve_open": [_S, _I, _I, _VP, _P(_VP)],
@@ -146,6 +152,8 @@ _SIGS = {
     "clb3d_batch_init_fields": [_VP, _I, _D, _D, _D, _D, _D],
     "clb3d_batch_step": [_VP, _L],
     "clb3d_batch_set_tile": [_VP, _I, _I],
+    "clb3d_batch_set_chains": [_VP, _I],
+    "clb3d_batch_get_chains": [_VP, _P(_I)],
     "clb3d_batch_get_launch": [_VP, _P(_I), _P(_I), _P(_I), _P(ctypes.c_longlong)],
 }
 _RESTYPES = {"clb_destroy": None, "clb_batch_destroy": None, "clb_serve_close": None,
@@ -377,6 +385,15 @@ class Lattice:
         _check(lib().clb_get_pipeline(self._h, ctypes.byref(st), ctypes.byref(rows)))
         return st.value, rows.value
 
+    def set_steps_per_launch(self, steps: int = 0):
+        """1, or 0 for the library's own choice (1 or 2)."""
+        _check(lib().clb_set_steps_per_launch(self._h, int(steps)))
+
+    def steps_per_launch(self) -> int:
+        v = _I()
+        _check(lib().clb_get_steps_per_launch(self._h, ctypes.byref(v)))
+        return v.value
+
     def buffers(self):
         """(current buffer, other buffer, elements per chunked row, nodes per chunk): element
         (i, x, y) lies at y * row_elems + (x // chunk) * 14 * chunk + i * chunk + x % chunk."""
@@ -418,6 +435,15 @@ class Thermal:
 
     def sync(self):
         _check(lib().clb_thermal_sync(self._h))
+
+    def set_steps_per_launch(self, steps: int = 0):
+        """1, or 0 for the library's own choice (1 or 4)."""
+        _check(lib().clb_thermal_set_steps_per_launch(self._h, int(steps)))
+
+    def steps_per_launch(self) -> int:
+        v = _I()
+        _check(lib().clb_thermal_get_steps_per_launch(self._h, ctypes.byref(v)))
+        return v.value
 
     def temperature(self):
         T = np.empty((self.ny, self.nx))
@@ -508,8 +534,17 @@ class Batch:
         _check(lib().clb_batch_autotune(self._h, ctypes.byref(tx), ctypes.byref(ty), ctypes.byref(npt)))
         return tx.value, ty.value, npt.value
 
+    def set_steps_per_launch(self, steps: int = 0):
+        """1, or 0 for the library's own choice (1 or 2)."""
+        _check(lib().clb_batch_set_steps_per_launch(self._h, int(steps)))
+
+    def steps_per_launch(self) -> int:
+        v = _I()
+        _check(lib().clb_batch_get_steps_per_launch(self._h, ctypes.byref(v)))
+        return v.value
+
     def launch(self) -> dict:
-        """Geometry of the next batched step: tile (threads x, threads y, nodes per thread), groups
+        """Geometry of the next launch of one step: tile (threads x, threads y, nodes per thread), groups
         of rows each block steps, and blocks per launch."""
         tx, ty, npt, groups, blocks = _I(), _I(), _I(), _I(), ctypes.c_long()
         _check(lib().clb_batch_get_launch(self._h, ctypes.byref(tx), ctypes.byref(ty), ctypes.byref(npt),
@@ -768,6 +803,15 @@ class Batch3D:
 
     def set_tile(self, block_x: int, block_y: int = 1):
         _check(lib().clb3d_batch_set_tile(self._h, int(block_x), int(block_y)))
+
+    def set_chains(self, chains: bool):
+        """Whether the graphs hold a chain of launches per lattice, or one launch per step for all."""
+        _check(lib().clb3d_batch_set_chains(self._h, int(bool(chains))))
+
+    def chains(self) -> bool:
+        v = _I()
+        _check(lib().clb3d_batch_get_chains(self._h, ctypes.byref(v)))
+        return bool(v.value)
 
     def launch(self) -> dict:
         bx, by, groups, blocks = _I(), _I(), _I(), ctypes.c_longlong()

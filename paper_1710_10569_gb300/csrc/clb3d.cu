@@ -1731,14 +1731,33 @@ extern "C" clb_status clb3d_batch_set_tile(clb3d_batch* b, int block_x, int bloc
         return set_error(CLB_EINVAL, "tile %d x %d: block_x in [32, 256] multiple of 32, block_x * block_y <= 256",
                          block_x, block_y);
     CLB_CUDA(cudaStreamSynchronize(b->stream));
+    if (block_x != b->bx || block_y != b->by) b->chains = false;  // the present tile set again changes nothing
     b->bx = block_x;
     b->by = block_y;
-    b->chains = false;
     try {
         return batch3_tables(b);
     } catch (const std::bad_alloc&) {
         return set_error(CLB_ENOMEM, "host allocation failed");
     }
+}
+
+extern "C" clb_status clb3d_batch_set_chains(clb3d_batch* b, int chains)
+{
+    CHECK_B3(b);
+    if (chains != 0 && chains != 1) return set_error(CLB_EINVAL, "chains %d: 0 or 1", chains);
+    if (b->chains == (chains == 1)) return CLB_OK;
+    CLB_CUDA(cudaStreamSynchronize(b->stream));
+    drop_batch3_graphs(b);
+    b->chains = chains == 1;
+    return CLB_OK;
+}
+
+extern "C" clb_status clb3d_batch_get_chains(clb3d_batch* b, int* chains)
+{
+    CHECK_B3(b);
+    if (!chains) return set_error(CLB_EINVAL, "chains must not be NULL");
+    *chains = b->chains ? 1 : 0;
+    return CLB_OK;
 }
 
 extern "C" clb_status clb3d_batch_get_launch(clb3d_batch* b, int* block_x, int* block_y, int* groups,

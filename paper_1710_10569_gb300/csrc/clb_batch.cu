@@ -934,11 +934,39 @@ extern "C" clb_status clb_batch_set_tile(clb_batch* b, int tile_x, int tile_y, i
                                          "tile_x * tile_y <= 256, nodes per thread 1, 2 or 4",
                              tile_x, tile_y, nodes_per_thread);
         cudaStreamSynchronize(b->E.stream);
+        // the present tile set again changes nothing
+        if (tile_x != b->E.tile_x || tile_y != b->E.tile_y || nodes_per_thread != b->E.npt) b->E.one_step = true;
         b->E.tile_x = tile_x;
         b->E.tile_y = tile_y;
         b->E.npt = nodes_per_thread;
-        b->E.one_step = true;
         b->E.mark_dirty();
+        return CLB_OK;
+    } catch (const std::bad_alloc&) {
+        return host_alloc_failed();
+    }
+}
+
+extern "C" clb_status clb_batch_set_steps_per_launch(clb_batch* b, int steps)
+{
+    try {
+        if (!b) return set_error(CLB_EINVAL, "batch is NULL");
+        if (steps != 0 && steps != 1) return set_error(CLB_EINVAL, "steps per launch %d: 1, or 0 for the library's choice", steps);
+        cudaStreamSynchronize(b->E.stream);
+        b->E.one_step = steps == 1;
+        b->E.mark_dirty();
+        return CLB_OK;
+    } catch (const std::bad_alloc&) {
+        return host_alloc_failed();
+    }
+}
+
+extern "C" clb_status clb_batch_get_steps_per_launch(clb_batch* b, int* steps)
+{
+    try {
+        if (!b) return set_error(CLB_EINVAL, "batch is NULL");
+        if (!steps) return set_error(CLB_EINVAL, "steps is NULL");
+        CLB_TRY(b->E.rebuild());
+        *steps = b->E.march > 0 ? 2 : 1;
         return CLB_OK;
     } catch (const std::bad_alloc&) {
         return host_alloc_failed();

@@ -848,12 +848,16 @@ clb_status check_launch(const clb_handle* h, const Launch& L)
     return CLB_OK;
 }
 
+bool same_shape(const Launch& a, const Launch& b)
+{
+    return a.bx == b.bx && a.by == b.by && a.npt == b.npt && a.stages == b.stages && a.rows == b.rows;
+}
+
 clb_status apply_launch(clb_handle* h, const Launch& L)
 {
     CLB_TRY(check_launch(h, L));
     const Launch c = current_launch(h);
-    if (c.bx != L.bx || c.by != L.by || c.npt != L.npt || c.stages != L.stages || c.rows != L.rows ||
-        c.march != L.march) {
+    if (!same_shape(c, L) || c.march != L.march) {
         DeviceGuard dg(h->device);
         cudaStreamSynchronize(h->stream);
         drop_graphs(h);
@@ -876,7 +880,7 @@ extern "C" clb_status clb_set_launch(clb_handle* h, int block_x, int block_y, in
     if (block_y) L.by = block_y;
     if (nodes_per_thread) L.npt = nodes_per_thread;
     if (L.npt == 1) L.stages = 0;
-    L.march = 0;
+    if (!same_shape(L, current_launch(h))) L.march = 0;  // the present shape set again changes nothing
     return apply_launch(h, L);
 }
 
@@ -886,8 +890,30 @@ extern "C" clb_status clb_set_pipeline(clb_handle* h, int stages, int rows)
     Launch L = current_launch(h);
     L.stages = stages;
     if (rows) L.rows = rows;
-    L.march = 0;
+    if (!same_shape(L, current_launch(h))) L.march = 0;
     return apply_launch(h, L);
+}
+
+extern "C" clb_status clb_set_steps_per_launch(clb_handle* h, int steps)
+{
+    CHECK_H(h);
+    if (steps != 0 && steps != 1) return set_error(CLB_EINVAL, "steps per launch %d: 1, or 0 for the library's choice", steps);
+    Launch L = current_launch(h);
+    L.march = 0;
+    if (steps == 0) {
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+        L.march = march_rows_rule(h->nx, h->ny, h->p, std::max(1, sms));
+    }
+    return apply_launch(h, L);
+}
+
+extern "C" clb_status clb_get_steps_per_launch(clb_handle* h, int* steps)
+{
+    CHECK_H(h);
+    if (!steps) return set_error(CLB_EINVAL, "steps is NULL");
+    *steps = h->march > 0 ? 2 : 1;
+    return CLB_OK;
 }
 
 extern "C" clb_status clb_get_launch(clb_handle* h, int* block_x, int* block_y, int* nodes_per_thread)

@@ -694,6 +694,35 @@ extern "C" clb_status clb_thermal_init(clb_thermal* h, const double* T, const do
     return CLB_OK;
 }
 
+extern "C" clb_status clb_thermal_set_steps_per_launch(clb_thermal* h, int steps)
+{
+    if (!h) return set_error(CLB_EINVAL, "handle is NULL");
+    if (steps != 0 && steps != 1) return set_error(CLB_EINVAL, "steps per launch %d: 1, or 0 for the library's choice", steps);
+    int march = 0;
+    if (steps == 0) {
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+        march = thermal_rows_rule(h->nx, h->ny, h->p, std::max(1, sms));
+    }
+    if (march == h->march) return CLB_OK;
+    CLB_CUDA(cudaStreamSynchronize(h->stream));
+    for (auto& g : h->graph)
+        if (g) {
+            cudaGraphExecDestroy(g);
+            g = nullptr;
+        }
+    h->march = march;
+    return CLB_OK;
+}
+
+extern "C" clb_status clb_thermal_get_steps_per_launch(clb_thermal* h, int* steps)
+{
+    if (!h) return set_error(CLB_EINVAL, "handle is NULL");
+    if (!steps) return set_error(CLB_EINVAL, "steps is NULL");
+    *steps = h->march > 0 ? kSteps : 1;
+    return CLB_OK;
+}
+
 extern "C" clb_status clb_thermal_step(clb_thermal* h, long n)
 {
     if (!h) return set_error(CLB_EINVAL, "handle is NULL");

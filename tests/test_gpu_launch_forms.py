@@ -1,0 +1,119 @@
+"""Which launch form a handle uses (one, two or four steps per launch; chains of launches per 3-D box),
+and the calls that report, change and restore it."""
+import numpy as np
+import pytest
+
+from paper_1710_10569_gb300 import workloads as W
+
+pytestmark = pytest.mark.gpu
+
+F64, F32, F16 = W.STORAGE_F64, W.STORAGE_F32, W.STORAGE_F16DEV
+P, D, A, WET = W.WALL_PERIODIC, W.WALL_DIRICHLET, W.WALL_ADIABATIC, W.WALL_WET
+LAYOUTS = {"periodic": (P, P, P, P), "layer": (P, P, D, D), "box": (D, A, A, D), "cavity": (D, D, A, A), "sides": (A, D, P, P)}
+
+
+@pytest.fixture(scope="module")
+def clb():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    from paper_1710_10569_gb300 import clb as c
+    return c
+
+
+# The sizes at which test_gpu_two_steps compares several steps per launch with one: the default arm
+# does take them, and an explicit shape does not.
+@pytest.mark.parametrize("layout", sorted(LAYOUTS))
+def test_sizes_compared_elsewhere_take_several_steps(clb, layout):
+    for nx, ny in [(53, 19001), (60, 17003), (59, 17200), (118, 8701), (121, 9002), (1001, 1003), (2048, 517), (30011, 41)]:
+        lat = clb.Lattice(nx, ny, W.default_params(storage=F32, wall=LAYOUTS[layout]))
+        assert lat.steps_per_launch() == 2, (nx, ny)
+        lat.set_launch(128, 1, 2)
+        assert lat.steps_per_launch() == 1, (nx, ny)
+        lat.close()
+    for nx, ny in [(8193, 49), (4096, 101), (1121, 358), (112, 3601), (55, 7301), (703, 702)]:
+        h = clb.Thermal(nx, ny, W.default_params(storage=F32 if (nx + ny) % 2 == 0 else F16, wall=LAYOUTS[layout]))
+        assert h.steps_per_launch() == 4, (nx, ny)
+        h.set_steps_per_launch(1)
+        assert h.steps_per_launch() == 1
+        h.set_steps_per_launch(0)
+        assert h.steps_per_launch() == 4
+        with pytest.raises(clb.CLBError):
+            h.set_steps_per_launch(2)
+        h.close()
+
+
+@pytest.mark.parametrize("sizes", [[(512, 512), (61, 70), (333, 129), (64, 64), (2, 3), (120, 900)], [(700, 700)],
+                                   [(60, 35)] * 230, [(1025, 31)] * 15 + [(59, 300)] * 9], ids=["mixed", "one", "many", "wide"])
+def test_batches_compared_elsewhere_take_two_steps(clb, sizes):
+    b = clb.Batch([W.random_problem(nx, ny, seed=k, storage=F32) for k, (nx, ny) in enumerate(sizes)])
+    assert b.steps_per_launch() == 2
+    b.set_tile(*b.launch()["tile"])  # as it is: nothing changes
+    assert b.steps_per_launch() == 2
+    b.set_tile(64, 2, 2)
+    assert b.steps_per_launch() == 1
+    b.set_steps_per_launch(0)
+    assert b.steps_per_launch() == 2 and b.launch()["tile"] == (64, 2, 2)
+    b.set_steps_per_launch(1)
+    assert b.steps_per_launch() == 1
+    with pytest.raises(clb.CLBError):
+        b.set_steps_per_launch(3)
+    b.close()
+
+
+def test_forms_not_taken(clb):
+    for nx, ny, storage, walls in [(1200, 1200, F64, LAYOUTS["layer"]), (1200, 1200, F16, LAYOUTS["layer"]), (64, 64, F32, LAYOUTS["layer"]),
+                                   (1200, 1200, F32, (P, P, WET, WET)), (1200, 1200, F32, (WET, WET, P, P))]:
+        lat = clb.Lattice(nx, ny, W.default_params(storage=storage, wall=walls))
+        assert lat.steps_per_launch() == 1
+        lat.set_steps_per_launch(0)
+        assert lat.steps_per_launch() == 1
+        lat.close()
+
+
+def test_lattice_form_survives_calls_that_change_nothing(clb):
+    prob = W.random_problem(1100, 1000, seed=3, storage=F32, walls=LAYOUTS["cavity"])
+    lat = clb.Lattice.from_problem(prob)
+    lat.set_launch()
+    lat.set_launch(*lat.launch())
+    lat.set_pipeline(*lat.pipeline())
+    lat.set_pipeline(0)
+    assert lat.steps_per_launch() == 2
+    lat.step(35)
+    ref = lat.fields()
+    shape = lat.launch()
+    lat.set_launch(128, 2, 2)
+    assert lat.steps_per_launch() == 1 and lat.launch() == (128, 2, 2)
+    lat.set_steps_per_launch(0)
+    assert lat.steps_per_launch() == 2
+    lat.set_launch(*shape)
+    lat.set_steps_per_launch(1)
+    lat.init_fields(*prob.fields())
+    lat.step(35)
+    assert lat.steps_per_launch() == 1
+    for x, y in zip(lat.fields(), ref):
+        assert np.array_equal(x, y)
+    with pytest.raises(clb.CLBError):
+        lat.set_steps_per_launch(2)
+    lat.close()
+
+
+def test_3d_batch_form_survives_the_present_tile(clb):
+    b = clb.Batch3D([W.random_problem3d(20 + k, 18, 16, seed=k, storage=F32) for k in range(4)])
+    assert b.chains()
+    b.set_tile(*b.launch()["block"])
+    assert b.chains()
+    b.step(33)
+    ref = [b.fields(k) for k in range(4)]
+    b.set_tile(64, 2)
+    assert not b.chains()
+    for chains in (True, False):
+        b.set_chains(chains)
+        assert b.chains() == chains
+        for k in range(4):
+            b.init_fields(k, *b.problems[k].fields())
+        b.step(33)
+        for k in range(4):
+            for x, y in zip(b.fields(k), ref[k]):
+                assert np.array_equal(x, y), (chains, k)
+    b.close()
