@@ -188,3 +188,19 @@ def test_default_batch_form_is_not_the_slower_one(clb, size, walls, rates):
     b.set_steps_per_launch(1)
     assert us <= 1.05 * step_us(b)
     b.close()
+
+
+# Lattices just above the size at which two steps per launch begin: the default is not the slower form.
+@pytest.mark.parametrize("rates", [1.0, 1.2])
+@pytest.mark.parametrize("size,walls,steps", [((1024, 1024), "cavity", 1), ((1024, 1024), "layer", 2), ((2048, 512), "cavity", 2),
+                                              ((60, 17003), "cavity", 2), ((1100, 1000), "cavity", 2), ((17003, 60), "cavity", 2)])
+def test_default_lattice_form_is_not_the_slower_one(clb, size, walls, steps, rates):
+    prob = W.random_problem(*size, seed=1, storage=F32, walls=LAYOUTS[walls])
+    prob.params.update(s_3=rates, s_4=rates, lambda2=rates)
+    prob.T, prob.ux, prob.uy = 0.1 * prob.T, 0.1 * prob.ux, 0.1 * prob.uy
+    lat = clb.Lattice.from_problem(prob)
+    assert lat.steps_per_launch() == steps
+    us = step_us(lat)
+    lat.set_steps_per_launch(1)
+    assert us <= 1.01 * step_us(lat)
+    lat.close()
