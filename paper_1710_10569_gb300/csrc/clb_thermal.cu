@@ -554,12 +554,23 @@ MarchGeom thermal_geom(int nx, int ny, int rows)
 // resident warps is taken, counting two rounds at least: warps that all start together load and
 // compute in step, and one round runs at half the rate (2048 x 2048: one of 22 rows 17.2 us per step,
 // two of 12 to 14 rows 14.7 - 15.2; 4096 x 4096: two of 44 rows 45.9, three of 28 46.8).
+// Between x walls the windows next to them, which take the wall rules every turn, end last, the more so for
+// lambda2 other than 1 and in the FP16 form; rows of three windows and more need more nodes for that to pay
+// (us per step, one step per launch against four): FP32 640 x 640 3.6 / 4.1, 1024 x 1024 6.2 / 6.5, 300 x 2000 5.5 / 5.3,
+// 1500 x 1000 8.4 / 7.2; lambda2 = 1.3 1024 x 1024 6.2 / 7.0, 500 x 3000 9.2 / 9.8, 1800 x 1200 14.7 / 11.5; FP16 1024 x 1024
+// 6.2 / 6.6, 1500 x 1000 8.1 / 7.8; lambda2 = 1.3 1800 x 1200 11.0 / 11.9, 2048 x 2048 24.6 / 18.6. Narrower rows
+// gain at any size (100 x 6000 FP32 7.9 / 6.0, lambda2 = 1.3 7.9 / 6.3).
 constexpr long long kMarchNodesT = 400000;
+constexpr long long kMarchNodesTWalls[2][2] = {{1200000, 2000000}, {1200000, 3000000}};  // FP32, FP16; lambda2 = 1, other
 int thermal_rows_rule(int nx, int ny, const clb_params& p, int sms)
 {
     const bool wet = p.wall[0] == CLB_WALL_WET || p.wall[2] == CLB_WALL_WET;
     if (p.storage == CLB_F64 || wet || (long long)nx * ny < kMarchNodesT || ny < 24) return 0;
-    if ((double)nx < 0.7 * kMarchOutT * thermal_geom(nx, ny, 6).strips) return 0;
+    const int strips = thermal_geom(nx, ny, 6).strips;
+    if ((double)nx < 0.7 * kMarchOutT * strips) return 0;
+    if (p.wall[0] != CLB_PERIODIC && strips > 2 &&
+        (long long)nx * ny < kMarchNodesTWalls[p.storage == CLB_F16DEV][p.lambda2 != 1.0])
+        return 0;
     int best = 6;
     long long least = 1LL << 60;
     for (int rows = 6; rows <= 64; ++rows) {

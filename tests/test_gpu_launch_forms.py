@@ -47,7 +47,9 @@ def test_sizes_compared_elsewhere_take_several_steps(clb, layout):
         lat.set_launch(128, 1, 2)
         assert lat.steps_per_launch() == 1, (nx, ny)
         lat.close()
-    for nx, ny in [(8193, 49), (4096, 101), (1121, 358), (112, 3601), (55, 7301), (703, 702)]:
+    # (between x walls, wider rows take four steps from more nodes on: see the next test)
+    wide = [] if LAYOUTS[layout][0] != P else [(8193, 49), (4096, 101), (1121, 358), (703, 702)]
+    for nx, ny in wide + [(112, 3601), (55, 7301)]:
         h = clb.Thermal(nx, ny, W.default_params(storage=F32 if (nx + ny) % 2 == 0 else F16, wall=LAYOUTS[layout]))
         assert h.steps_per_launch() == 4, (nx, ny)
         h.set_steps_per_launch(1)
@@ -57,6 +59,46 @@ def test_sizes_compared_elsewhere_take_several_steps(clb, layout):
         with pytest.raises(clb.CLBError):
             h.set_steps_per_launch(2)
         h.close()
+
+
+def thermal(clb, nx, ny, storage, walls, lambda2):
+    p = W.default_params(nu=0.05, kappa=0.03, storage=storage, wall=LAYOUTS[walls], T_wall=(0.3, -0.2, 0.5, -0.4), lambda2=lambda2,
+                         u_wall=((0, 0.02), (0, 0.01), (0.02, 0.03), (0.01, -0.02)))
+    rng = np.random.default_rng(nx)
+    h = clb.Thermal(nx, ny, p)
+    h.init(*(a * (rng.random((ny, nx)) - 0.5) for a in (1.0, 0.2, 0.2)))
+    return h
+
+
+@pytest.mark.parametrize("storage", [F32, F16])
+@pytest.mark.parametrize("walls", ["box", "cavity", "sides"])
+@pytest.mark.parametrize("lambda2", [1.0, 1.3])
+def test_four_thermal_steps_between_x_walls(clb, walls, lambda2, storage):
+    """Rows of many windows between x walls, of the size from which they take four steps per launch:
+    bitwise equal to one step per launch."""
+    got = []
+    for steps in (4, 1):
+        h = thermal(clb, 2051, 1501, storage, walls, lambda2)
+        if steps == 1:
+            h.set_steps_per_launch(1)
+        assert h.steps_per_launch() == steps
+        h.step(9)
+        got.append(h.populations())
+        h.close()
+    assert np.isfinite(got[0]).all() and np.array_equal(*got)
+
+
+# Four steps per launch between x walls took up to 1.18 times as long as one on lattices of 0.4 to 2 million
+# nodes (3% for the timing and the sizes next to the line).
+@pytest.mark.parametrize("storage", [F32, F16])
+@pytest.mark.parametrize("lambda2", [1.0, 1.3])
+@pytest.mark.parametrize("shape", [(640, 640), (1024, 1024), (1500, 1000), (100, 6000), (2048, 2048)], ids=lambda s: "%dx%d" % s)
+def test_default_thermal_form_is_not_the_slower_one(clb, shape, lambda2, storage):
+    h = thermal(clb, *shape, storage, "cavity", lambda2)
+    us = step_us(h)
+    h.set_steps_per_launch(1)
+    assert us <= 1.03 * step_us(h)
+    h.close()
 
 
 MIXED = [(512, 512), (61, 70), (333, 129), (64, 64), (2, 3), (120, 900)]
