@@ -441,8 +441,10 @@ clb_status take_snapshot(clb_handle* h)
 // and FP16: two and four nodes per thread, the packed instructions' and the widest loads' count, where
 // the lattice fills the chip with them; below, more and shorter warps (128 x 128, FP16: 1.9 us against
 // 3.4). Blocks of few warps, so that a ragged row end idles few of them (513 x 385, FP32: 4.3 us at
-// 128 x 1, 3.7 at 32 x 2; 640 x 640, FP16: 6.5 and 5.7); large FP32 rows that fill blocks of two warps take
-// them side by side (1024 x 950: 13.6 us against 13.8; 701 x 699, which fills eleven warps: 7.4 and 7.0).
+// 128 x 1, 3.7 at 32 x 2; 640 x 640, FP16: 6.5 and 5.7); large FP32 rows that fill blocks of two warps
+// to the last node take them side by side, at 64 x 1 (1024 x 950: 14.0 us against 14.2, 1280 x 700 12.4 and
+// 12.6, 896 x 1000 12.5 and 12.6), all others do not, whatever the number of their warps (200 x 4000: 18.2
+// and 16.3, 600 x 700 6.9 and 6.5, 1000 x 700 9.6 and 9.4, 701 x 699 7.8 and 7.1; 30 sizes measured).
 void default_shape(int storage, int nx, int ny, int sms, int* bx, int* by, int* npt)
 {
     const long long nodes = (long long)nx * ny;
@@ -462,7 +464,7 @@ void default_shape(int storage, int nx, int ny, int sms, int* bx, int* by, int* 
     *npt = small ? 1 : 2;
     if (small) *by = 4;
     if (storage == CLB_F16DEV && nodes >= kSplitNodes) *npt = 4;
-    if (storage == CLB_F32 && nodes >= kSplitNodes && (nx + 63) / 64 % 2 == 0) {
+    if (storage == CLB_F32 && nodes >= kSplitNodes && nx % 128 == 0) {
         *bx = 64;
         *by = 1;
     }

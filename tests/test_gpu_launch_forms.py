@@ -246,3 +246,19 @@ def test_default_lattice_form_is_not_the_slower_one(clb, size, walls, steps, rat
     lat.set_steps_per_launch(1)
     assert us <= 1.01 * step_us(lat)
     lat.close()
+
+
+# Large FP32 lattices: blocks of two warps side by side only where the rows fill them (they took up to 1.11
+# times as long elsewhere).
+@pytest.mark.parametrize("size", [(200, 4000), (600, 700), (1000, 700), (701, 699), (1024, 950)], ids=lambda s: "%dx%d" % s)
+def test_default_block_is_not_the_slower_one(clb, size):
+    prob = W.random_problem(*size, seed=1, storage=F32, walls=LAYOUTS["layer"])
+    prob.params.update(s_3=1.0, s_4=1.0, lambda2=1.0)
+    prob.T, prob.ux, prob.uy = 0.1 * prob.T, 0.1 * prob.ux, 0.1 * prob.uy
+    lat = clb.Lattice.from_problem(prob)
+    assert lat.launch() == ((64, 1, 2) if size[0] % 128 == 0 else (32, 2, 2))
+    us = step_us(lat)
+    for shape in ((64, 1, 2), (32, 2, 2)):
+        lat.set_launch(*shape)
+        assert us <= 1.02 * step_us(lat), shape
+    lat.close()
