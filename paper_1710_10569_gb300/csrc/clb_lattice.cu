@@ -352,13 +352,13 @@ clb_status launch_step(clb_handle* h, int from, cudaStream_t s, const Launch& L)
     return CLB_OK;
 }
 
-clb_status build_graph(clb_handle* h, int start)
+// A graph of `steps` steps (an even number of launches) of launch shape L from buffer `start`.
+clb_status capture_steps(clb_handle* h, int start, const Launch& L, int steps, cudaGraphExec_t* out)
 {
     CLB_CUDA(cudaStreamBeginCapture(h->cap, cudaStreamCaptureModeThreadLocal));
     clb_status st = CLB_OK;
-    const Launch L = current_launch(h);
-    const int per = L.march > 0 ? 2 : 1;  // steps per launch; kGraphChunk / per launches are an even number
-    for (int k = 0; k < kGraphChunk / per && st == CLB_OK; ++k)
+    const int per = L.march > 0 ? 2 : 1;  // steps per launch
+    for (int k = 0; k < steps / per && st == CLB_OK; ++k)
         st = per == 2 ? launch_two(h, start ^ (k & 1), h->cap, L) : launch_step(h, start ^ (k & 1), h->cap, L);
     cudaGraph_t g = nullptr;
     cudaError_t e = cudaStreamEndCapture(h->cap, &g);
@@ -367,10 +367,15 @@ clb_status build_graph(clb_handle* h, int start)
         return st;
     }
     if (e != cudaSuccess) return set_error(CLB_ECUDA, "graph capture: %s", cudaGetErrorString(e));
-    e = cudaGraphInstantiate(&h->graph[start], g, 0);
+    e = cudaGraphInstantiate(out, g, 0);
     cudaGraphDestroy(g);
     if (e != cudaSuccess) return set_error(CLB_ECUDA, "graph instantiate: %s", cudaGetErrorString(e));
     return CLB_OK;
+}
+
+clb_status build_graph(clb_handle* h, int start)
+{
+    return capture_steps(h, start, current_launch(h), kGraphChunk, &h->graph[start]);
 }
 
 clb_status launch_init(clb_handle* h, const double* rho, const double* ux, const double* uy,
@@ -956,41 +961,66 @@ extern "C" clb_status clb_autotune(clb_handle* h, int* block_x, int* block_y, in
         void* save = nullptr;
         CLB_CUDA(cudaMallocAsync(&save, bb, h->stream));
         CLB_CUDA(cudaMemcpyAsync(save, h->buf[h->cur], bb, cudaMemcpyDeviceToDevice, h->stream));
-        std::vector<Launch> cands;
-        const int shapes[][2] = {{64, 1}, {128, 1}, {256, 1}, {32, 4}, {64, 2}, {128, 2}};
+        // the untuned default first: another shape replaces it only by a clear margin
+        int sms = 0;
+        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
+        sms = std::max(1, sms);
+        std::vector<Launch> cands(1, Launch{128, 1, 1, 0, 8, 0});
+        default_shape(h->p.storage, h->nx, h->ny, sms, &cands[0].bx, &cands[0].by, &cands[0].npt);
+        cands.push_back(current_launch(h));
+        cands[1].march = 0;
+        const int shapes[][2] = {{64, 1}, {128, 1}, {256, 1}, {32, 1}, {32, 2}, {32, 4}, {64, 2}, {128, 2}};
         for (int npt : {1, 2, 4})
             for (auto& sh : shapes) cands.push_back({sh[0], sh[1], npt, 0, 8, 0});
         for (int npt : {2, 4})
             for (int st : {2, 3, 4})
                 for (int rows : {4, 8, 16}) cands.push_back({128, 1, npt, st, rows, 0});
-        int sms = 0;
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-        if (const int rows = march_rows_rule(h->nx, h->ny, h->p, std::max(1, sms)))
-            cands.push_back({128, 1, 2, 0, 8, rows});  // two steps per launch
         cudaEvent_t e0, e1;
         cudaEventCreate(&e0);
         cudaEventCreate(&e1);
-        float best = 1e30f;
-        Launch bl = current_launch(h);
-        const int reps = 10;
         clb_status st = CLB_OK;
-        for (const Launch& c : cands) {
-            if (c.bx * c.npt > 2 * h->nx + 64 && c.bx * c.npt > 64) continue;  // far wider than the lattice
-            if (c.stages > 0 && check_launch(h, c) != CLB_OK) continue;
-            const int per = c.march > 0 ? 2 : 1;  // steps per launch
-            const auto launch = [&](int from) { return per == 2 ? launch_two(h, from, h->stream, c) : launch_step(h, from, h->stream, c); };
-            for (int k = 0; k < 4 && st == CLB_OK; ++k) st = launch((h->cur + k) & 1);
-            cudaEventRecord(e0, h->stream);
-            for (int k = 0; k < reps / per && st == CLB_OK; ++k) st = launch((h->cur + k) & 1);
-            cudaEventRecord(e1, h->stream);
-            if (st != CLB_OK) break;
-            cudaEventSynchronize(e1);
-            float ms = 0;
-            cudaEventElapsedTime(&ms, e0, e1);
-            if (ms < best) {
+        // time of a graph of 12 steps (60 on small lattices, whose launches are short), as clb_step replays them:
+        // the lesser of two runs after an untimed one (large lattices: one)
+        const long long nodes = (long long)h->nx * h->ny;
+        const int steps = nodes < 300000 ? 60 : 12, runs = nodes < 2000000 ? 2 : 1;
+        const auto time_of = [&](const Launch& c) {
+            float least = 1e30f;
+            cudaGraphExec_t g = nullptr;
+            st = capture_steps(h, h->cur, c, steps, &g);
+            if (st != CLB_OK) return least;
+            cudaError_t e = cudaGraphLaunch(g, h->stream);
+            for (int k = 0; k < runs && e == cudaSuccess; ++k) {
+                cudaEventRecord(e0, h->stream);
+                e = cudaGraphLaunch(g, h->stream);
+                cudaEventRecord(e1, h->stream);
+                if (e == cudaSuccess) e = cudaEventSynchronize(e1);
+                float ms = 0;
+                if (e == cudaSuccess) e = cudaEventElapsedTime(&ms, e0, e1);
+                if (e == cudaSuccess) least = std::min(least, ms);
+            }
+            cudaGraphExecDestroy(g);
+            if (e != cudaSuccess) st = set_error(CLB_ECUDA, "autotune: %s", cudaGetErrorString(e));
+            return least;
+        };
+        Launch bl = cands[0];
+        const float base = time_of(bl);
+        float best = base;
+        for (size_t k = 1; k < cands.size() && st == CLB_OK; ++k) {
+            const Launch& c = cands[k];
+            if (same_shape(c, cands[0]) || (k > 1 && same_shape(c, cands[1]))) continue;
+            if (k > 1 && c.bx * c.npt > 2 * h->nx + 64 && c.bx * c.npt > 64) continue;  // far wider than the lattice
+            if (check_launch(h, c) != CLB_OK) continue;
+            const float ms = time_of(c);
+            if (ms < best && ms < 0.98f * base) {
                 best = ms;
                 bl = c;
             }
+        }
+        // two steps per launch, where the rule takes them (odd steps in the shape found)
+        if (const int rows = march_rows_rule(h->nx, h->ny, h->p, sms); rows > 0 && st == CLB_OK) {
+            Launch two = bl;
+            two.march = rows;
+            if (time_of(two) < best) bl = two;
         }
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);

@@ -262,3 +262,19 @@ def test_default_block_is_not_the_slower_one(clb, size):
         lat.set_launch(*shape)
         assert us <= 1.02 * step_us(lat), shape
     lat.close()
+
+
+# The autotuner times the default it replaces, and two steps per launch at any width: what it picks is no
+# slower than the untuned handle (it lacked the default blocks, and two steps on narrow lattices).
+@pytest.mark.parametrize("size,storage", [((256, 256), F64), ((60, 17003), F32), ((90, 12000), F32), ((701, 699), F32), ((640, 640), F16),
+                                          ((2048, 600), F32)], ids=str)
+def test_tuned_shape_is_not_the_slower_one(clb, size, storage):
+    prob = W.random_problem(*size, seed=1, storage=storage, walls=LAYOUTS["layer"])
+    prob.T, prob.ux, prob.uy = 0.1 * prob.T, 0.1 * prob.ux, 0.1 * prob.uy
+    lat = clb.Lattice.from_problem(prob)
+    steps = lat.steps_per_launch()
+    us = step_us(lat)
+    shape = lat.autotune()
+    assert lat.launch() == shape and lat.steps_per_launch() == steps
+    assert step_us(lat) <= 1.03 * us
+    lat.close()
