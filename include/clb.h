@@ -196,8 +196,10 @@ clb_status clb_load(clb_handle *h, const void *buf, size_t bytes);
  * current value. Defaults: by storage and size, 1 (FP64, and small lattices) to 4 nodes per thread (large
  * FP16 ones).
  * clb_autotune times candidate shapes on the live lattice (the populations are restored
- * afterwards; it allocates one buffer-sized scratch with cudaMallocAsync) and keeps the fastest;
- * results are cached per (storage, nx, ny) for later clb_create calls. The shape never changes
+ * afterwards; it allocates one buffer-sized scratch with cudaMallocAsync) and keeps the default unless
+ * another is faster by 2%; results are cached for later clb_create calls with the same device, storage,
+ * extents, kind of walls on either axis (periodic, wet, other) and kind of rates (high-order rates of 1 or
+ * not). The shape never changes
  * the results (the per-node arithmetic does not depend on it). Lattices whose default takes two
  * steps per launch step one at a time, with the given shape, once clb_set_launch or
  * clb_set_pipeline has changed it (the present shape set again changes nothing), until

@@ -475,8 +475,16 @@ void default_shape(int storage, int nx, int ny, int sms, int* bx, int* by, int* 
     }
 }
 
+// Tuned launches by all that decides which is fastest: device, storage, extents, the kind of walls on either
+// axis (periodic, wet, other) and the collision form.
+using TuneKey = std::tuple<int, int, int, int, int, int, int>;
+TuneKey tune_key(int device, int nx, int ny, const clb_params& p)
+{
+    const auto kind = [](int w) { return w == CLB_PERIODIC ? 0 : w == CLB_WALL_WET ? 2 : 1; };
+    return TuneKey(device, p.storage, nx, ny, kind(p.wall[0]), kind(p.wall[2]), collide_form(p));
+}
 std::mutex g_tune_mu;
-std::map<std::tuple<int, int, int>, std::array<int, 6>> g_tune_cache;
+std::map<TuneKey, std::array<int, 6>> g_tune_cache;
 
 }  // namespace
 
@@ -543,15 +551,14 @@ extern "C" clb_status clb_create(int nx, int ny, const clb_params* p, void* stre
         h->march = march_rows_rule(nx, ny, *p, std::max(1, sms));
         {
             std::lock_guard<std::mutex> lk(g_tune_mu);
-            auto it = g_tune_cache.find(std::make_tuple(p->storage, nx, ny));
+            auto it = g_tune_cache.find(tune_key(h->device, nx, ny, *p));
             if (it != g_tune_cache.end()) {
                 h->bx = it->second[0];
                 h->by = it->second[1];
                 h->npt = it->second[2];
                 h->pipe_stages = it->second[3];
                 h->pipe_rows = it->second[4];
-                // two steps per launch only where these walls allow it (the cache knows sizes alone)
-                if (h->march > 0) h->march = it->second[5];
+                h->march = it->second[5];
             }
         }
         // the padding of each row's last chunk is never read, but keep it defined
@@ -1032,7 +1039,7 @@ extern "C" clb_status clb_autotune(clb_handle* h, int* block_x, int* block_y, in
         CLB_TRY(apply_launch(h, bl));
         {
             std::lock_guard<std::mutex> lk(g_tune_mu);
-            g_tune_cache[std::make_tuple(h->p.storage, h->nx, h->ny)] = {bl.bx, bl.by, bl.npt, bl.stages, bl.rows, bl.march};
+            g_tune_cache[tune_key(h->device, h->nx, h->ny, h->p)] = {bl.bx, bl.by, bl.npt, bl.stages, bl.rows, bl.march};
         }
         if (block_x) *block_x = bl.bx;
         if (block_y) *block_y = bl.by;

@@ -278,3 +278,23 @@ def test_tuned_shape_is_not_the_slower_one(clb, size, storage):
     assert lat.launch() == shape and lat.steps_per_launch() == steps
     assert step_us(lat) <= 1.03 * us
     lat.close()
+
+
+# The tuner's choice for a lattice with wet walls, which the two-step kernel does not know, is not that of a
+# lattice of the same size without them; nor is that of the other kind of rates.
+def test_tuned_shapes_are_kept_by_walls_and_rates(clb):
+    nx, ny = 2048, 604
+    wet = clb.Lattice(nx, ny, W.default_params(storage=F32, wall=(P, P, WET, WET)))
+    wet.autotune()
+    wet.close()
+    lat = clb.Lattice(nx, ny, W.default_params(storage=F32, wall=LAYOUTS["layer"]))
+    assert lat.steps_per_launch() == 2
+    shape = lat.autotune()
+    assert lat.steps_per_launch() == 2
+    lat.close()
+    again = clb.Lattice(nx, ny, W.default_params(storage=F32, wall=LAYOUTS["layer"]))
+    assert again.launch() == shape and again.steps_per_launch() == 2
+    again.close()
+    general = clb.Lattice(nx, ny, W.default_params(storage=F32, wall=LAYOUTS["layer"], s_3=1.2))
+    assert general.launch() == (64, 1, 2) and general.steps_per_launch() == 2
+    general.close()
