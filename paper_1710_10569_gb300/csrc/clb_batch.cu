@@ -10,6 +10,7 @@
 #include <deque>
 #include <map>
 #include <memory>
+#include <utility>
 #include <vector>
 
 #include "clb_diag.cuh"
@@ -226,6 +227,7 @@ struct Lattice {
     double nu = 0, er = INFINITY;
     int status = CLB_OK;
     bool active = true;
+    MarchGeom march{};  // its windows in the two-step launch (one row per segment; set by carve)
 };
 
 size_t lattice_bytes(int nx, int ny, int storage)
@@ -240,6 +242,7 @@ void carve(Lattice& L, char* base)
     const size_t N = (size_t)L.nx * L.ny;
     const size_t bb = buffer_slot_bytes(L.nx, L.ny, L.p.storage);
     L.mem = base;
+    L.march = march_geom(L.nx, L.ny, 1);
     L.buf[0] = base;
     L.buf[1] = base + bb;
     L.snap = (double*)(base + 2 * bb);
@@ -261,9 +264,8 @@ Member<A> make_member(const Lattice& L, int tile_x, int npt, int tile_begin, int
     m.tiles_x = (L.nx + tile_x * npt - 1) / (tile_x * npt);
     m.tile_begin = tile_begin;
     m.row_begin = row_begin;
-    const MarchGeom mg = march_geom(L.nx, L.ny, 1);
-    m.strip_width = mg.width;
-    m.strips = mg.strips;
+    m.strip_width = L.march.width;
+    m.strips = L.march.strips;
     m.march_begin = march_begin;
     m.axis = L.axis;
     const NuGeom g = nu_geom(L.nx, L.ny, L.p, L.axis);
@@ -408,11 +410,26 @@ public:
         for (int g = 2; g * threads * npt <= kBlockNodes && tiles_with(g) >= kMinWaves * resident; g *= 2) groups = g;
     }
 
+    // Warps of the two-step launch for segments of so many rows, from march_strips: the numbers of windows
+    // per row, summed over the active lattices of equal numbers of rows. march_rows_for asks for 61 numbers of
+    // rows at every change of membership, which took most of its time while it went through all lattices (256
+    // lattices: 57 us with no two-step launch, 148 with all lattices counted, 65 so).
     long march_warps(int rows) const
     {
         long t = 0;
-        for (const Lattice* L : active) t += march_geom(L->nx, L->ny, rows).warps();
+        for (const auto& [ny, strips] : march_strips) t += strips * ((ny + rows - 1) / rows);
         return t;
+    }
+    void count_strips()
+    {
+        march_strips.clear();
+        strips_of.assign(kCountedRows + 1, 0);
+        for (const Lattice* L : active) {
+            if (L->ny > kCountedRows) march_strips.emplace_back(L->ny, L->march.strips);
+            else strips_of[L->ny] += L->march.strips;
+        }
+        for (int ny = 0; ny <= kCountedRows; ++ny)
+            if (strips_of[ny]) march_strips.emplace_back(ny, strips_of[ny]);
     }
 
     // Rows per segment of the two-step launch, 0 for one step per launch: the rule of a single lattice
@@ -439,6 +456,7 @@ public:
         int dev = 0, sms = 1;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        count_strips();
         march = march_rows_for([&](int rows) { return march_warps(rows); }, std::max(1, sms), limit);
         if (march && (size_t)march_warps(march) > cap_march) march = 0;
     }
@@ -485,7 +503,7 @@ public:
             std::fill(owner + t, owner + t + tx * ty, int(k));
             std::fill(row_owner + r, row_owner + r + L.ny, int(k));
             if (march) {
-                const int n = march_geom(L.nx, L.ny, march).warps();
+                const int n = L.march.strips * ((L.ny + march - 1) / march);
                 std::fill(march_owner + mw, march_owner + mw + n, int(k));
                 mw += n;
             }
@@ -655,6 +673,9 @@ public:
 private:
     bool dirty = true;
     std::vector<Lattice*> active;
+    static constexpr int kCountedRows = 1024;        // lattices of more rows are listed one by one
+    std::vector<std::pair<int, long>> march_strips;  // (rows, windows per row) of the active lattices
+    std::vector<long> strips_of;
     void* d_tables = nullptr;  // members | (diagnostics outputs: in the mirror) | tile, row and march owners
     void* h_tables = nullptr;  // pinned mirror of the same layout
     size_t off_members = 0, off_diag = 0, off_owner = 0, off_rows = 0, off_march = 0, table_bytes = 0;
