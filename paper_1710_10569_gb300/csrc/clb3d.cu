@@ -27,7 +27,6 @@
 #include <cstring>
 #include <new>
 #include <vector>
-#include <cstddef>
 
 #include "../../include/clb3d.h"
 #include "clb_core.cuh"
@@ -447,7 +446,6 @@ struct Member3 {
     void* buf[2];
     int xblocks;     // blocks along x
     int tile_begin;  // the lattice's first block
-    int flip;        // the lattice's current state is in buf[parity ^ flip]
     int high1;       // s_3 = s_4 = s_5 = s_6 = 1: the collision form that skips those moments
 };
 
@@ -479,9 +477,8 @@ __global__ void __maxnreg__(ST == ST_F32 ? 64 : ST == ST_F16DEV ? 80 : 255) k_st
     if (x >= M.P.nx) return;
     const int rows = blockDim.y * groups;
     const int r_end = min(M.P.ny * M.P.nz, (rb + 1) * rows);
-    const int cur = parity ^ M.flip;
-    const T* src = (const T*)M.buf[cur];
-    T* dst = (T*)M.buf[cur ^ 1];
+    const T* src = (const T*)M.buf[parity];
+    T* dst = (T*)M.buf[parity ^ 1];
     for (int r = rb * rows + threadIdx.y; r < r_end; r += blockDim.y) {
         if (M.high1) step3_node<ST, true>(src, dst, M.P, x, r % M.P.ny, r / M.P.ny);
         else step3_node<ST, false>(src, dst, M.P, x, r % M.P.ny, r / M.P.ny);
@@ -1202,10 +1199,12 @@ extern "C" clb_status clb3d_run(clb3d_lattice* h, double tol, long max_steps, lo
     return st;
 }
 
-extern "C" clb_status clb3d_init_fields(clb3d_lattice* h, const double* rho, const double* ux, const double* uy,
-                                        const double* uz, const double* T)
+namespace {
+
+// clb3d_init_fields into buffer `buf`.
+clb_status init_fields3(clb3d_lattice* h, int buf, const double* rho, const double* ux, const double* uy,
+                        const double* uz, const double* T)
 {
-    CHECK_H3(h);
     if (!rho || !ux || !uy || !uz || !T) return set_error(CLB_EINVAL, "field pointers must not be NULL");
     const long long n = nodes_of(h);
     const double* src[5] = {rho, ux, uy, uz, T};
@@ -1213,18 +1212,27 @@ extern "C" clb_status clb3d_init_fields(clb3d_lattice* h, const double* rho, con
         CLB_CUDA(cudaMemcpyAsync(h->stage + q * n, src[q], n * sizeof(double), cudaMemcpyHostToDevice, h->stream));
     const unsigned grid = unsigned((n + 255) / 256);
     if (h->p.storage == CLB_F64)
-        k_init3<ST_F64><<<grid, 256, 0, h->stream>>>((double*)h->buf[0], h->Pd, h->stage, n);
+        k_init3<ST_F64><<<grid, 256, 0, h->stream>>>((double*)h->buf[buf], h->Pd, h->stage, n);
     else if (h->p.storage == CLB_F32)
-        k_init3<ST_F32><<<grid, 256, 0, h->stream>>>((float*)h->buf[0], h->Pf, h->stage, n);
+        k_init3<ST_F32><<<grid, 256, 0, h->stream>>>((float*)h->buf[buf], h->Pf, h->stage, n);
     else
-        k_init3<ST_F16DEV><<<grid, 256, 0, h->stream>>>((__half*)h->buf[0], h->Pf, h->stage, n);
+        k_init3<ST_F16DEV><<<grid, 256, 0, h->stream>>>((__half*)h->buf[buf], h->Pf, h->stage, n);
     CLB_CUDA(cudaGetLastError());
-    h->cur = 0;
+    h->cur = buf;
     h->steps = 0;
     // the residual's first snapshot: the initial fields
     double er = 0.0;
     CLB_TRY(residual3(h, &er));
     return CLB_OK;
+}
+
+}  // namespace
+
+extern "C" clb_status clb3d_init_fields(clb3d_lattice* h, const double* rho, const double* ux, const double* uy,
+                                        const double* uz, const double* T)
+{
+    CHECK_H3(h);
+    return init_fields3(h, 0, rho, ux, uy, uz, T);
 }
 
 extern "C" clb_status clb3d_step(clb3d_lattice* h, long n)
@@ -1426,13 +1434,11 @@ struct clb3d_batch {
     cudaStream_t stream = nullptr;
     cudaStream_t cap = nullptr;  // private stream used only to capture graphs
     std::vector<clb3d_lattice*> lat;
-    std::vector<int> flip;       // lattice k's current state is in buf[parity ^ flip[k]]
-    std::vector<char> host_members;
     void* d_members = nullptr;
     int* d_owner = nullptr;
     long long ntiles = 0;
     int bx = 128, by = 2, groups = 1;
-    int parity = 0;
+    int parity = 0;              // every lattice's current state is in buf[parity]
     cudaGraphExec_t graph[2] = {nullptr, nullptr};
     bool chains = true;          // graphs hold chains of single-lattice launches (until a tile shape is set)
     int chunk = kChunk;          // steps per graph
@@ -1478,7 +1484,7 @@ void drop_batch3_graphs(clb3d_batch* b)
 }
 
 template <typename A>
-Member3<A> member3(const clb3d_batch* b, const clb3d_lattice* h, int flip, int tile_begin, const Lat3<A>& P)
+Member3<A> member3(const clb3d_batch* b, const clb3d_lattice* h, int tile_begin, const Lat3<A>& P)
 {
     Member3<A> m;
     std::memset(&m, 0, sizeof(m));
@@ -1487,7 +1493,6 @@ Member3<A> member3(const clb3d_batch* b, const clb3d_lattice* h, int flip, int t
     m.buf[1] = h->buf[1];
     m.xblocks = (h->nx + b->bx - 1) / b->bx;
     m.tile_begin = tile_begin;
-    m.flip = flip;
     m.high1 = h->p.s_3 == 1.0 && h->p.s_4 == 1.0 && h->p.s_5 == 1.0 && h->p.s_6 == 1.0;
     return m;
 }
@@ -1506,17 +1511,17 @@ clb_status batch3_tables(clb3d_batch* b)
     const long long tiles = batch3_tiles(b, b->groups);
     if (tiles > 0x7fffffffLL) return set_error(CLB_EINVAL, "batch of %lld blocks per step is too large", tiles);
     const size_t msz = b->storage == CLB_F64 ? sizeof(Member3<double>) : sizeof(Member3<float>);
-    b->host_members.assign(msz * b->lat.size(), 0);
+    std::vector<char> members(msz * b->lat.size(), 0);
     std::vector<int> owner((size_t)tiles);
     long long t0 = 0;
     for (size_t k = 0; k < b->lat.size(); ++k) {
         const clb3d_lattice* h = b->lat[k];
         if (b->storage == CLB_F64) {
-            const Member3<double> m = member3<double>(b, h, b->flip[k], (int)t0, h->Pd);
-            std::memcpy(b->host_members.data() + k * msz, &m, msz);
+            const Member3<double> m = member3<double>(b, h, (int)t0, h->Pd);
+            std::memcpy(members.data() + k * msz, &m, msz);
         } else {
-            const Member3<float> m = member3<float>(b, h, b->flip[k], (int)t0, h->Pf);
-            std::memcpy(b->host_members.data() + k * msz, &m, msz);
+            const Member3<float> m = member3<float>(b, h, (int)t0, h->Pf);
+            std::memcpy(members.data() + k * msz, &m, msz);
         }
         const long long n = (long long)((h->nx + b->bx - 1) / b->bx) *
                             (((long long)h->ny * h->nz + (long long)b->by * b->groups - 1) / ((long long)b->by * b->groups));
@@ -1527,11 +1532,11 @@ clb_status batch3_tables(clb3d_batch* b)
     cudaFree(b->d_owner);
     b->d_members = nullptr;
     b->d_owner = nullptr;
-    CLB_CUDA(cudaMalloc(&b->d_members, b->host_members.size()));
+    CLB_CUDA(cudaMalloc(&b->d_members, members.size()));
     CLB_CUDA(cudaMalloc((void**)&b->d_owner, std::max<size_t>(1, owner.size()) * sizeof(int)));
-    CLB_CUDA(cudaMemcpyAsync(b->d_members, b->host_members.data(), b->host_members.size(), cudaMemcpyHostToDevice, b->stream));
+    CLB_CUDA(cudaMemcpyAsync(b->d_members, members.data(), members.size(), cudaMemcpyHostToDevice, b->stream));
     CLB_CUDA(cudaMemcpyAsync(b->d_owner, owner.data(), owner.size() * sizeof(int), cudaMemcpyHostToDevice, b->stream));
-    CLB_CUDA(cudaStreamSynchronize(b->stream));  // the host vectors are reused or die
+    CLB_CUDA(cudaStreamSynchronize(b->stream));  // the host vectors die
     b->ntiles = tiles;
     return CLB_OK;
 }
@@ -1569,7 +1574,7 @@ clb_status batch3_chains(clb3d_batch* b, int start, cudaGraph_t g)
         const int k = order[i];
         CLB_CUDA(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
         clb_status st = CLB_OK;
-        for (int q = 0; q < b->chunk && st == CLB_OK; ++q) st = launch_step3(b->lat[k], start ^ b->flip[k] ^ (q & 1), b->cap);
+        for (int q = 0; q < b->chunk && st == CLB_OK; ++q) st = launch_step3(b->lat[k], start ^ (q & 1), b->cap);
         cudaGraph_t child = nullptr;
         cudaError_t e = cudaStreamEndCapture(b->cap, &child);
         if (st == CLB_OK && e == cudaSuccess)
@@ -1631,14 +1636,10 @@ extern "C" clb_status clb3d_batch_create(int n, const int* nx, const int* ny, co
     clb_status st = CLB_OK;
     try {
         b->lat.reserve(n);
-        b->flip.reserve(n);
         for (int k = 0; k < n && st == CLB_OK; ++k) {
             clb3d_lattice* h = nullptr;
             st = clb3d_create(nx[k], ny[k], nz[k], &p[k], stream, &h);
-            if (st == CLB_OK) {
-                b->lat.push_back(h);
-                b->flip.push_back(0);
-            }
+            if (st == CLB_OK) b->lat.push_back(h);
         }
         if (st == CLB_OK && cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess)
             st = set_error(CLB_ECUDA, "batch set-up: %s", cudaGetErrorString(cudaGetLastError()));
@@ -1683,22 +1684,8 @@ extern "C" clb_status clb3d_batch_init_fields(clb3d_batch* b, int k, const doubl
 {
     CHECK_B3(b);
     CHECK_K3(b, k);
-    const clb_status st = clb3d_init_fields(b->lat[k], rho, ux, uy, uz, T);
-    if (st != CLB_OK && st != CLB_ENAN) return st;
-    // the lattice's state is now in buf[0]: buf[parity ^ flip] with flip = parity (the chains' graphs
-    // hold buffers, so a changed flip makes them again)
-    if (b->flip[k] != b->parity && b->chains) {
-        CLB_CUDA(cudaStreamSynchronize(b->stream));
-        drop_batch3_graphs(b);
-    }
-    b->flip[k] = b->parity;
-    const size_t msz = b->storage == CLB_F64 ? sizeof(Member3<double>) : sizeof(Member3<float>);
-    const size_t off = msz * k + (b->storage == CLB_F64 ? offsetof(Member3<double>, flip) : offsetof(Member3<float>, flip));
-    std::memcpy(b->host_members.data() + off, &b->flip[k], sizeof(int));
-    CLB_CUDA(cudaMemcpyAsync((char*)b->d_members + off, b->host_members.data() + off, sizeof(int),
-                             cudaMemcpyHostToDevice, b->stream));
-    CLB_CUDA(cudaStreamSynchronize(b->stream));
-    return st;
+    // into the buffer that holds the others' state, so that graphs and tables, which know buffers, stay valid
+    return init_fields3(b->lat[k], b->parity, rho, ux, uy, uz, T);
 }
 
 extern "C" clb_status clb3d_batch_step(clb3d_batch* b, long n)
@@ -1718,7 +1705,7 @@ extern "C" clb_status clb3d_batch_step(clb3d_batch* b, long n)
         b->parity ^= 1;
     }
     for (size_t k = 0; k < b->lat.size(); ++k) {
-        b->lat[k]->cur = b->parity ^ b->flip[k];
+        b->lat[k]->cur = b->parity;
         b->lat[k]->steps += total;
     }
     return CLB_OK;

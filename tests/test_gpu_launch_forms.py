@@ -298,3 +298,37 @@ def test_tuned_shapes_are_kept_by_walls_and_rates(clb):
     general = clb.Lattice(nx, ny, W.default_params(storage=F32, wall=LAYOUTS["layer"], s_3=1.2))
     assert general.launch() == (64, 1, 2) and general.steps_per_launch() == 2
     general.close()
+
+
+# A lattice initialised again goes to the buffer the others are in: after an odd number of steps the graphs
+# of chains stay as they are (they were made again, which took tens of steps' time, for every such call).
+def test_reinitialised_box_keeps_the_graphs(clb):
+    import time
+    import torch
+    probs = [W.random_problem3d(16, 15, 14, seed=k, storage=F32) for k in range(48)]
+    for p in probs:
+        p.ux, p.uy, p.uz, p.T = 0.1 * p.ux, 0.1 * p.uy, 0.1 * p.uz, 0.1 * p.T
+    b = clb.Batch3D(probs)
+    b.set_chains(True)
+    b.step(65)
+
+    def step_ms():
+        torch.cuda.synchronize()
+        t0 = time.perf_counter()
+        b.step(32)
+        torch.cuda.synchronize()
+        return (time.perf_counter() - t0) * 1e3
+
+    before = min(step_ms() for _ in range(5))
+    after = []
+    for _ in range(5):
+        b.step(1)  # the state changes buffers
+        b.init_fields(7, *probs[7].fields())
+        after.append(step_ms())
+    assert min(after) <= 2 * before
+    lat = clb.Lattice3D.from_problem(probs[7])
+    lat.step(32)
+    for x, y in zip(lat.populations(), b.member(7).populations()):
+        assert np.isfinite(x).all() and np.array_equal(x, y)
+    lat.close()
+    b.close()
