@@ -159,8 +159,9 @@ clb_status clb3d_batch_init_fields(clb3d_batch* b, int k, const double* rho, con
 /* n >= 0 time steps of every lattice, enqueued on the stream. */
 clb_status clb3d_batch_step(clb3d_batch* b, long n);
 /* Steps are replayed from graphs that hold a chain of single-lattice launches per lattice, side by
- * side (chains = 1, the default), or one launch per step for all lattices (chains = 0); the steps left
- * over go through the latter. Setting another tile sets chains to 0. Results do not depend on it. */
+ * side (chains = 1), or one launch per step for all lattices (chains = 0); the steps left over go through
+ * the latter. The default is by storage, number and size of the lattices, and takes the chains once the
+ * steps asked for so far are worth the making of their graphs; chains set explicitly are taken at once. Setting another tile sets chains to 0. Results do not depend on it. */
 clb_status clb3d_batch_set_chains(clb3d_batch* b, int chains);
 clb_status clb3d_batch_get_chains(clb3d_batch* b, int* chains);
 /* Thread block of the batched step: block_x threads along x (a multiple of 32, <= 256) times block_y

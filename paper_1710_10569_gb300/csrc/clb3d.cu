@@ -1422,12 +1422,15 @@ extern "C" clb_status clb3d_buffers(clb3d_lattice* h, void** current, long long*
 
 // ---------------------------------------------------------------------------------------------
 // Batches of 3-D lattices: every lattice is an ordinary handle (its own memory, fields, Nusselt
-// number, residual); the time steps of all of them go through one k_step3_batched launch per step
-// over their concatenated tiles, replayed from CUDA graphs of kChunk steps.
+// number, residual). Their time steps are replayed from CUDA graphs, which hold either one
+// k_step3_batched launch per step over the concatenated tiles of all lattices (kChunk steps), or a chain
+// of single-lattice launches per lattice (batch3_chains); steps that fill no graph go through the former.
 
-// Chains of the graphs of a batch at most, and the steps per graph of batches of many nodes.
+// Chains of the graphs of a batch that run at once, the steps per graph of batches of many nodes and of
+// more launches per graph than kGraphLaunches, and the cost in us of making a graph, per launch.
 constexpr size_t kMaxChains = 32;
-constexpr int kShortChunk = 8;
+constexpr int kShortChunk = 8, kGraphLaunches = 4096;
+constexpr double kGraphLaunchUs = 4.5;
 
 struct clb3d_batch {
     int storage = CLB_F64;
@@ -1439,9 +1442,12 @@ struct clb3d_batch {
     long long ntiles = 0;
     int bx = 128, by = 2, groups = 1;
     int parity = 0;              // every lattice's current state is in buf[parity]
-    cudaGraphExec_t graph[2] = {nullptr, nullptr};
-    bool chains = true;          // graphs hold chains of single-lattice launches (until a tile shape is set)
-    int chunk = kChunk;          // steps per graph
+    cudaGraphExec_t single[2] = {nullptr, nullptr};  // graphs of one launch per step, by parity
+    cudaGraphExec_t graph[2] = {nullptr, nullptr};   // graphs of chains of single-lattice launches
+    bool chains = false;         // steps go through the latter (until a tile shape is set)
+    int chunk = kChunk;          // steps per graph of chains (even)
+    double chains_gain = 0;      // us per step that chains save by the estimate; 0: they are wanted at once
+    long long stepped = 0;       // steps taken while the chains are not worth their graphs
 };
 
 namespace {
@@ -1476,11 +1482,45 @@ long long batch3_tiles(const clb3d_batch* b, int g)
 
 void drop_batch3_graphs(clb3d_batch* b)
 {
-    for (auto& g : b->graph)
-        if (g) {
-            cudaGraphExecDestroy(g);
-            g = nullptr;
-        }
+    for (auto* graphs : {b->single, b->graph})
+        for (int par = 0; par < 2; ++par)
+            if (graphs[par]) {
+                cudaGraphExecDestroy(graphs[par]);
+                graphs[par] = nullptr;
+            }
+}
+
+// Whether chains of single-lattice launches step the batch faster than one launch for all, by how much, and
+// the steps per graph of chains. Times in us, fitted to batches of 12 to 1,000 equal boxes of edge 8 to 48 and
+// uneven ones: a chain's launch costs 0.32 us of the whole device however small its box, 0.39 in short graphs;
+// one launch for all takes 3.1 ns per block of 128 x 2 nodes, up to 4.8 on batches of fewer blocks; in the FP16
+// form a quarter more, and in FP64 twice as long as chains at any size. Chains / one launch, FP32: 12 boxes of
+// edge 16 8.3 / 11.5 us per step, 48 of 12 19.9 / 21.8, 200 of 8 to 40 111 / 146, 1,000 of 16 387 / 398, but 12
+// of edge 8 6.5 / 5.3, 256 of 8 70 / 44, 800 of 14 314 / 254, 1,000 of 8 293 / 121.
+void batch3_choose(clb3d_batch* b)
+{
+    double tiles = 0, nodes = 0;
+    for (const clb3d_lattice* h : b->lat) {
+        tiles += double((h->nx + 127) / 128) * (((long long)h->ny * h->nz + 1) / 2);
+        nodes += double(nodes_of(h));
+    }
+    const size_t n = b->lat.size();
+    b->chunk = nodes >= 500000 ? kShortChunk : kChunk;
+    while (b->chunk > kShortChunk && b->chunk * n > kGraphLaunches) b->chunk /= 2;
+    const double chains = 2.5 + (b->chunk > kShortChunk ? 0.32 : 0.39) * n;
+    const double all = tiles * (3.1e-3 + 1.7e-3 * std::min(1.0, 1e4 / tiles));
+    b->chains_gain = b->storage == CLB_F64   ? 1.5e-3 * nodes
+                     : b->storage == CLB_F32 ? 4.0 + all - chains
+                                             : 10.0 + 1.25 * all - chains;
+    b->chains = b->chains_gain > 0;
+    b->stepped = 0;
+}
+
+// An explicit choice: chains from the next step on, or not at all.
+void batch3_form(clb3d_batch* b, bool chains)
+{
+    b->chains = chains;
+    b->chains_gain = 0;
 }
 
 template <typename A>
@@ -1556,8 +1596,8 @@ clb_status batch3_launch(clb3d_batch* b, int par, cudaStream_t s)
     return CLB_OK;
 }
 
-// A graph of b->chunk steps of every lattice, each lattice's steps a child graph of its own. The lattices of a batch do not depend on one another, so they are chains of launches of the
-// single-lattice step, which reads its parameters from the constant bank where the batched kernel
+// A graph of b->chunk steps of every lattice, each lattice's steps a child graph of its own. The lattices
+// of a batch do not depend on one another, so they are chains of launches of the single-lattice step, which reads its parameters from the constant bank where the batched kernel
 // reads them from shared memory under a register cap, and lets the hardware run the chains side by
 // side: 12 boxes of edge 24 to 128 (3.1 million nodes) 175.0 -> 138.6 us per step in FP32, 194.7 -> 111.6 in
 // FP16; 12 of edge 16 to 48 33.6 -> 16.2; 48 of edge 16 to 32 62.8 -> 35.9 (16 chains). Fewer chains leave
@@ -1586,11 +1626,12 @@ clb_status batch3_chains(clb3d_batch* b, int start, cudaGraph_t g)
     return CLB_OK;
 }
 
-clb_status batch3_graph(clb3d_batch* b, int start)
+// The graph of chains, or of kChunk steps of one launch each, from buffer `start`.
+clb_status batch3_graph(clb3d_batch* b, int start, bool chains)
 {
     cudaGraph_t g = nullptr;
     clb_status st = CLB_OK;
-    if (b->chains) {
+    if (chains) {
         CLB_CUDA(cudaGraphCreate(&g, 0));
         try {
             st = batch3_chains(b, start, g);
@@ -1599,12 +1640,12 @@ clb_status batch3_graph(clb3d_batch* b, int start)
         }
     } else {
         CLB_CUDA(cudaStreamBeginCapture(b->cap, cudaStreamCaptureModeThreadLocal));
-        for (int k = 0; k < b->chunk && st == CLB_OK; ++k) st = batch3_launch(b, start ^ (k & 1), b->cap);
+        for (int k = 0; k < kChunk && st == CLB_OK; ++k) st = batch3_launch(b, start ^ (k & 1), b->cap);
         const cudaError_t e = cudaStreamEndCapture(b->cap, &g);
         if (st == CLB_OK && e != cudaSuccess) st = set_error(CLB_ECUDA, "graph capture: %s", cudaGetErrorString(e));
     }
     if (st == CLB_OK) {
-        const cudaError_t e = cudaGraphInstantiate(&b->graph[start], g, 0);
+        const cudaError_t e = cudaGraphInstantiate(chains ? &b->graph[start] : &b->single[start], g, 0);
         if (e != cudaSuccess) st = set_error(CLB_ECUDA, "graph instantiate: %s", cudaGetErrorString(e));
     }
     if (g) cudaGraphDestroy(g);
@@ -1643,9 +1684,7 @@ extern "C" clb_status clb3d_batch_create(int n, const int* nx, const int* ny, co
         }
         if (st == CLB_OK && cudaStreamCreateWithFlags(&b->cap, cudaStreamNonBlocking) != cudaSuccess)
             st = set_error(CLB_ECUDA, "batch set-up: %s", cudaGetErrorString(cudaGetLastError()));
-        long long nodes = 0;
-        for (const clb3d_lattice* h : b->lat) nodes += nodes_of(h);
-        if (nodes >= 500000) b->chunk = kShortChunk;
+        if (st == CLB_OK) batch3_choose(b);
         if (st == CLB_OK) st = batch3_tables(b);
     } catch (const std::bad_alloc&) {
         st = set_error(CLB_ENOMEM, "host allocation failed");
@@ -1693,12 +1732,23 @@ extern "C" clb_status clb3d_batch_step(clb3d_batch* b, long n)
     CHECK_B3(b);
     if (n < 0) return set_error(CLB_EINVAL, "n = %ld < 0", n);
     const long total = n;
-    if (n >= b->chunk)
+    // Chains once the steps asked for so far would have paid for their graph (256 boxes of edge 16: 9 ms, 28 us
+    // saved per step), one launch per step until then.
+    bool chains = b->chains;
+    if (chains && !b->graph[b->parity]) {
+        b->stepped += n;
+        chains = n >= b->chunk && double(b->stepped) * b->chains_gain >= kGraphLaunchUs * b->chunk * double(b->lat.size());
+        chains = chains || b->chains_gain == 0;
+    }
+    const int chunk = chains ? b->chunk : kChunk;
+    cudaGraphExec_t* graphs = chains ? b->graph : b->single;
+    // (graphs of chains cost more to make: only the parity that is needed)
+    if (n >= chunk)
         for (int par = 0; par < 2; ++par)
-            if (!b->graph[par]) CLB_TRY(batch3_graph(b, par));
-    while (n >= b->chunk) {
-        CLB_CUDA(cudaGraphLaunch(b->graph[b->parity], b->stream));
-        n -= b->chunk;
+            if (!graphs[par] && (par == b->parity || !chains)) CLB_TRY(batch3_graph(b, par, chains));
+    while (n >= chunk) {
+        CLB_CUDA(cudaGraphLaunch(graphs[b->parity], b->stream));
+        n -= chunk;
     }
     for (; n > 0; --n) {
         CLB_TRY(batch3_launch(b, b->parity, b->stream));
@@ -1718,7 +1768,7 @@ extern "C" clb_status clb3d_batch_set_tile(clb3d_batch* b, int block_x, int bloc
         return set_error(CLB_EINVAL, "tile %d x %d: block_x in [32, 256] multiple of 32, block_x * block_y <= 256",
                          block_x, block_y);
     CLB_CUDA(cudaStreamSynchronize(b->stream));
-    if (block_x != b->bx || block_y != b->by) b->chains = false;  // the present tile set again changes nothing
+    if (block_x != b->bx || block_y != b->by) batch3_form(b, false);  // the present tile set again changes nothing
     b->bx = block_x;
     b->by = block_y;
     try {
@@ -1735,7 +1785,7 @@ extern "C" clb_status clb3d_batch_set_chains(clb3d_batch* b, int chains)
     if (b->chains == (chains == 1)) return CLB_OK;
     CLB_CUDA(cudaStreamSynchronize(b->stream));
     drop_batch3_graphs(b);
-    b->chains = chains == 1;
+    batch3_form(b, chains == 1);
     return CLB_OK;
 }
 
