@@ -69,7 +69,9 @@ inline cudaError_t launch_chained(void (*kernel)(P...), dim3 grid, dim3 block, s
     cfg.stream = s;
     cfg.attrs = &at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+    if (e != cudaSuccess) cudaGetLastError();  // reported here; not again by the caller's next call
+    return e;
 }
 
 constexpr long long kMaxNodes = 1LL << 30;  // index arithmetic and memory bound
