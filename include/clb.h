@@ -225,7 +225,8 @@ clb_status clb_get_steps_per_launch(clb_handle *h, int *steps);
 /* The CUDA stream the handle enqueues on (to time its work with events on that stream). */
 void *clb_stream(clb_handle *h);
 
-/* How the FP16 storage form splits a time step (host only, no device work; for tools and tests).
+/* How the FP16 storage form splits a time step of a lattice of 400,000 nodes or more (host only, no device
+ * work; for tools and tests; the partition of smaller ones, which step in one kernel, is reported too).
  * The warps of the interior, whose 32 * npt nodes lie inside the row with no wall next to any of
  * them, run in one kernel; the others (rows next to a y wall or on a wet y wall, the columns next to
  * an x wall or on a wet x wall or holding the ragged end of the rows) run in a second kernel beside

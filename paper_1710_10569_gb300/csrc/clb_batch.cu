@@ -359,9 +359,9 @@ public:
         return CLB_OK;
     }
 
-    // One device allocation (and one pinned host mirror) for the member descriptors, the
-    // diagnostics outputs and the tile- and row-owner tables, at the given capacities. Lattices of more
-    // than max_march windows and segments step one step per launch.
+    // One device allocation (and one pinned host mirror) for the member descriptors and the tile-, row- and
+    // march-owner tables, at the given capacities; behind the mirror, the diagnostics outputs. Lattices of
+    // more than max_march windows and segments step one step per launch.
     clb_status reserve(size_t max_members, size_t max_tiles, size_t max_rows, size_t max_march)
     {
         cap_members = std::max<size_t>(1, max_members);
@@ -370,17 +370,18 @@ public:
         cap_march = storage == CLB_F32 ? max_march : 0;
         const size_t msz = std::max(sizeof(Member<double>), sizeof(Member<float>));
         off_members = 0;
-        off_diag = align256(cap_members * msz);
-        off_owner = off_diag + align256(cap_members * kDiagStride * sizeof(double));
+        off_owner = align256(cap_members * msz);
         off_rows = off_owner + align256(cap_tiles * sizeof(int));
         off_march = off_rows + align256(cap_rows * sizeof(int));
         table_bytes = off_march + align256(cap_march * sizeof(int));
+        off_diag = table_bytes;
+        const size_t host_bytes = table_bytes + cap_members * kDiagStride * sizeof(double);
         cudaError_t e = cudaMalloc(&d_tables, table_bytes);
         if (e != cudaSuccess)
             return set_error(e == cudaErrorMemoryAllocation ? CLB_ENOMEM : CLB_ECUDA, "launch tables (%zu bytes): %s",
                              table_bytes, cudaGetErrorString(e));
-        e = cudaMallocHost(&h_tables, table_bytes);
-        if (e != cudaSuccess) return set_error(CLB_ENOMEM, "pinned launch tables (%zu bytes): %s", table_bytes, cudaGetErrorString(e));
+        e = cudaMallocHost(&h_tables, host_bytes);
+        if (e != cudaSuccess) return set_error(CLB_ENOMEM, "pinned launch tables (%zu bytes): %s", host_bytes, cudaGetErrorString(e));
         return CLB_OK;
     }
 
@@ -676,8 +677,8 @@ private:
     static constexpr int kCountedRows = 1024;        // lattices of more rows are listed one by one
     std::vector<std::pair<int, long>> march_strips;  // (rows, windows per row) of the active lattices
     std::vector<long> strips_of;
-    void* d_tables = nullptr;  // members | (diagnostics outputs: in the mirror) | tile, row and march owners
-    void* h_tables = nullptr;  // pinned mirror of the same layout
+    void* d_tables = nullptr;  // members | tile, row and march owners
+    void* h_tables = nullptr;  // pinned mirror of the same layout | diagnostics outputs
     size_t off_members = 0, off_diag = 0, off_owner = 0, off_rows = 0, off_march = 0, table_bytes = 0;
     size_t cap_members = 0, cap_tiles = 0, cap_rows = 0, cap_march = 0;
     cudaEvent_t copied = nullptr;  // recorded after the last copy of the mirrors

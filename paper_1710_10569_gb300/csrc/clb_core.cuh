@@ -79,7 +79,8 @@ __device__ __forceinline__ double scale_down(double x)
     const bool keep = e == 0x7ff, tiny = e <= N;
     return __hiloint2double(keep ? hi : tiny ? hi & (int)0x80000000 : hi - (N << 20), !keep && tiny ? 0 : __double2loint(x));
 }
-// 2 x by its exponent (zero and subnormal numbers, which lack the hidden bit, by an addition).
+// 2 x by its exponent: zero and subnormal numbers give a signed zero; infinities, NaN and numbers from 2^1023
+// on, whose double is infinite, stay as they are.
 __device__ __forceinline__ double scale_up1(double x)
 {
     const int hi = __double2hiint(x);
@@ -88,7 +89,8 @@ __device__ __forceinline__ double scale_up1(double x)
 }
 // 1 / x from the hardware's approximation r (relative error e below 2^-19) by one step of Halley's
 // third-order iteration, r + r (e + e^2) with e = 1 - x r: three FMAs in place of the six of the
-// correctly rounded reciprocal, and within one unit of the last place of it.
+// correctly rounded reciprocal, and within one unit of the last place of it. For densities: 1 / 0 and 1 / inf
+// are NaN here (a node whose density is either has no finite fields in any form).
 __device__ __forceinline__ double rcp_halley(double x)
 {
     double r;

@@ -115,7 +115,7 @@ struct DeviceGuard {
 int diag_segments(int nx) { return (nx + kDiagNodes - 1) / kDiagNodes; }
 
 struct Layout {
-    size_t buf[2], snap, stage, partial, diag, total;
+    size_t buf[2], snap, stage, partial, total;
 };
 
 Layout layout(int nx, int ny, int storage)
@@ -129,7 +129,6 @@ Layout layout(int nx, int ny, int storage)
     L.snap = off; off += align256(3 * N * sizeof(double));
     L.stage = off; off += align256(4 * N * sizeof(double));
     L.partial = off; off += align256((size_t)ny * diag_segments(nx) * RS_N * sizeof(double));
-    L.diag = off; off += align256(16 * sizeof(double));
     L.total = off;
     return L;
 }
