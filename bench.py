@@ -223,26 +223,24 @@ def aggregate(units: float, seconds: float, world: int):
     return float(u.item()), float(s.item())
 
 
-def steps_per_launch(storage: int, nodes: int) -> int:
-    """Time steps that one launch advances a Rayleigh-Benard lattice by under the library's default:
-    two for FP32 lattices of a million nodes or more."""
-    return 2 if storage == W.STORAGE_F32 and nodes >= 1_000_000 else 1
+def split_step(storage: int, nodes: int) -> bool:
+    """An FP16 lattice of this size splits its step into an interior kernel and an edge kernel (wall rows)
+    that run side by side."""
+    return storage == W.STORAGE_F16DEV and nodes >= 400_000
 
 
-def step_kernels(storage: int, nodes: int, steps: int) -> int:
-    """Step kernels that clb_run launches over `steps` steps (DIAG_INTERVAL at a time) on a
-    Rayleigh-Benard lattice: an odd step is a launch by itself where launches take two, and an FP16
-    lattice of this size splits its step into an interior kernel and an edge kernel (wall rows) that
-    run side by side."""
-    per = steps_per_launch(storage, nodes)
+def step_kernels(storage: int, nodes: int, per: int, steps: int) -> int:
+    """Step kernels that clb_run launches over `steps` steps (DIAG_INTERVAL at a time) on a lattice that
+    advances `per` steps per launch (Lattice.steps_per_launch): an odd step is a launch by itself where
+    launches take two."""
     parts = [min(DIAG_INTERVAL, steps - k) for k in range(0, steps, DIAG_INTERVAL)]
-    return sum(-(-n // per) for n in parts) * (2 if storage == W.STORAGE_F16DEV else 1)
+    return sum(-(-n // per) for n in parts) * (2 if split_step(storage, nodes) else 1)
 
 
-def step_kernel_name(storage: int, nodes: int) -> str:
-    if storage == W.STORAGE_F16DEV:
+def step_kernel_name(storage: int, nodes: int, per: int) -> str:
+    if split_step(storage, nodes):
         return "k_step_inner_f16x4_hi1 + k_step_edge<f16dev> (one step)"
-    if steps_per_launch(storage, nodes) == 2:
+    if per == 2:
         return f"k_step_two ({W.STORAGE_NAMES[storage]}, two steps)"
     return f"k_step<{W.STORAGE_NAMES[storage]}>"
 
@@ -383,9 +381,9 @@ def thermal_run(storage: int, steps: int, nx: int = 4096, ny: int = 4096):
     e1.record(stream)
     torch.cuda.synchronize()
     dt = e0.elapsed_time(e1) / 1e3
+    per = th.steps_per_launch()
     th.close()
     per_node = {W.STORAGE_F64: 96, W.STORAGE_F32: 48, W.STORAGE_F16DEV: 28}[storage]
-    per = 1 if storage == W.STORAGE_F64 else 4  # steps per launch of a lattice of this size
     peak, _ = measured_peaks()
     gbs = per_node * nx * ny * steps / per / dt / 1e9
     return {"workload": f"thermal_only_{nx}x{ny}_cellular_flow", "mlups": nx * ny * steps / dt / 1e6,
@@ -418,14 +416,14 @@ def batched_run(storage: int, count: int = 256, steps: int = 1000, seq_subset: i
     def time_batch(ps, k):
         b = clb.Batch(ps)
         b.autotune()
-        launch = b.launch()
+        launch = dict(b.launch(), steps=b.steps_per_launch())
         b.step(64)
         dt = device_seconds(b.stream, lambda: b.step(k))
         b.close()
         return dt, launch
 
     dt_all, launch = time_batch(probs, steps)
-    per = 2 if storage == W.STORAGE_F32 else 1  # steps per launch of a batch of this size
+    per = launch["steps"]
     peak, _ = measured_peaks()
     sub = probs[:seq_subset]
     sub_nodes = sum(p.nodes for p in sub)
@@ -512,7 +510,7 @@ def batched3d_run(steps: int, count: int = 48, seq_subset: int = 12):
         b = clb.Batch3D(ps)
         b.step(64)
         dt = timed(b.stream, lambda: b.step(steps))
-        launch = b.launch()
+        launch = dict(b.launch(), chains=b.chains())
         b.close()
         return dt, launch
 
@@ -534,7 +532,7 @@ def batched3d_run(steps: int, count: int = 48, seq_subset: int = 12):
         lat.close()
     gbs = BYTES_PER_NODE_3D[st] * nodes * steps / dt / 1e9
     return {"instances": count, "nodes": nodes, "steps": steps, "storage": W.STORAGE_NAMES[st],
-            "block": list(launch["block"]), "row_groups_per_block": launch["groups"],
+            "chains": launch["chains"], "block": list(launch["block"]), "row_groups_per_block": launch["groups"],
             "blocks_per_launch": launch["blocks"], "mlups": nodes * steps / dt / 1e6,
             "achieved_gbs": gbs, "hbm_frac": gbs / peak,
             "subset": {"instances": seq_subset, "batched_mlups": sub_nodes * steps / dt_sub / 1e6,
@@ -713,7 +711,7 @@ def run_ours(args):
     units, tmax = aggregate(float(nodes) * args.steps, secs, world)
     mlups = units / tmax / 1e6
     peak, peak_kind = measured_peaks()
-    per = steps_per_launch(storage, nodes)
+    per = lat.steps_per_launch()
     launches = k_steps // per
     per_launch_s = secs_kernel / launches
     alg_bytes = BYTES_PER_NODE[storage] * nodes
@@ -732,7 +730,7 @@ def run_ours(args):
                 l2.autotune()
             k = max(200, args.steps // (8 if st == W.STORAGE_F64 else 2))
             s2 = time_steps(l2, k, max(3, args.warmup // 4), 1)
-            per2 = steps_per_launch(st, p2.nodes)
+            per2 = l2.steps_per_launch()
             variants[W.STORAGE_NAMES[st]] = {
                 "workload": f"rayleigh_benard_{p2.nx}x{p2.ny}_Ra1e7_Pr0.71",
                 "mlups": p2.nodes * k / s2 / 1e6,
@@ -784,14 +782,14 @@ def run_ours(args):
                          "steps_per_launch": per, "kernel_launches_timed": launches,
                          "kernel_us_per_launch": per_launch_s * 1e6,
                          "algorithmic_bytes_per_launch": alg_bytes,
-                         "kernel": step_kernel_name(storage, nodes),
+                         "kernel": step_kernel_name(storage, nodes, per),
                          "flops_per_node": flops_per_node(storage),
                          "peak_kind": f"{peak_kind} HBM copy bandwidth (MEASURED_PEAKS.json hbm_gbs)"},
             "cpu_baseline": cpu,
             "e2e": e2e,
             # the step kernels (two steps each in the FP32 form at this size; the FP16 form: an interior
             # and an edge kernel per step), plus the two reduction kernels of each check
-            "gpu_launches": step_kernels(storage, nodes, args.steps) + 2 * diag_checks(args.steps),
+            "gpu_launches": step_kernels(storage, nodes, per, args.steps) + 2 * diag_checks(args.steps),
             "clocks": clocks.summary(),
             "variants": variants,
             "thermal_only": thermal,
