@@ -457,7 +457,7 @@ class Thermal:
 
 
 class Batch:
-    """Many lattices stepped in one launch per time step (clb_batch_*)."""
+    """Many lattices stepped in shared launches of one or two time steps (clb_batch_*)."""
 
     def __init__(self, problems, stream=None):
         L = lib()
@@ -754,7 +754,7 @@ class _Member3D(Lattice3D):
 
 
 class Batch3D:
-    """Many 3-D lattices (clb3d_batch_*) stepped by one launch per time step. `member(k)` gives a
+    """Many 3-D lattices (clb3d_batch_*) stepped side by side or by one launch per time step. `member(k)` gives a
     Lattice3D view of lattice k for fields, populations, Nusselt number and residual."""
 
     def __init__(self, problems, stream=None):

@@ -1596,10 +1596,10 @@ clb_status batch3_launch(clb3d_batch* b, int par, cudaStream_t s)
     return CLB_OK;
 }
 
-// A graph of b->chunk steps of every lattice, each lattice's steps a child graph of its own. The lattices
-// of a batch do not depend on one another, so they are chains of launches of the single-lattice step, which reads its parameters from the constant bank where the batched kernel
-// reads them from shared memory under a register cap, and lets the hardware run the chains side by
-// side: 12 boxes of edge 24 to 128 (3.1 million nodes) 175.0 -> 138.6 us per step in FP32, 194.7 -> 111.6 in
+// A graph of b->chunk steps of every lattice, each lattice's steps a child graph of its own. The lattices of
+// a batch do not depend on one another, so they are chains of launches of the single-lattice step, which
+// reads its parameters from the constant bank where the batched kernel reads them from shared memory under a
+// register cap, and lets the hardware run the chains side by side: 12 boxes of edge 24 to 128 (3.1 million nodes) 175.0 -> 138.6 us per step in FP32, 194.7 -> 111.6 in
 // FP16; 12 of edge 16 to 48 33.6 -> 16.2; 48 of edge 16 to 32 62.8 -> 35.9 (16 chains). Fewer chains leave
 // the chip idle (12 boxes: 4 chains 150.5, 2 166.7). At most kMaxChains run at once, largest first.
 // Steps that fill no graph go through the batched kernel, one launch for all lattices; graphs of large
@@ -1737,8 +1737,8 @@ extern "C" clb_status clb3d_batch_step(clb3d_batch* b, long n)
     bool chains = b->chains;
     if (chains && !b->graph[b->parity]) {
         b->stepped += n;
-        chains = n >= b->chunk && double(b->stepped) * b->chains_gain >= kGraphLaunchUs * b->chunk * double(b->lat.size());
-        chains = chains || b->chains_gain == 0;
+        const double graph_us = kGraphLaunchUs * b->chunk * double(b->lat.size());
+        chains = b->chains_gain == 0 || (n >= b->chunk && double(b->stepped) * b->chains_gain >= graph_us);
     }
     const int chunk = chains ? b->chunk : kChunk;
     cudaGraphExec_t* graphs = chains ? b->graph : b->single;

@@ -305,14 +305,16 @@ long tiles_of(int nx, int ny, int tile_x, int tile_y, int npt)
 constexpr double kMarchBatchNodes = 400000, kBatchStepUs = 3.0, kBatchNodeUs = 112.0 / 6.2e6;
 
 // Batches below kL2BatchNodes, whose buffers stay in L2, have a time of one step that depends on their rows: a
-// row of 64 nodes or more is cut into warps of 64 (1.10 ns each, 1.22 between x walls), a shorter one goes
-// node by node (0.030 ns). Two steps per launch take kMarchFit times march_rows_for's time, more between x
-// walls and for general rates (one step per launch: 4% more). us per step, one step per launch against two:
-// 120 of 64 x 64 9.6 / 14.4 and 8 of 256 x 256 9.8 / 10.4, whose rows fill their warps, and 50 of 125 x 90
-// 12.5 / 13.0, stay with one; 300 of 40 x 40 17.1 / 11.3, 12 of 200 x 200 11.4 / 9.4 and 12 of edge 64 to
-// 400 10.6 / 9.4 take two (fitted to 28 batches of 0.1 to 1 million nodes).
-constexpr double kL2BatchNodes = 1.0e6, kRowWarpUs = 1.10e-3, kRowWarpWallUs = 1.22e-3, kShortNodeUs = 3.0e-5;
-constexpr double kMarchFit = 1.10, kMarchXWalls = 0.11, kMarchGeneral = 1.11, kOneGeneral = 1.04;
+// row of 64 nodes or more is cut into warps of 64 (1.05 ns each, 8% more between x walls; an odd row's last
+// node half a warp), a shorter one goes node by node (0.030 ns); 5% more for general rates. Two steps per
+// launch take kMarchFit times march_rows_for's time, more for general rates, between x walls and on rows of
+// odd length. us per step, one step per launch against two: 120 of 64 x 64 9.6 / 14.4 and 8 of 256 x 256
+// 9.8 / 10.4, whose rows fill their warps, and 50 of 125 x 90 12.5 / 13.0, stay with one; 300 of 40 x 40
+// 17.1 / 11.3, 12 of 200 x 200 11.4 / 9.4 and 12 of edge 64 to 400 10.6 / 9.4 take two. Fitted to 40 batches
+// of 0.1 to 1 million nodes; between 0.4 and 1 million the choice costs 5% at most against the better one.
+constexpr double kL2BatchNodes = 1.0e6, kL2StepUs = 0.5, kRowWarpUs = 1.05e-3, kShortNodeUs = 3.0e-5;
+constexpr double kOneXWalls = 0.08, kOneGeneral = 1.05;
+constexpr double kMarchFit = 1.12, kMarchXWalls = 0.11, kMarchOddRows = 0.10, kMarchGeneral = 1.11;
 
 constexpr int kDiagStride = 16;  // doubles of diagnostics output per member
 
@@ -439,19 +441,21 @@ public:
     {
         march = 0;
         if (storage != CLB_F32 || one_step) return;
-        double nodes = 0, walled = 0, one = 0;  // walled: nodes of lattices between x walls
+        double nodes = 0, walled = 0, odd = 0, one = kL2StepUs;  // walled, odd: nodes of lattices between x walls, of odd rows
         for (const Lattice* L : active) {
             if (L->p.wall[0] == CLB_WALL_WET || L->p.wall[2] == CLB_WALL_WET) return;
             const double n = double(L->nx) * L->ny;
             const bool x_walls = L->p.wall[0] != CLB_PERIODIC;
             nodes += n;
             if (x_walls) walled += n;
-            one += L->nx >= 64 ? (L->nx + 63) / 64 * double(L->ny) * (x_walls ? kRowWarpWallUs : kRowWarpUs) : n * kShortNodeUs;
+            if (L->nx % 2) odd += n;
+            const double rows = ((L->nx - L->nx % 2 + 63) / 64 + 0.5 * (L->nx % 2)) * double(L->ny) * kRowWarpUs;
+            one += (L->nx >= 64 ? rows : n * kShortNodeUs) * (x_walls ? 1.0 + kOneXWalls : 1.0);
         }
         if (nodes < kMarchBatchNodes) return;
         double limit = kBatchStepUs + nodes * kBatchNodeUs;  // march_rows_for's time has to be less
         if (nodes < kL2BatchNodes) {
-            const double two = kMarchFit * (1.0 + kMarchXWalls * walled / nodes) * (form == 0 ? kMarchGeneral : 1.0);
+            const double two = kMarchFit * (1.0 + (kMarchXWalls * walled + kMarchOddRows * odd) / nodes) * (form == 0 ? kMarchGeneral : 1.0);
             limit = std::min(limit, one * (form == 0 ? kOneGeneral : 1.0) / two);
         }
         int dev = 0, sms = 1;

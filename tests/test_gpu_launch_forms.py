@@ -392,3 +392,19 @@ def test_first_steps_of_a_3d_batch(clb):
 
     first_ms(False)
     assert min(first_ms(True) for _ in range(3)) <= 1.3 * min(first_ms(False) for _ in range(3))
+
+
+# The same for uneven batches near 400,000 nodes, some of odd widths.
+@pytest.mark.parametrize("rates", [1.0, 1.2])
+@pytest.mark.parametrize("sizes", [[(300, 300), (500, 400), (129, 1000), (64, 90)], [(513, 385), (301, 700)], [(257, 300)] * 6,
+                                   [(91, 120)] * 40, [(180, 180)] * 13, [(101, 101)] * 40], ids=["uneven", "odd", "257", "91", "180", "101"])
+def test_default_form_of_uneven_batches_is_not_the_slower_one(clb, sizes, rates):
+    probs = [W.random_problem(nx, ny, seed=k, storage=F32, walls=sorted(LAYOUTS.values())[k % 5]) for k, (nx, ny) in enumerate(sizes)]
+    for p in probs:
+        p.params.update(s_3=rates, s_4=rates, lambda2=rates)
+        p.T, p.ux, p.uy = 0.1 * p.T, 0.1 * p.ux, 0.1 * p.uy
+    b = clb.Batch(probs)
+    us = step_us(b)
+    b.set_steps_per_launch(1)
+    assert us <= 1.05 * step_us(b)
+    b.close()
