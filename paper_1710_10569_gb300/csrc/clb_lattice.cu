@@ -299,11 +299,13 @@ Launch current_launch(const clb_handle* h)
 // bandwidth, is less (few rows, or rows that fill their windows badly), and below kMarchNodes: the two
 // buffers of such lattices sit in the 129 MB L2, from where one step per launch runs without the
 // repeated columns and rows (1024 x 512: 6.9 us against 7.9). Up to kL2Nodes most of it still does, and the
-// bytes at the copy bandwidth are more than one step takes: 0.97 ns per warp of 64 nodes there, 12% more for general
-// rates, against the two-step kernel's time with its x walls (19%) and general rates (11%; 5% otherwise).
-// Cavity of 1024 x 1024: 16.0 us with one step per launch, 16.3 with two, general rates 18.0 and 18.1; layer 15.8
-// and 14.7; cavity of 2048 x 512 15.9 and 14.2.
-constexpr long long kMarchNodes = 1000000, kL2Nodes = 1080000;
+// bytes at the copy bandwidth are more than one step takes: 0.97 ns per warp of 64 nodes there, a third more for a
+// row's last warp if it is not full, 12% more for general rates, against the two-step kernel's time with its x
+// walls (19%; 3% otherwise), general rates (11%) and odd rows of four windows or fewer (22%). Cavity of 1024 x 1024: 16.0
+// us with one step per launch, 16.3 with two, general rates 18.0 and 18.1; of 128 x 9019 19.1 and 24.5; layer of
+// 121 x 9002 with general rates 23.4 and 26.2, but of 1024 x 1024 15.8 and 14.7, cavities of 2048 x 512 15.9 and
+// 14.2, 305 x 3700 21.7 and 19.8 (24 shapes, both kinds of walls and rates: the choice costs 5% at most).
+constexpr long long kMarchNodes = 1000000, kL2Nodes = 1200000;
 int march_rows_rule(int nx, int ny, const clb_params& p, int sms)
 {
     const bool wet = p.wall[0] == CLB_WALL_WET || p.wall[2] == CLB_WALL_WET;
@@ -312,8 +314,9 @@ int march_rows_rule(int nx, int ny, const clb_params& p, int sms)
     double limit = 1.0 + 112.0 * nodes / 6.7e6;  // march_rows_for's time has to be less
     if (nodes < kL2Nodes) {
         const bool general = collide_form(p) == 0;
-        const double one = 1.51e-5 * ((nx + 63) / 64 * 64.0 * ny) * (general ? 1.12 : 1.0);
-        limit = std::min(limit, one / ((p.wall[0] != CLB_PERIODIC ? 1.19 : 1.05) * (general ? 1.11 : 1.0)));
+        const double one = 0.966e-3 * (nx / 64 + (nx % 64 ? 1.35 : 0.0)) * ny * (general ? 1.12 : 1.0);
+        const double odd = nx % 2 && march_geom(nx, ny, 1).strips <= 4 ? 0.22 : 0.0;
+        limit = std::min(limit, one / ((p.wall[0] != CLB_PERIODIC ? 1.19 : 1.03) * (1.0 + odd) * (general ? 1.11 : 1.0)));
     }
     return march_rows_for([&](int rows) { return march_geom(nx, ny, rows).warps(); }, sms, limit);
 }

@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 F32, F16 = W.STORAGE_F32, W.STORAGE_F16DEV
 P, D, A, WET = W.WALL_PERIODIC, W.WALL_DIRICHLET, W.WALL_ADIABATIC, W.WALL_WET
-CASES = [(F32, (1011, 1013), (P, P, P, P)), (F32, (1011, 1013), (D, A, A, D)), (F32, (59, 17201), (P, P, D, D)), (F32, (121, 9002), (A, D, D, A)), (F32, (53, 20011), (D, D, A, A)),
+CASES = [(F32, (1011, 1013), (P, P, P, P)), (F32, (1011, 1013), (D, A, A, D)), (F32, (59, 17201), (P, P, D, D)), (F32, (113, 10090), (A, D, D, A)), (F32, (53, 20011), (D, D, A, A)),
          (F32, (20011, 53), (A, D, P, P)), (F16, (801, 603), (D, D, A, A)), (F16, (801, 603), (WET, WET, WET, WET)),
          (F16, (641, 640), (P, P, P, P)), (F16, (130001, 4), (P, P, D, D))]
 

@@ -266,7 +266,9 @@ def test_default_batch_form_is_not_the_slower_one(clb, size, walls, rates):
 # Lattices just above the size at which two steps per launch begin: the default is not the slower form.
 @pytest.mark.parametrize("rates", [1.0, 1.2])
 @pytest.mark.parametrize("size,walls,steps", [((1024, 1024), "cavity", 1), ((1024, 1024), "layer", 2), ((2048, 512), "cavity", 2),
-                                              ((60, 17003), "cavity", 2), ((1100, 1000), "cavity", 2), ((17003, 60), "cavity", 2)])
+                                              ((60, 17003), "cavity", 2), ((1100, 1000), "cavity", 2), ((17003, 60), "cavity", 2),
+                                              ((128, 9019), "cavity", 1), ((121, 9002), "layer", 1), ((121, 9002), "cavity", 1),
+                                              ((305, 3700), "cavity", 2)])
 def test_default_lattice_form_is_not_the_slower_one(clb, size, walls, steps, rates):
     prob = W.random_problem(*size, seed=1, storage=F32, walls=LAYOUTS[walls])
     prob.params.update(s_3=rates, s_4=rates, lambda2=rates)
