@@ -451,7 +451,11 @@ clb_status take_snapshot(clb_handle* h)
 // 128 x 1, 3.7 at 32 x 2; 640 x 640, FP16: 6.5 and 5.7); large FP32 rows that fill blocks of two warps
 // to the last node take them side by side, at 64 x 1 (1024 x 950: 14.0 us against 14.2, 1280 x 700 12.4 and
 // 12.6, 896 x 1000 12.5 and 12.6), all others do not, whatever the number of their warps (200 x 4000: 18.2
-// and 16.3, 600 x 700 6.9 and 6.5, 1000 x 700 9.6 and 9.4, 701 x 699 7.8 and 7.1; 30 sizes measured).
+// and 16.3, 600 x 700 6.9 and 6.5, 1000 x 700 9.6 and 9.4, 701 x 699 7.8 and 7.1; 30 sizes measured). FP32 lattices
+// whose warps are one round of resident ones, more than half full, take blocks of four warps side by side where
+// the rows end in ragged warps but fill their blocks to three quarters and more (32 x 2 against 128 x 1: 252 x
+// 807 layer 4.7 and 4.0 us, cavity 4.4 and 4.0; 232 x 905 4.4 and 3.8, 4.5 and 4.0; 500 x 400 4.3 and 3.9); in
+// lattices of fewer or more warps they gain nothing or lose (232 x 1300 cavity 5.8 and 6.5; 68 sizes measured).
 void default_shape(int storage, int nx, int ny, int sms, int* bx, int* by, int* npt)
 {
     const long long nodes = (long long)nx * ny;
@@ -471,8 +475,14 @@ void default_shape(int storage, int nx, int ny, int sms, int* bx, int* by, int* 
     *npt = small ? 1 : 2;
     if (small) *by = 4;
     if (storage == CLB_F16DEV && nodes >= kSplitNodes) *npt = 4;
-    if (storage == CLB_F32 && nodes >= kSplitNodes && nx % 128 == 0) {
+    if (storage != CLB_F32 || small) return;
+    const long long warps = (long long)((nx + 63) / 64) * ny;
+    const bool one_round = warps >= 13LL * sms && warps <= 24LL * sms;
+    if (nodes >= kSplitNodes && nx % 128 == 0) {
         *bx = 64;
+        *by = 1;
+    } else if (one_round && nx <= 1024 && nx % 64 != 0 && 4 * nx >= 3 * ((nx + 255) / 256 * 256)) {
+        *bx = 128;
         *by = 1;
     }
 }

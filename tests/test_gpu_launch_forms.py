@@ -441,3 +441,22 @@ def test_default_form_of_uneven_batches_is_not_the_slower_one(clb, sizes, rates)
     b.set_steps_per_launch(1)
     assert us <= 1.05 * step_us(b)
     b.close()
+
+
+# Mid-sized FP32 lattices: blocks of four warps side by side where the rows fill them and the lattice is one
+# round of resident warps (two rows of one warp took up to 1.2 times as long there).
+@pytest.mark.parametrize("walls", ["cavity", "layer"])
+@pytest.mark.parametrize("size,shape", [((232, 905), (128, 1, 2)), ((250, 800), (128, 1, 2)), ((500, 400), (128, 1, 2)), ((964, 192), (128, 1, 2)),
+                                        ((232, 1300), (32, 2, 2)), ((513, 385), (32, 2, 2)), ((300, 700), (32, 2, 2)), ((128, 1500), (32, 2, 2))])
+def test_default_block_of_mid_sized_lattices(clb, size, shape, walls):
+    prob = W.random_problem(*size, seed=1, storage=F32, walls=LAYOUTS[walls])
+    prob.params.update(s_3=1.0, s_4=1.0, lambda2=1.0)
+    prob.T, prob.ux, prob.uy = 0.1 * prob.T, 0.1 * prob.ux, 0.1 * prob.uy
+    lat = clb.Lattice.from_problem(prob)
+    assert lat.launch() == shape
+    us = step_us(lat, 640)
+    for other in ((32, 2, 2), (128, 1, 2)):
+        if size != (232, 1300) or walls == "cavity":
+            lat.set_launch(*other)
+            assert us <= 1.03 * step_us(lat, 640), other
+    lat.close()
