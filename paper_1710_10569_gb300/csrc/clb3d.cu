@@ -1494,9 +1494,10 @@ void drop_batch3_graphs(clb3d_batch* b)
 // the steps per graph of chains. Times in us, fitted to batches of 12 to 1,000 equal boxes of edge 8 to 48 and
 // uneven ones: a chain's launch costs 0.32 us of the whole device however small its box, 0.39 in short graphs;
 // one launch for all takes 3.1 ns per block of 128 x 2 nodes, up to 4.8 on batches of fewer blocks; in the FP16
-// form a quarter more, and in FP64 twice as long as chains at any size. Chains / one launch, FP32: 12 boxes of
-// edge 16 8.3 / 11.5 us per step, 48 of 12 19.9 / 21.8, 200 of 8 to 40 111 / 146, 1,000 of 16 387 / 398, but 12
-// of edge 8 6.5 / 5.3, 256 of 8 70 / 44, 800 of 14 314 / 254, 1,000 of 8 293 / 121.
+// form a quarter more, and in FP64 twice as long as chains at any size. A chain's step takes 8 us or more, however
+// few they are. Chains / one launch, FP32: 12 boxes of edge 16 8.3 / 11.5 us per step, 48 of 12 19.9 / 21.8, 200 of
+// 8 to 40 111 / 146, 1,000 of 16 387 / 398, but 5 of 14 8.3 / 6.4, 12 of 8 6.5 / 5.3, 256 of 8 70 / 44, 800 of 14
+// 314 / 254, 1,000 of 8 293 / 121.
 void batch3_choose(clb3d_batch* b)
 {
     double tiles = 0, nodes = 0;
@@ -1507,11 +1508,11 @@ void batch3_choose(clb3d_batch* b)
     const size_t n = b->lat.size();
     b->chunk = nodes >= 500000 ? kShortChunk : kChunk;
     while (b->chunk > kShortChunk && b->chunk * n > kGraphLaunches) b->chunk /= 2;
-    const double chains = 2.5 + (b->chunk > kShortChunk ? 0.32 : 0.39) * n;
+    const double least = b->storage == CLB_F32 ? 8.0 : 8.8;  // a step of a chain by itself
+    const double chains = std::max(least, 2.5 + (b->chunk > kShortChunk ? 0.32 : 0.39) * n);
     const double all = tiles * (3.1e-3 + 1.7e-3 * std::min(1.0, 1e4 / tiles));
-    b->chains_gain = b->storage == CLB_F64   ? 1.5e-3 * nodes
-                     : b->storage == CLB_F32 ? 4.0 + all - chains
-                                             : 10.0 + 1.25 * all - chains;
+    const double all16 = std::min(6.0 + 8.5e-3 * tiles, 10.0 + 1.25 * all);
+    b->chains_gain = b->storage == CLB_F64 ? 1.5e-3 * nodes : (b->storage == CLB_F32 ? 4.0 + all : all16) - chains;
     b->chains = b->chains_gain > 0;
     b->stepped = 0;
 }

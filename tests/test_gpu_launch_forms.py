@@ -222,21 +222,21 @@ def test_lattice_form_survives_calls_that_change_nothing(clb):
 
 
 def test_3d_batch_form_survives_the_present_tile(clb):
-    b = clb.Batch3D([W.random_problem3d(20 + k, 18, 16, seed=k, storage=F32) for k in range(4)])
+    b = clb.Batch3D([W.random_problem3d(24 + k, 22, 20, seed=k, storage=F32) for k in range(8)])
     assert b.chains()
     b.set_tile(*b.launch()["block"])
     assert b.chains()
     b.step(33)
-    ref = [b.fields(k) for k in range(4)]
+    ref = [b.fields(k) for k in range(8)]
     b.set_tile(64, 2)
     assert not b.chains()
     for chains in (True, False):
         b.set_chains(chains)
         assert b.chains() == chains
-        for k in range(4):
+        for k in range(8):
             b.init_fields(k, *b.problems[k].fields())
         b.step(33)
-        for k in range(4):
+        for k in range(8):
             for x, y in zip(b.fields(k), ref[k]):
                 assert np.array_equal(x, y), (chains, k)
     b.close()
@@ -391,7 +391,7 @@ def test_chains_equal_single_boxes(clb, storage):
 
 # Chains were taken for every batch: 1,000 boxes of edge 8 stepped in 293 us instead of 121. The default is
 # not the slower form (8% for the estimate).
-@pytest.mark.parametrize("count,edge,storage", [(12, 8, F32), (256, 8, F32), (1000, 8, F32), (48, 12, F32), (512, 12, F32), (800, 14, F32),
+@pytest.mark.parametrize("count,edge,storage", [(12, 8, F32), (6, 10, F32), (5, 14, F32), (16, 6, F16), (256, 8, F32), (1000, 8, F32), (48, 12, F32), (512, 12, F32), (800, 14, F32),
                                                 (256, 16, F32), (12, 32, F32), (256, 8, F16), (100, 12, F16), (256, 8, F64)])
 def test_default_3d_batch_form_is_not_the_slower_one(clb, count, edge, storage):
     b = clb.Batch3D([W.rayleigh_benard3d(edge, edge, edge, Ra=2e3, storage=storage)] * count)
@@ -447,7 +447,8 @@ def test_default_form_of_uneven_batches_is_not_the_slower_one(clb, sizes, rates)
 # round of resident warps (two rows of one warp took up to 1.2 times as long there).
 @pytest.mark.parametrize("walls", ["cavity", "layer"])
 @pytest.mark.parametrize("size,shape", [((232, 905), (128, 1, 2)), ((250, 800), (128, 1, 2)), ((500, 400), (128, 1, 2)), ((964, 192), (128, 1, 2)),
-                                        ((232, 1300), (32, 2, 2)), ((513, 385), (32, 2, 2)), ((300, 700), (32, 2, 2)), ((128, 1500), (32, 2, 2))])
+                                        ((408, 506), (32, 2, 2)), ((232, 1300), (32, 2, 2)), ((513, 385), (32, 2, 2)),
+                                        ((300, 700), (32, 2, 2)), ((128, 1500), (32, 2, 2))])
 def test_default_block_of_mid_sized_lattices(clb, size, shape, walls):
     prob = W.random_problem(*size, seed=1, storage=F32, walls=LAYOUTS[walls])
     prob.params.update(s_3=1.0, s_4=1.0, lambda2=1.0)
