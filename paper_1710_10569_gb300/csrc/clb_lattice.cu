@@ -452,12 +452,14 @@ clb_status take_snapshot(clb_handle* h)
 // to the last node take them side by side, at 64 x 1 (1024 x 950: 14.0 us against 14.2, 1280 x 700 12.4 and
 // 12.6, 896 x 1000 12.5 and 12.6), all others do not, whatever the number of their warps (200 x 4000: 18.2
 // and 16.3, 600 x 700 6.9 and 6.5, 1000 x 700 9.6 and 9.4, 701 x 699 7.8 and 7.1; 30 sizes measured). FP32 lattices
-// whose warps are one round of resident ones, more than half full, take blocks of four warps side by side where
-// the rows end in ragged warps but fill their blocks to three quarters and more (32 x 2 against 128 x 1: 252 x
-// 807 layer 4.7 and 4.0 us, cavity 4.4 and 4.0; 232 x 905 4.4 and 3.8, 4.5 and 4.0; 500 x 400 4.3 and 3.9); in
-// lattices of fewer or more warps they gain nothing or lose (232 x 1300 cavity 5.8 and 6.5; 68 sizes measured).
-void default_shape(int storage, int nx, int ny, int sms, int* bx, int* by, int* npt)
+// that are at most one round of resident blocks of four warps side by side (six per SM) take these where the
+// rows end in ragged warps but fill their blocks to three quarters and more (32 x 2 against 128 x 1: 252 x 807
+// layer 4.7 and 4.0 us, cavity 4.4 and 4.0; 232 x 905 4.4 and 3.8, 4.5 and 4.0; 500 x 400 4.3 and 3.9); with more
+// blocks they lose (408 x 506 3.8 and 4.5, 232 x 1300 cavity 5.8 and 6.5), and with few warps, between x walls
+// fewer than 13 per SM, they gain nothing (237 x 152 cavity up to a third more; 68 sizes measured).
+void default_shape(const clb_params& p, int nx, int ny, int sms, int* bx, int* by, int* npt)
 {
+    const int storage = p.storage;
     const long long nodes = (long long)nx * ny;
     const bool small = nodes < 32768;
     *bx = 32;
@@ -477,11 +479,12 @@ void default_shape(int storage, int nx, int ny, int sms, int* bx, int* by, int* 
     if (storage == CLB_F16DEV && nodes >= kSplitNodes) *npt = 4;
     if (storage != CLB_F32 || small) return;
     const long long warps = (long long)((nx + 63) / 64) * ny;
-    const bool one_round = warps >= 13LL * sms && warps <= 24LL * sms;
+    const bool periodic = p.wall[0] == CLB_PERIODIC;
+    const bool one_round = warps >= (periodic ? 5LL : 13LL) * sms && (long long)((nx + 255) / 256) * ny <= 6LL * sms;
     if (nodes >= kSplitNodes && nx % 128 == 0) {
         *bx = 64;
         *by = 1;
-    } else if (one_round && nx <= 1024 && nx % 64 != 0 && 4 * nx >= 3 * ((nx + 255) / 256 * 256)) {
+    } else if (one_round && nx <= (periodic && warps < 13LL * sms ? 512 : 1024) && nx % 64 != 0 && 4 * nx >= 3 * ((nx + 255) / 256 * 256)) {
         *bx = 128;
         *by = 1;
     }
@@ -559,7 +562,7 @@ extern "C" clb_status clb_create(int nx, int ny, const clb_params* p, void* stre
         h->Pf = make_lat_params<float>(nx, ny, *p);
         int sms = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
-        default_shape(p->storage, nx, ny, std::max(1, sms), &h->bx, &h->by, &h->npt);
+        default_shape(*p, nx, ny, std::max(1, sms), &h->bx, &h->by, &h->npt);
         h->march = march_rows_rule(nx, ny, *p, std::max(1, sms));
         {
             std::lock_guard<std::mutex> lk(g_tune_mu);
@@ -985,7 +988,7 @@ extern "C" clb_status clb_autotune(clb_handle* h, int* block_x, int* block_y, in
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, h->device);
         sms = std::max(1, sms);
         std::vector<Launch> cands(1, Launch{128, 1, 1, 0, 8, 0});
-        default_shape(h->p.storage, h->nx, h->ny, sms, &cands[0].bx, &cands[0].by, &cands[0].npt);
+        default_shape(h->p, h->nx, h->ny, sms, &cands[0].bx, &cands[0].by, &cands[0].npt);
         cands.push_back(current_launch(h));
         cands[1].march = 0;
         const int shapes[][2] = {{64, 1}, {128, 1}, {256, 1}, {32, 1}, {32, 2}, {32, 4}, {64, 2}, {128, 2}};
