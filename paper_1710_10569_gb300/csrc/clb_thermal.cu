@@ -554,15 +554,15 @@ MarchGeom thermal_geom(int nx, int ny, int rows)
 // resident warps is taken, counting two rounds at least: warps that all start together load and
 // compute in step, and one round runs at half the rate (2048 x 2048: one of 22 rows 17.2 us per step,
 // two of 12 to 14 rows 14.7 - 15.2; 4096 x 4096: two of 44 rows 45.9, three of 28 46.8).
-// One step per launch is kept where the two estimates say so (both fitted to 266 shapes of 0.4 to 4 million
+// One step per launch is kept where the two estimates say so (both fitted to 330 shapes of 0.4 to 4 million
 // nodes, to 5 and 10%, in us per step): one step takes 0.37 ns per warp of 64 nodes and 0.44 per block of
 // 256, less the more nodes share the launch, and the FP32 bytes at the copy bandwidth where those leave L2; a
 // turn of the pipeline takes a + b w at w warps per SM, more between x walls, whose windows take the wall rules
-// every turn and end last, more for lambda2 other than 1 and in the FP16 form, and a third more on odd rows,
-// whose velocities load one by one. One step per launch / four: FP32 cavities 640 x 640 3.6 / 4.1, 1024 x 1024 6.2 /
+// every turn and end last, more on rows of three or four windows between them, more for lambda2 other than 1 and in the
+// FP16 form, and 1.2 to 1.5 times as long on odd rows, whose velocities load one by one. One step per launch / four: FP32 cavities 640 x 640 3.6 / 4.1, 1024 x 1024 6.2 /
 // 6.5, 802 x 829 5.5 / 4.9, 1500 x 1000 8.4 / 7.2; FP16 with lambda2 = 1.3 cavities 1800 x 1200 11.0 / 11.9,
 // 162 x 5968 9.0 / 7.9, 2048 x 2048 24.6 / 18.6; layers 2971 x 220 4.6 / 5.4, 727 x 1495 6.8 / 7.5, 1024 x 1024
-// 6.2 / 5.6. The choice costs 0.3% on average against the better one (four always: 2.5%).
+// 6.2 / 5.6. The choice costs 0.2% on average against the better one (four always: 2.5%).
 constexpr long long kMarchNodesT = 400000;
 struct TurnCost {
     double a, b;
@@ -570,17 +570,22 @@ struct TurnCost {
 // [FP32, FP16][no x walls, x walls][lambda2 = 1, other]
 constexpr TurnCost kTurn[2][2][2] = {{{{0.55, 0.046}, {0.60, 0.053}}, {{0.75, 0.064}, {0.80, 0.072}}},
                                      {{{0.55, 0.053}, {0.55, 0.062}}, {{0.75, 0.065}, {0.80, 0.077}}}};
-constexpr double kOddRowsTurn = 1.4, kOddRowsTurnWalls = 1.1;
+constexpr double kOddRowsOne = 1.03, kOddRowsTurn[2] = {1.4, 1.5}, kOddRowsTurnWalls = 1.2, kFewWindowsWalls = 1.2;
 bool several_steps_pay(int nx, int ny, const clb_params& p, int rows, int sms)
 {
     const double n = double(nx) * ny;
     double one = 1.96 + 0.367e-3 * ((nx + 63) / 64) * ny + 0.438e-3 * ((nx + 255) / 256) * ny - 3.38e-6 * std::min(n, 2.5e6);
+    const bool odd = nx % 2 != 0;
+    if (odd) one *= kOddRowsOne;
     if (p.storage == CLB_F32 && n >= 1.8e6) one = std::max(one, n * 48.0 / 7.0e6);
     const bool x_walls = p.wall[0] != CLB_PERIODIC;
     const TurnCost c = kTurn[p.storage == CLB_F16DEV][x_walls][p.lambda2 != 1.0];
     const double turns = double(rows + 2 * (kSteps - 1)) / kSteps;
-    const double four = turns * (c.a + c.b * thermal_geom(nx, ny, rows).warps() / sms);
-    return four * (nx % 2 == 0 ? 1.0 : x_walls ? kOddRowsTurnWalls : kOddRowsTurn) < one;
+    const MarchGeom G = thermal_geom(nx, ny, rows);
+    double four = turns * (c.a + c.b * G.warps() / sms);
+    if (odd) four *= x_walls ? kOddRowsTurnWalls : kOddRowsTurn[p.lambda2 != 1.0];
+    if (x_walls && G.strips > 2 && G.strips <= 4) four *= kFewWindowsWalls;
+    return four < one;
 }
 int thermal_rows_rule(int nx, int ny, const clb_params& p, int sms)
 {
