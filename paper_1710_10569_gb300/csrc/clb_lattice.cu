@@ -456,7 +456,8 @@ clb_status take_snapshot(clb_handle* h)
 // rows end in ragged warps but fill their blocks to three quarters and more (32 x 2 against 128 x 1: 252 x 807
 // layer 4.7 and 4.0 us, cavity 4.4 and 4.0; 232 x 905 4.4 and 3.8, 4.5 and 4.0; 500 x 400 4.3 and 3.9); with more
 // blocks they lose (408 x 506 3.8 and 4.5, 232 x 1300 cavity 5.8 and 6.5), and with few warps, between x walls
-// fewer than 13 per SM, they gain nothing (237 x 152 cavity up to a third more; 68 sizes measured).
+// fewer than 13 per SM, they gain nothing (237 x 152 cavity up to a third more; 68 sizes measured); wet walls,
+// whose rows end last, keep 32 x 2 (912 x 144 4.5 and 4.7).
 void default_shape(const clb_params& p, int nx, int ny, int sms, int* bx, int* by, int* npt)
 {
     const int storage = p.storage;
@@ -478,13 +479,14 @@ void default_shape(const clb_params& p, int nx, int ny, int sms, int* bx, int* b
     if (small) *by = 4;
     if (storage == CLB_F16DEV && nodes >= kSplitNodes) *npt = 4;
     if (storage != CLB_F32 || small) return;
+    const bool wet = p.wall[0] == CLB_WALL_WET || p.wall[2] == CLB_WALL_WET;
     const long long warps = (long long)((nx + 63) / 64) * ny;
     const bool periodic = p.wall[0] == CLB_PERIODIC;
     const bool one_round = warps >= (periodic ? 5LL : 13LL) * sms && (long long)((nx + 255) / 256) * ny <= 6LL * sms;
     if (nodes >= kSplitNodes && nx % 128 == 0) {
         *bx = 64;
         *by = 1;
-    } else if (one_round && nx <= (periodic && warps < 13LL * sms ? 512 : 1024) && nx % 64 != 0 && 4 * nx >= 3 * ((nx + 255) / 256 * 256)) {
+    } else if (one_round && !wet && nx <= (periodic && warps < 13LL * sms ? 512 : 1024) && nx % 64 != 0 && 4 * nx >= 3 * ((nx + 255) / 256 * 256)) {
         *bx = 128;
         *by = 1;
     }
