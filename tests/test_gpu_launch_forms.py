@@ -107,7 +107,7 @@ def test_four_thermal_steps_on_odd_rows(clb, walls, lambda2, storage):
 
 
 # Four steps per launch between x walls took up to 1.18 times as long as one on lattices of 0.4 to 2 million
-# nodes (3% for the timing and the sizes next to the line).
+# nodes (5% for the timing and the sizes next to the line).
 @pytest.mark.parametrize("storage", [F32, F16])
 @pytest.mark.parametrize("lambda2", [1.0, 1.3])
 @pytest.mark.parametrize("shape", [(640, 640), (1024, 1024), (1500, 1000), (100, 6000), (2048, 2048)], ids=lambda s: "%dx%d" % s)
@@ -115,7 +115,7 @@ def test_default_thermal_form_is_not_the_slower_one(clb, shape, lambda2, storage
     h = thermal(clb, *shape, storage, "cavity", lambda2)
     us = step_us(h)
     h.set_steps_per_launch(1)
-    assert us <= 1.03 * step_us(h)
+    assert us <= 1.05 * step_us(h)
     h.close()
 
 
@@ -277,7 +277,7 @@ def test_default_lattice_form_is_not_the_slower_one(clb, size, walls, steps, rat
     assert lat.steps_per_launch() == steps
     us = step_us(lat)
     lat.set_steps_per_launch(1)
-    assert us <= 1.01 * step_us(lat)
+    assert us <= 1.05 * step_us(lat)
     lat.close()
 
 
@@ -293,7 +293,7 @@ def test_default_block_is_not_the_slower_one(clb, size):
     us = step_us(lat)
     for shape in ((64, 1, 2), (32, 2, 2)):
         lat.set_launch(*shape)
-        assert us <= 1.02 * step_us(lat), shape
+        assert us <= 1.04 * step_us(lat), shape
     lat.close()
 
 
@@ -309,7 +309,7 @@ def test_tuned_shape_is_not_the_slower_one(clb, size, storage):
     us = step_us(lat)
     shape = lat.autotune()
     assert lat.launch() == shape and lat.steps_per_launch() == steps
-    assert step_us(lat) <= 1.03 * us
+    assert step_us(lat) <= 1.04 * us
     lat.close()
 
 
@@ -459,5 +459,5 @@ def test_default_block_of_mid_sized_lattices(clb, size, shape, walls):
     for other in ((32, 2, 2), (128, 1, 2)):
         if size != (232, 1300) or walls == "cavity":
             lat.set_launch(*other)
-            assert us <= 1.03 * step_us(lat, 640), other
+            assert us <= 1.04 * step_us(lat, 640), other
     lat.close()
