@@ -193,7 +193,7 @@ clb_status clb_load(clb_handle *h, const void *buf, size_t bytes);
 
 /* Launch shape of the step kernel: threads per block along x (32..256, multiple of 32), rows per
  * block (1..8, block_x * block_y <= 256) and nodes per thread along x (1, 2 or 4). 0 keeps the
- * current value. Defaults: by storage and size, 1 (FP64, and small lattices) to 4 nodes per thread (large
+ * current value. Defaults: by storage, size and walls, 1 (FP64, and small lattices) to 4 nodes per thread (large
  * FP16 ones).
  * clb_autotune times candidate shapes on the live lattice (the populations are restored
  * afterwards; it allocates one buffer-sized scratch with cudaMallocAsync) and keeps the default unless
